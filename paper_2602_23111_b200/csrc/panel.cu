@@ -93,6 +93,14 @@ __global__ void gaussian_kernel(uint64_t seed, uint64_t dc, long long d, long lo
 // per rotation) and writes them back; the CTAs then meet at a grid barrier.  One outer sweep =
 // (number of blocks - 1) barriers instead of the (n - 1) of element-wise Jacobi.
 constexpr int JAC_MAX_SWEEPS = 30;
+// A sweep that met no squared cosine above JAC_DONE_COS2 is the last one: what the result may lack of
+// orthogonality has been measured, at the level that fp32 keeps.  (Convergence is quadratic only between well
+// separated eigenvalues.  Columns of nearly equal norm turn by large angles however small their cosines are,
+// and a sweep shrinks those by a small factor only: a rule that stopped after cosines of 3e-4 and trusted the
+// square left |U^T U - I| at 2e-3 for 64 columns on a spectrum of 0.1 % spread, where this one leaves 1e-6.
+// The sweep that confirms is one of seven or eight on a power law.)
+// Sweeps that run out are an error only where a cosine of 1e-4 is left (JAC_FAIL_COS2).
+constexpr float JAC_DONE_COS2 = 1e-13f, JAC_FAIL_COS2 = 1e-8f;
 struct JacobiInfo {
   GridBarrierState bar;             // zeroed before the launch
   int sweeps;
@@ -216,6 +224,7 @@ __global__ void jacobi_kernel(double* At, int n, int b, int max_sweeps, double t
   const unsigned nctas = gridDim.x;
   unsigned bar = 0;
   bool alive = true, converged = false;
+  float mc2 = 1.f;
   int sweep = 0;
   for (; alive && sweep < max_sweeps && !converged; ++sweep) {
     for (int step = 0; alive && step < nbr - 1; ++step) {
@@ -274,20 +283,17 @@ __global__ void jacobi_kernel(double* At, int n, int b, int max_sweeps, double t
       }
       alive = grid_barrier(&info->bar, ++bar * nctas, poll_limit);
     }
-    // Every CTA reads the same values after the barrier of the sweep's last step.  Convergence is
-    // quadratic: once the largest cosine rotated away in a sweep is below 1e-4, what is left is
-    // of the order of its square, far below the threshold, and the sweep that would only confirm
-    // it is skipped.
+    // Every CTA reads the same values after the barrier of the sweep's last step.
     if (alive) {
       const int rot = *reinterpret_cast<volatile int*>(&info->rotations[sweep]);
-      const float mc2 = __int_as_float(*reinterpret_cast<volatile int*>(&info->max_cos2[sweep]));
-      converged = (rot == 0) || (mc2 < 1e-8f);
+      mc2 = __int_as_float(*reinterpret_cast<volatile int*>(&info->max_cos2[sweep]));
+      converged = (rot == 0) || (mc2 < JAC_DONE_COS2);
     }
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     info->sweeps = sweep;
     if (!alive && dev_status) atomicOr(dev_status, DEV_WAIT_EXPIRED);
-    else if (!converged && dev_status) atomicOr(dev_status, DEV_JACOBI_NOCONV);
+    else if (!converged && mc2 >= JAC_FAIL_COS2 && dev_status) atomicOr(dev_status, DEV_JACOBI_NOCONV);
   }
 }
 
@@ -334,6 +340,7 @@ __global__ void __launch_bounds__(256) jacobi_gram_kernel(double* At, int n, int
   const unsigned nctas = gridDim.x;
   unsigned bar = 0;
   bool alive = true, converged = false;
+  float mc2 = 1.f;
   int sweep = 0;
   for (; alive && sweep < max_sweeps && !converged; ++sweep) {
     for (int step = 0; alive && step < nbr - 1; ++step) {
@@ -477,14 +484,14 @@ __global__ void __launch_bounds__(256) jacobi_gram_kernel(double* At, int n, int
     }
     if (alive) {
       const int rot = *reinterpret_cast<volatile int*>(&info->rotations[sweep]);
-      const float mc2 = __int_as_float(*reinterpret_cast<volatile int*>(&info->max_cos2[sweep]));
-      converged = (rot == 0) || (mc2 < 1e-8f);
+      mc2 = __int_as_float(*reinterpret_cast<volatile int*>(&info->max_cos2[sweep]));
+      converged = (rot == 0) || (mc2 < JAC_DONE_COS2);
     }
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     info->sweeps = sweep;
     if (!alive && dev_status) atomicOr(dev_status, DEV_WAIT_EXPIRED);
-    else if (!converged && dev_status) atomicOr(dev_status, DEV_JACOBI_NOCONV);
+    else if (!converged && mc2 >= JAC_FAIL_COS2 && dev_status) atomicOr(dev_status, DEV_JACOBI_NOCONV);
   }
 }
 
@@ -560,6 +567,7 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
   const double inv_scale = info->inv_scale;
   unsigned bar = 0;
   bool alive = true, converged = false;
+  float mc2 = 1.f;
   int sweep = 0;
   for (; alive && sweep < max_sweeps && !converged; ++sweep) {
     for (int step = 0; alive && step < nb - 1; ++step) {
@@ -704,13 +712,13 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
           // meanwhile: the largest cosine between columns that this visit is about to rotate (four more warps;
           // G[0] is intact until the second round has begun to write it, so its copy is taken from `part`)
           const int e = threadIdx.x - 128;           // the 64 entries of the crossing tile, the pairs within the blocks
-          float mc2 = 0.f;
+          float c2 = 0.f;
           const int i = (e >> 3) & 7, j = e & 7;
           double ii = 0.0, jj = 0.0, ij = 0.0;
           if (e < 64) {
 #pragma unroll
             for (int w8 = 0; w8 < 8; ++w8) { ii += part[w8][0][i * 9]; jj += part[w8][2][j * 9]; ij += part[w8][1][i * 8 + j]; }
-            mc2 = static_cast<float>(ij * ij / (ii * jj));
+            c2 = static_cast<float>(ij * ij / (ii * jj));
           } else if (full && i < j) {
             double jj2 = 0.0, kk2 = 0.0, jk2 = 0.0;
 #pragma unroll
@@ -718,10 +726,10 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
               ii += part[w8][0][i * 9]; jj += part[w8][0][j * 9]; ij += part[w8][0][i * 8 + j];
               jj2 += part[w8][2][i * 9]; kk2 += part[w8][2][j * 9]; jk2 += part[w8][2][i * 8 + j];
             }
-            mc2 = static_cast<float>(fmax(ij * ij / (ii * jj), jk2 * jk2 / (jj2 * kk2)));
+            c2 = static_cast<float>(fmax(ij * ij / (ii * jj), jk2 * jk2 / (jj2 * kk2)));
           }
-          mc2 = mc2 > 0.f ? fminf(mc2, 1.f) : 0.f;      // (NaN counts as nothing to rotate)
-          const int bits = __reduce_max_sync(0xffffffffu, __float_as_int(mc2));   // non-negative floats order as ints
+          c2 = c2 > 0.f ? fminf(c2, 1.f) : 0.f;      // (NaN counts as nothing to rotate)
+          const int bits = __reduce_max_sync(0xffffffffu, __float_as_int(c2));   // non-negative floats order as ints
           if (lane == 0) atomicMax(&info->max_cos2[sweep], bits);
         }
       }
@@ -734,17 +742,14 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
       }
     }
     if (alive) {
-      // Convergence is quadratic (measured: 2.6e-3 -> 1.2e-4 -> 9e-9, 8e-3 -> 1.4e-4 -> 4e-8): after a sweep
-      // that met no cosine above 3e-4 what is left is a few 1e-7 at most, the level at which the result
-      // is stored, and the sweep that would only confirm it is skipped.
-      const float mc2 = __int_as_float(*reinterpret_cast<volatile int*>(&info->max_cos2[sweep]));
-      converged = mc2 < 1e-7f;
+      mc2 = __int_as_float(*reinterpret_cast<volatile int*>(&info->max_cos2[sweep]));
+      converged = mc2 < JAC_DONE_COS2;
     }
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     info->sweeps = sweep;
     if (!alive && dev_status) atomicOr(dev_status, DEV_WAIT_EXPIRED);
-    else if (!converged && dev_status) atomicOr(dev_status, DEV_JACOBI_NOCONV);
+    else if (!converged && mc2 >= JAC_FAIL_COS2 && dev_status) atomicOr(dev_status, DEV_JACOBI_NOCONV);
   }
 }
 
