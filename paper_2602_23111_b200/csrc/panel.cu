@@ -499,13 +499,15 @@ __global__ void __launch_bounds__(256) jacobi_gram_kernel(double* At, int n, int
 // What bounded jacobi_gram_kernel at n = 128 (6.5 us per visit, 120 visits): the eight rounds' dependent
 // fp64 chains with two block barriers each (3.2 us), then the columns' trip into shared memory, through
 // the accumulated rotation and out again.  Here 64 threads walk the rounds on the visit's 16 x 16 Gram
-// matrix alone, in fp32 (it is formed in double, afresh for every visit, and only steers the angles;
-// each rotation is made orthogonal to double accuracy before it touches a column): thread (u, v)
+// matrix alone (in double; the angles are fp32, each rotation is made orthogonal to double accuracy
+// before it touches a column): thread (u, v)
 // holds the 2 x 2 block where pairs u and v meet and works out both pairs' angles itself, so a round
 // is one barrier of two warps.  ROWS other threads hold one row each of the sixteen columns in registers
 // and apply the rounds in double as their angles are published: the update costs nothing beyond the
-// rounds, and no column passes through shared memory.  n = 128: 781 -> 370 us (8 -> 7 sweeps); of a visit's 7000
-// cycles the rounds take 360 each, forming G 900, the columns' way to the next CTA (store, barrier, load) 2600.
+// rounds, and no column passes through shared memory.  n = 128: 112 -> 61 us a sweep; of a visit's 7800
+// cycles the rounds take 500 each, forming G 900, the columns' way to the next CTA (store, barrier, load) 2600.
+// (With G in fp32 and the rotations of G not on the unit circle a round takes 360 cycles, but the diagonal of
+// G then drifts by more than the columns of a cluster differ by: 18 to 30 sweeps there instead of 7 to 14.)
 //
 // Pairs of a round as slots: the first visit of a sweep plays the full round robin on 16 items (item 15
 // fixed, the others y[0..14] moving up by one per round: (15, y[0]), (y[i], y[15 - i])); every other
@@ -542,8 +544,8 @@ __device__ __forceinline__ void stream_pair(bool full, int is, int u, int& a, in
 // a' = c a + o b, b' = c b - o a make the columns orthogonal: with d = |b|^2 - |a|^2 and g = 2 a.b the
 // tangent of the smaller such angle is sign(d) g / (|d| + |(d, g)|).  (The hardware's approximations:
 // the angle only has to shrink the inner product.)
-__device__ __forceinline__ float2 stream_angle(float aa, float bb, float ab) {
-  const float d = bb - aa, g = 2.f * ab;
+__device__ __forceinline__ float2 stream_angle(double aa, double bb, double ab) {
+  const float d = static_cast<float>(bb - aa), g = 2.f * static_cast<float>(ab);
   const float q = fmaf(d, d, fmaf(g, g, 1e-36f));
   const float t = copysignf(1.f, d) * g * rcp_approx(fmaf(q, rsqrt_fast(q), fabsf(d)));
   const float c = rsqrt_fast(fmaf(t, t, 1.f));
@@ -555,7 +557,7 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
     double* At, int n, int max_sweeps, JacobiInfo* info, int* dev_status, unsigned poll_limit) {
   grid_dep_wait();
   __shared__ double part[8][3][64];
-  __shared__ float G[2][JG_M][JG_P];
+  __shared__ double G[2][JG_M][JG_P];
   __shared__ float2 coef[JG_M][JG_B];            // every round of the visit, per pair: c, o
   __shared__ double2 unit[ROWS / 32][2][JG_B];   // two rounds of them on the unit circle, per row warp
   const int b = JG_B;
@@ -676,35 +678,39 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
           double sum = 0.0;
 #pragma unroll
           for (int w8 = 0; w8 < 8; ++w8) sum += part[w8][tile][r * 8 + c];
-          G[0][ei][ej] = static_cast<float>(sum * inv_scale * inv_scale);
+          G[0][ei][ej] = sum * inv_scale * inv_scale;
         }
         named_sync(1, JS_G_THREADS);
         if (threadIdx.x < JS_R_THREADS) {
           const int u = threadIdx.x >> 3, v = threadIdx.x & 7;
-          float* Gc = &G[0][0][0];
-          float* Gn = &G[1][0][0];
+          double* Gc = &G[0][0][0];
+          double* Gn = &G[1][0][0];
           int au, bu, av, bv;
           stream_pair(full, 0, u, au, bu);
           stream_pair(full, 0, v, av, bv);
 #pragma unroll 1
           for (int is = 0; is < rounds; ++is) {
             const int ra = au * JG_P, rb = bu * JG_P, sa = av * JG_P, sb = bv * JG_P;
-            const float uaa = Gc[ra + au], ubb = Gc[rb + bu], uab = Gc[ra + bu];
-            const float vaa = Gc[sa + av], vbb = Gc[sb + bv], vab = Gc[sa + bv];
-            const float x = Gc[ra + av], y = Gc[ra + bv], z = Gc[rb + av], w = Gc[rb + bv];
+            const double uaa = Gc[ra + au], ubb = Gc[rb + bu], uab = Gc[ra + bu];
+            const double vaa = Gc[sa + av], vbb = Gc[sb + bv], vab = Gc[sa + bv];
+            const double x = Gc[ra + av], y = Gc[ra + bv], z = Gc[rb + av], w = Gc[rb + bv];
             const float2 cu = stream_angle(uaa, ubb, uab), cv = stream_angle(vaa, vbb, vab);
+            const double uc = cu.x, uo = cu.y, vc = cv.x, vo = cv.y;
+            // (both pairs' Newton step towards the unit circle, beside the products: without it the diagonal
+            // drifts by 2^-22 per round, more than the columns of a cluster differ by)
+            const double fix = fma(-0.5, fma(uc, uc, uo * uo), 1.5) * fma(-0.5, fma(vc, vc, vo * vo), 1.5);
             // the block of R_u^T G R_v
-            const float x1 = fmaf(cv.x, x, cv.y * y), y1 = fmaf(cv.x, y, -cv.y * x);
-            const float z1 = fmaf(cv.x, z, cv.y * w), w1 = fmaf(cv.x, w, -cv.y * z);
-            Gn[ra + av] = fmaf(cu.x, x1, cu.y * z1);
-            Gn[rb + av] = fmaf(cu.x, z1, -cu.y * x1);
-            Gn[ra + bv] = fmaf(cu.x, y1, cu.y * w1);
-            Gn[rb + bv] = fmaf(cu.x, w1, -cu.y * y1);
+            const double x1 = fma(vc, x, vo * y), y1 = fma(vc, y, -vo * x);
+            const double z1 = fma(vc, z, vo * w), w1 = fma(vc, w, -vo * z);
+            Gn[ra + av] = fix * fma(uc, x1, uo * z1);
+            Gn[rb + av] = fix * fma(uc, z1, -uo * x1);
+            Gn[ra + bv] = fix * fma(uc, y1, uo * w1);
+            Gn[rb + bv] = fix * fma(uc, w1, -uo * y1);
             if (u == v) coef[is][u] = cu;
             // (the next round's items are worked out before the barrier)
             stream_pair(full, is + 1, u, au, bu);
             stream_pair(full, is + 1, v, av, bv);
-            float* t = Gc; Gc = Gn; Gn = t;
+            double* t = Gc; Gc = Gn; Gn = t;
             named_sync(1, JS_R_THREADS);
             if ((is & 1) == 1 || is == rounds - 1) named_arrive(2 + (is >> 1), JS_R_THREADS + ROWS);
           }
