@@ -163,9 +163,10 @@ __global__ void __launch_bounds__(256) jacobi_prepare_kernel(const double* __res
 
 // One rotation of the shared-memory columns cp, cq (length n) by one warp.  With R > 0 each lane
 // keeps its R elements of both columns in registers between the dot products and the update, so
-// a rotation reads and writes shared memory once; R = 0 re-reads (any n).  Returns 1 if rotated.
+// a rotation reads and writes shared memory once; R = 0 re-reads (any n).  scale brings squared column
+// norms into the range of fp32.  Returns 1 if rotated.
 template <int R>
-__device__ __forceinline__ int rotate_pair(double* cp, double* cq, int n, int lane, double tol, float& max_cos2) {
+__device__ __forceinline__ int rotate_pair(double* cp, double* cq, int n, int lane, double tol, double scale, float& max_cos2) {
   double alpha = 0.0, beta = 0.0, gamma = 0.0;
   double xr[R > 0 ? R : 1], yr[R > 0 ? R : 1];
   if (R > 0) {
@@ -188,7 +189,7 @@ __device__ __forceinline__ int rotate_pair(double* cp, double* cq, int n, int la
   // The angle only has to shrink the inner product, so tan is taken in fp32 (double-precision
   // divisions and square roots are slow here); cos and sin are then formed in double from that
   // tangent, which keeps the rotation orthogonal to double accuracy.
-  const float zeta = static_cast<float>(beta - alpha) / (2.f * static_cast<float>(gamma));
+  const float zeta = static_cast<float>((beta - alpha) * scale) / (2.f * static_cast<float>(gamma * scale));
   const float az = fabsf(zeta);
   const float t32 = (az > 1e15f) ? 0.5f / zeta : copysignf(1.f, zeta) / (az + sqrtf(1.f + az * az));
   const double t = static_cast<double>(t32);
@@ -222,6 +223,7 @@ __global__ void jacobi_kernel(double* At, int n, int b, int max_sweeps, double t
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m = 2 * b;
   const unsigned nctas = gridDim.x;
+  const double inv_scale = info->inv_scale;
   unsigned bar = 0;
   bool alive = true, converged = false;
   float mc2 = 1.f;
@@ -261,13 +263,13 @@ __global__ void jacobi_kernel(double* At, int n, int b, int max_sweeps, double t
           for (int is = 0; is < m - 1; ++is) {
             int p, q;
             rr_pair(m, is, warp, p, q);
-            rotated += rotate_pair<R>(cols + p * n, cols + q * n, n, lane, tol, max_cos2);
+            rotated += rotate_pair<R>(cols + p * n, cols + q * n, n, lane, tol, inv_scale * inv_scale, max_cos2);
             __syncthreads();
           }
         } else {
           for (int is = 0; is < b; ++is) {
             const int p = warp, q = b + (warp + is) % b;
-            rotated += rotate_pair<R>(cols + p * n, cols + q * n, n, lane, tol, max_cos2);
+            rotated += rotate_pair<R>(cols + p * n, cols + q * n, n, lane, tol, inv_scale * inv_scale, max_cos2);
             __syncthreads();
           }
         }
@@ -338,6 +340,7 @@ __global__ void __launch_bounds__(256) jacobi_gram_kernel(double* At, int n, int
   const int g = lane >> 2, q4 = lane & 3;
   const int ei = threadIdx.x >> 4, ej = threadIdx.x & 15;   // this thread's element of the 16 x 16 matrices
   const unsigned nctas = gridDim.x;
+  const double inv_scale = info->inv_scale;                 // (G is scaled with it: its entries are taken to fp32)
   unsigned bar = 0;
   bool alive = true, converged = false;
   float mc2 = 1.f;
@@ -388,7 +391,7 @@ __global__ void __launch_bounds__(256) jacobi_gram_kernel(double* At, int n, int
           double sum = 0.0;
 #pragma unroll
           for (int w8 = 0; w8 < 8; ++w8) sum += part[w8 * 192 + tile * 64 + r * 8 + c];
-          G0[ei][ej] = sum;
+          G0[ei][ej] = sum * inv_scale * inv_scale;
           J0[ei][ej] = (ei == ej) ? 1.0 : 0.0;
         }
         __syncthreads();
