@@ -41,7 +41,9 @@
  *    tensor-core speed: the rows are fetched in groups that share one offset from the 16-byte
  *    grid.  That path reads a few elements of the neighbouring rows as padding, so the
  *    matrix must hold finite numbers throughout, and its results equal those of the aligned
- *    layout up to the order of the fp32 sums.  Any other layout is served by slower kernels
+ *    layout up to the order of the fp32 sums.  (prac_compress with k + r <= 128 keeps an Inf or
+ *    NaN in its own row of Z all the same, and prac_compress lets nothing that lies between the
+ *    rows of a view, ldx > d, into Z.)  Any other layout is served by slower kernels
  *    with identical semantics.
  *  - The CUDA context/device current at prac_basis_create() must be current in later calls.
  */

@@ -171,6 +171,7 @@ struct TcParams {
   int cls_shift[8];
   int cls_sub;        // token-major launches by classes: piece (split) = class * cls_sub + part of its tokens; else 0
   int piece_rows;     // PIECES > 1: the bf16 pieces of B lie this many rows (of K) apart, zeros between them
+  const float* b32;   // K-major by classes, optional: B as K x N fp32, for the rows of C that are not finite
 };
 
 // K-major A whose row pitch is not a multiple of 16 bytes, fetched by TMA all the same.  With
@@ -620,7 +621,7 @@ __device__ __forceinline__ void gemm_tc_body(const CUtensorMap& tmap_a, const CU
     const int half = (warp - 2) >> 2;      // 0 or 1
     const int ewarp = warp - 2;            // 0 .. EPI_WARPS - 1: owner of a staging area
     int acc_iter = 0;
-    bool ok = true;
+    bool ok = true, not_finite = false;
     constexpr bool EPI_RMS = (EPI == EPI_RMS1 || EPI == EPI_RMS2);
     constexpr bool EPI_ACT = C::ACT;
     // Activation and RMSNorm epilogues: the element-wise factor of every 32-row x 64-column block
@@ -833,6 +834,12 @@ __device__ __forceinline__ void gemm_tc_body(const CUtensorMap& tmap_a, const CU
             ptx::tmem_ld_32x32(taddr + c * 32, v);
             ptx::tmem_ld_wait();
           }
+          if (CLS_K && p.b32 != nullptr) {
+            uint32_t m = 0u;
+#pragma unroll
+            for (int j = 0; j < 32; ++j) m = __vmaxu2(m, v[j] & 0x7fff7fffu);
+            not_finite = not_finite || (m & 0xffffu) >= 0x7f80u || (m >> 16) >= 0x7f80u;
+          }
           // A tile store writes whole 16-byte pieces: where the row ends inside one, the piece's other
           // bytes (row padding, the neighbouring columns of a wider buffer, or, by classes, the start of
           // the next row) would be overwritten.  The block holding such a row end, and by classes also
@@ -949,6 +956,35 @@ __device__ __forceinline__ void gemm_tc_body(const CUtensorMap& tmap_a, const CU
       }
     }
     if (EPI != EPI_PARTIAL && lane == 0) ptx::bulk_wait_group<0>();   // tile stores have landed
+    // What lies next to a row of A (up to seven elements in front of it) was multiplied by zeros, and B may have
+    // come in pieces: an Inf or NaN there, or in the row itself, leaves a row of C that is not finite, and nothing
+    // else does.  Such rows are formed again from their own elements and the fp32 B, a lane per column, after
+    // the warp's last tile, so that no accumulator is held meanwhile.  (Finding them costs the epilogue two
+    // instructions per pair; a second launch that read C took 3 to 8 us, a third of a small product.)
+    if (CLS_K && p.b32 != nullptr && __any_sync(0xffffffffu, not_finite)) {
+      __nv_bfloat16* const out = static_cast<__nv_bfloat16*>(p.C);
+      WorkIter again(p, worker, num_workers);
+      while (ok && again.next(p)) {
+        int mt, nt;
+        tile_coords<C::TILE_M, BN>(p, again.tile, mt, nt);
+        const int cls_j = mt % p.cls_count, m_rows = (p.M - cls_j + p.cls_count - 1) / p.cls_count;
+        const int row0 = (mt / p.cls_count) * C::TILE_M + static_cast<int>(cta_rank) * BM + quarter * 32;
+        for (int rr = 0; rr < 32 && row0 + rr < m_rows; ++rr) {
+          const long long row = static_cast<long long>(row0 + rr) * p.cls_count + cls_j;
+          for (int c = 2 * half; c < BN / 32; c = (c & 1) ? c + 3 : c + 1) {      // the warp's 64-column blocks, in halves
+            const int col = nt * BN + c * 32 + lane;
+            const bool mine = col < p.N;
+            const bool bad = mine && (reinterpret_cast<const unsigned short*>(out)[row * p.ldc + col] & 0x7f80u) == 0x7f80u;
+            if (!__any_sync(0xffffffffu, bad) || !mine) continue;
+            float sum = 0.f;
+#pragma unroll 4
+            for (int l = 0; l < p.K; ++l)
+              sum = fmaf(__bfloat162float(p.a_ptr[row * p.a_ld + l]), p.b32[static_cast<long long>(l) * p.N + col], sum);
+            out[row * p.ldc + col] = __float2bfloat16_rn(sum);
+          }
+        }
+      }
+    }
   }
 
   // ---------------------------------------------------------------- common exit
@@ -1576,7 +1612,7 @@ bool tc_rowclass_narrow_fits(const void* A, int64_t lda, int64_t M, int64_t N) {
 }
 int tc_gemm_kmajor_rowclass(const __nv_bfloat16* A, int64_t lda, const __nv_bfloat16* Bmn, int64_t ldb,
                             int64_t M, int64_t N, int64_t K, __nv_bfloat16* Cout, int64_t ldc,
-                            int* dev_status, cudaStream_t stream, int64_t piece_rows) {
+                            int* dev_status, cudaStream_t stream, int64_t piece_rows, const float* B32) {
   if (tc_init() != PRAC_OK) return PRAC_ECUDA;
   if (M <= 0 || N <= 0 || K <= 0 || lda < K) return PRAC_EINVAL;
   const bool narrow = piece_rows > 0;          // B as three pieces, one 128-wide tile per 256 rows
@@ -1621,6 +1657,7 @@ int tc_gemm_kmajor_rowclass(const __nv_bfloat16* A, int64_t lda, const __nv_bflo
   CUtensorMap tb;                              // rows = K, inner = N, boxes of 64 x 64
   if (make_map(&tb, Bmn, N, narrow ? 2 * piece_rows + K : K, ldb, 64) != PRAC_OK) return PRAC_ECUDA;
   p.piece_rows = static_cast<int>(piece_rows);
+  p.b32 = B32; p.a_ptr = A; p.a_ld = lda;
   p.M = static_cast<int>(M); p.N = static_cast<int>(N); p.K = static_cast<int>(K);
   p.cls_count = P;
   const int64_t rows0 = (M + P - 1) / P;       // the largest class

@@ -146,10 +146,12 @@ bool tc_kmajor_takes_unaligned_a(int64_t M, int64_t N);
 bool tc_rowclass_fits(const void* A, int64_t lda, int64_t M, int64_t N);
 // piece_rows > 0 (outputs of at most 128 columns, tc_rowclass_narrow_fits): B is an fp32 matrix as three
 // bf16 pieces, K rows each, piece_rows (>= K + 8) apart with zeros in between.
+// B32 != null (K x N fp32, contiguous): rows of C that are not finite are formed again from A's own elements
+// and B32, so that nothing next to a row of A gets into C.
 bool tc_rowclass_narrow_fits(const void* A, int64_t lda, int64_t M, int64_t N);
 int tc_gemm_kmajor_rowclass(const __nv_bfloat16* A, int64_t lda, const __nv_bfloat16* Bmn, int64_t ldb, int64_t M,
                             int64_t N, int64_t K, __nv_bfloat16* C, int64_t ldc, int* dev_status, cudaStream_t stream,
-                            int64_t piece_rows = 0);
+                            int64_t piece_rows = 0, const float* B32 = nullptr);
 // Whether tc_gemm_tokens takes an A with rows off the 16-byte grid by classes of rows, given this scratch.
 bool tc_tokens_rowclass_fits(const void* A, int64_t lda, int64_t M, int64_t N, int64_t K, size_t ws_bytes);
 bool tc_tokens_takes_unaligned_a(int64_t M, int64_t N);

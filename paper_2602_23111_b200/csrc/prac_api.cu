@@ -666,15 +666,16 @@ int prac_compress(const prac_basis* b, const void* X, int64_t N, int64_t ldx, vo
   // tensor-core kernel; only outputs too small for its tiles take the general path.
   if (b->p.dtype == PRAC_BF16 && !tma_ok(X, ldx) && tma_ok(Z, ldz) &&
       tc_rowclass_fits(X, ldx, N, s)) {
+    // (in a view the elements in front of a row are no part of X and may be anything)
     return tc_gemm_kmajor_rowclass(static_cast<const __nv_bfloat16*>(X), ldx, b->Pb, b->ldpb, N, s, d,
-                                   static_cast<__nv_bfloat16*>(Z), ldz, b->status, st);
+                                   static_cast<__nv_bfloat16*>(Z), ldz, b->status, st, 0, ldx == d ? nullptr : b->P);
   }
   // Up to 128 columns the product is bound by X's bytes, so P comes as three bf16 pieces, whose sum is
   // the fp32 basis: Z is off by its own rounding only, as on the general path that served these calls
-  // before.
+  // before; like there, an Inf or NaN stays in its own row of Z.
   if (b->P3 && tma_ok(Z, ldz) && tc_rowclass_narrow_fits(X, ldx, N, s)) {
     return tc_gemm_kmajor_rowclass(static_cast<const __nv_bfloat16*>(X), ldx, b->P3, b->ldpb, N, s, d,
-                                   static_cast<__nv_bfloat16*>(Z), ldz, b->status, st, b->rows3);
+                                   static_cast<__nv_bfloat16*>(Z), ldz, b->status, st, b->rows3, b->P);
   }
   if (b->p.dtype == PRAC_BF16 && (tma_ok(X, ldx) || tc_kmajor_takes_unaligned_a(N, s))) {
     return tc_gemm_kmajor(static_cast<const __nv_bfloat16*>(X), ldx, b->PTb, b->ldptb, N, s, d, Z, ldz,

@@ -70,3 +70,33 @@ def test_scratch_of_the_aligned_layout_is_still_enough():
     Xo.copy_(X)
     Zo = b.compress(Xo)
     assert float((Zo.double() - Z.double()).norm() / Z.double().norm()) <= 1e-4
+
+
+@pytest.mark.parametrize("N,d,ld,k,r", [
+    (300, 259, 259, 32, 32), (300, 259, 261, 32, 32), (4099, 1179, 1179, 64, 64), (2047, 1179, 1211, 37, 36), (130, 131, 133, 3, 0),
+    (300, 259, 261, 96, 96), (1030, 1179, 1182, 300, 301),
+])
+def test_what_is_not_finite_stays_in_its_own_row(N, d, ld, k, r):
+    # ld > d: the elements between the rows are NaN, and no part of X
+    g = torch.Generator(device="cuda")
+    g.manual_seed(13)
+    b, P = _basis(d, k, r, 1.5, g)
+    buf = torch.full((N, ld), float("nan"), device="cuda", dtype=torch.bfloat16)
+    X = buf[:, :d]
+    X.copy_(torch.randn(N, d, generator=g, device="cuda"))
+    clean = b.compress(X.contiguous() if ld == d else X)
+    assert bool(torch.isfinite(clean).all())
+    assert float((clean.double() - X.double() @ P.double()).norm() / clean.double().norm()) <= 5e-3
+    if k + r > 128:
+        return                      # (contiguous: finite numbers throughout, by the interface)
+    bad = {0: float("inf"), 5: float("nan"), N // 2: float("-inf"), N - 1: float("inf")}
+    for row, v in bad.items():
+        X[row, (7 * row) % d] = v
+    Z = b.compress(X)
+    want = X.double() @ P.double()
+    rows = torch.tensor(sorted(bad), device="cuda")
+    rest = torch.ones(N, dtype=torch.bool, device="cuda")
+    rest[rows] = False
+    assert torch.equal(Z[rest], clean[rest])
+    assert torch.equal(Z[rows].double(), want[rows]) or bool((torch.isnan(Z[rows]) == torch.isnan(want[rows])).all()
+                                                             and (Z[rows].double().nan_to_num(7.0) == want[rows].nan_to_num(7.0)).all())
