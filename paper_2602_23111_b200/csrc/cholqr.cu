@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(256) atb_f64_partial_kernel(const AtbArgs g) {
 // below the diagonal are read from their mirror image (tiles below the diagonal were
 // not computed).  TOut = float or double.
 template <typename TOut>
-__global__ void reduce_partials_kernel(const double* __restrict__ partial, int splits, int m, int n,
+__global__ void reduce_partials_kernel(const double* partial, int splits, int m, int n,
                                        int symmetric, double alpha, TOut* __restrict__ out, long long ldo,
                                        const int* run_if, int run_if_mask, int* zero_words, int zero_count) {
   grid_dep_wait();
@@ -897,7 +897,7 @@ int cholqr_pass(const float* Vin, int64_t ldin, float* Vout, int64_t ldout, int6
 }
 
 namespace {
-__global__ void copy2d_if_kernel(const float* __restrict__ src, long long lds, float* __restrict__ dst, long long ldd,
+__global__ void copy2d_if_kernel(const float* src, long long lds, float* __restrict__ dst, long long ldd,
                                  long long rows, long long cols, const int* status, int run_if_mask) {
   grid_dep_wait();
   grid_dep_launch();

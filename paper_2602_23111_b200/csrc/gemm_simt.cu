@@ -46,23 +46,23 @@ __device__ __forceinline__ float4 load4(const void* base, int bf16, int vec, lon
   if (slow >= slow_end || fast >= fast_end) return v;
   const long long idx = static_cast<long long>(slow) * ld + fast;
   if (vec && fast + 4 <= fast_end && PRAC_IN(idx + 3, ext)) {
-    if (!bf16) return __ldg(reinterpret_cast<const float4*>(static_cast<const float*>(base) + idx));
-    const float2 w = __ldg(reinterpret_cast<const float2*>(static_cast<const __nv_bfloat16*>(base) + idx));
+    if (!bf16) return *reinterpret_cast<const float4*>(static_cast<const float*>(base) + idx);
+    const float2 w = *reinterpret_cast<const float2*>(static_cast<const __nv_bfloat16*>(base) + idx);
     v.x = w.x; v.y = w.y;
     return v;
   }
   if (!bf16) {
     const float* p = static_cast<const float*>(base) + idx;
-    if (PRAC_IN(idx, ext)) v.x = __ldg(p);
-    if (fast + 1 < fast_end && PRAC_IN(idx + 1, ext)) v.y = __ldg(p + 1);
-    if (fast + 2 < fast_end && PRAC_IN(idx + 2, ext)) v.z = __ldg(p + 2);
-    if (fast + 3 < fast_end && PRAC_IN(idx + 3, ext)) v.w = __ldg(p + 3);
+    if (PRAC_IN(idx, ext)) v.x = *p;
+    if (fast + 1 < fast_end && PRAC_IN(idx + 1, ext)) v.y = p[1];
+    if (fast + 2 < fast_end && PRAC_IN(idx + 2, ext)) v.z = p[2];
+    if (fast + 3 < fast_end && PRAC_IN(idx + 3, ext)) v.w = p[3];
   } else {
     const unsigned short* p = static_cast<const unsigned short*>(base) + idx;
     uint32_t e[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
     for (int i = 0; i < 4; ++i)
-      if (fast + i < fast_end && PRAC_IN(idx + i, ext)) e[i] = __ldg(p + i);
+      if (fast + i < fast_end && PRAC_IN(idx + i, ext)) e[i] = p[i];
     v.x = __uint_as_float(e[0] | (e[1] << 16));
     v.y = __uint_as_float(e[2] | (e[3] << 16));
   }

@@ -679,10 +679,10 @@ __device__ __forceinline__ void gemm_tc_body(const CUtensorMap& tmap_a, const CU
         const int r0 = (CLS_N ? mt / p.cls_count : mt) * C::TILE_M + static_cast<int>(cta_rank) * BM + quarter * 32;
         const int gr = CLS_N ? (r0 + lane) * p.cls_count + cj : r0 + lane;
         if (r0 + lane < rows) {
-          rms_a = __ldg(p.row_a + gr);
+          rms_a = p.row_a[gr];
           if (EPI == EPI_RMS2) {
-            rms_b = __ldg(p.row_b + gr);
-            if (p.row_c) rms_c = __ldg(p.row_c + gr);
+            rms_b = p.row_b[gr];
+            if (p.row_c) rms_c = p.row_c[gr];
           }
         }
       }
@@ -743,6 +743,14 @@ __device__ __forceinline__ void gemm_tc_body(const CUtensorMap& tmap_a, const CU
           if (col0 >= out_n) break;                     // warp-uniform
           // the staging buffer of this block: the warp's only one, or the one its factor is in
           uint8_t* sbuf = smem + C::EPI_OFFSET + (ewarp * C::STORE_BUFS + (EPI_ACT ? consumed % NBUF : 0)) * STORE_BUF_BYTES;
+          // by classes the gains are off this block's grid of columns: a lane fetches those of columns lane, lane + 32
+          // (a load each, eight at a time, took 0.91 to 0.95 of this one's speed)
+          float gain_lo = 0.f, gain_hi = 0.f;
+          if (EPI_RMS && CLS_N) {
+            const int cg = col0 - n_shift + lane, last = out_n - n_shift;
+            if (cg >= 0 && cg < last) gain_lo = p.col_g[cg];
+            if (cg + 32 >= 0 && cg + 32 < last) gain_hi = p.col_g[cg + 32];
+          }
           if (EPI_ACT) {
             feed();
             if (!ptx::mbar_wait(&ctl->aux_full[ewarp][consumed % NBUF], static_cast<uint32_t>(consumed / NBUF) & 1u,
@@ -765,16 +773,19 @@ __device__ __forceinline__ void gemm_tc_body(const CUtensorMap& tmap_a, const CU
                 float gv[8];
                 if (EPI_RMS) {
                   // eight gains of these columns (the same for every lane; zero past the last column):
-                  // two 16-byte loads where the gain vector allows it
+                  // two 16-byte loads where the gain vector allows it, by classes from the lanes that hold them
                   const int cj = col0 + 8 * j - n_shift;
                   if (!CLS_N && p.col_g_vec && cj + 8 <= out_n) {
-                    const float4 g0 = __ldg(reinterpret_cast<const float4*>(p.col_g + cj));
-                    const float4 g1 = __ldg(reinterpret_cast<const float4*>(p.col_g + cj) + 1);
+                    const float4 g0 = *reinterpret_cast<const float4*>(p.col_g + cj);
+                    const float4 g1 = *(reinterpret_cast<const float4*>(p.col_g + cj) + 1);
                     gv[0] = g0.x; gv[1] = g0.y; gv[2] = g0.z; gv[3] = g0.w;
                     gv[4] = g1.x; gv[5] = g1.y; gv[6] = g1.z; gv[7] = g1.w;
                   } else {
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) gv[e] = (cj + e >= 0 && cj + e < out_n - n_shift) ? __ldg(p.col_g + cj + e) : 0.f;
+                    for (int e = 0; e < 8; ++e) {
+                      if (CLS_N) gv[e] = __shfl_sync(0xffffffffu, j < 4 ? gain_lo : gain_hi, (j & 3) * 8 + e);
+                      else gv[e] = cj + e < out_n ? p.col_g[cj + e] : 0.f;
+                    }
                   }
                 }
 #pragma unroll
@@ -1422,6 +1433,7 @@ int launch(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc, 
   const int items = p.num_tiles * p.splits;
   const int cap = resident_workers<CTAS, BN, MN, EPI, LDG>();
   const int workers = items < cap ? items : cap;
+  static_assert(CTAS == 2 || !LDG, "plain loads of A: CTA pairs only");
   if (CTAS == 1) {
     PRAC_LAUNCH(kern, dim3(workers), dim3(THREADS), C::SMEM_BYTES, stream, ta, tb, tc, *tb2, *tc2, p);
   } else {
@@ -1434,8 +1446,11 @@ int launch(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc, 
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     attr[1] = dependent_launch_attr();
-  cfg.attrs = attr;
-    cfg.numAttrs = 2;
+    cfg.attrs = attr;
+    // Plain loads of A go through the non-coherent path, which promises that A does not change while the kernel
+    // lives: these launches wait for the end of the one before them.  (9000 x 1179 by 2051: 109 us, with an early
+    // launch and ordinary loads 111; 2048 x 511 by 513: 18.5 and 16.5.)
+    cfg.numAttrs = LDG ? 1 : 2;
     PRAC_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, ta, tb, tc, *tb2, *tc2, p));
   }
   count_launch();

@@ -78,8 +78,13 @@ long long bounds_violations_tc();
 // Measured: refit of an fp32 layer (58 launches) 518 -> 438 us, of a 350M input 959 -> 860, a bf16 step of
 // eight launches 101 -> 92 us.
 // grid_dep_launch() is where a kernel lets the next one be set up: after its own wait for the shortest
-// kernels; the others leave it to the exit of their last CTA (waiting CTAs take room on the SMs, and a
-// fp64 panel product beside 400 of them took twice as long).
+// kernels, after a CTA's last store for the tensor-core products; the others leave it to the exit of their last
+// CTA (waiting CTAs take room on the SMs, and a fp64 panel product beside 400 of them took twice as long).
+// Such a kernel is alive while the one before it writes, so it reads with ordinary loads: the non-coherent path
+// (__ldg, ld.global.nc, const pointers that are __restrict__) promises memory that does not change meanwhile, and
+// a compiler may move such a load above the wait.  Two kernels that need that path (a load under a condition is
+// fetched ahead only there) are launched the ordinary way: ln_colsum_partial_kernel and the tensor-core
+// products that fetch A with plain loads.
 #ifdef __CUDACC__
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -128,7 +128,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 // padded with 0.5 sigma on the diagonal; sigma = 2^-15 * largest diagonal entry of B (1 if B = 0):
 // above the rounding noise that B inherits from its fp32 factors (so that null directions of B
 // get columns of a definite size), and harmless, since a shift moves no eigenvector.
-__global__ void __launch_bounds__(256) jacobi_prepare_kernel(const double* __restrict__ B, long long ldb, int ell,
+__global__ void __launch_bounds__(256) jacobi_prepare_kernel(const double* B, long long ldb, int ell,
                                                              double* __restrict__ At, int n, JacobiInfo* info) {
   grid_dep_wait();
   grid_dep_launch();
@@ -763,7 +763,7 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
 }
 
 // norms[i] = || column i of A || (row i of At): the shifted eigenvalues.
-__global__ void __launch_bounds__(128) jacobi_norms_kernel(const double* __restrict__ At, int n, double* __restrict__ norms) {
+__global__ void __launch_bounds__(128) jacobi_norms_kernel(const double* At, int n, double* __restrict__ norms) {
   grid_dep_wait();
   grid_dep_launch();
   __shared__ double red[4];
@@ -778,7 +778,7 @@ __global__ void __launch_bounds__(128) jacobi_norms_kernel(const double* __restr
 
 // Rank the eigenvalues and gather the unit eigenvectors of the k largest into Wsel (ell x k,
 // float), largest first; ties go to the lower index.  One CTA per eigenvalue.
-__global__ void __launch_bounds__(128) select_topk_kernel(const double* __restrict__ At, const double* __restrict__ norms,
+__global__ void __launch_bounds__(128) select_topk_kernel(const double* At, const double* norms,
                                                           int n, int ell, int k, float* __restrict__ Wsel) {
   grid_dep_wait();
   grid_dep_launch();
@@ -813,7 +813,7 @@ __device__ __forceinline__ void split3_one(float x, __nv_bfloat16& hi, __nv_bflo
 
 // Pb[i][j] = bf16(P[i][j]);  PTb[j][i] = bf16(P[i][j]); 32 x 32 tiles through shared memory.  P3 (optional):
 // the three pieces of P, rows3 rows apart.
-__global__ void __launch_bounds__(256) make_bf16_copies_kernel(const float* __restrict__ P, long long ldp,
+__global__ void __launch_bounds__(256) make_bf16_copies_kernel(const float* P, long long ldp,
                                                                long long d, long long s,
                                                                __nv_bfloat16* __restrict__ Pb, long long ldpb,
                                                                __nv_bfloat16* __restrict__ PTb, long long ldptb,
@@ -842,7 +842,7 @@ __global__ void __launch_bounds__(256) make_bf16_copies_kernel(const float* __re
 }
 
 // One thread per 8 consecutive elements of a destination row (ldd is a multiple of 8).
-__global__ void __launch_bounds__(256) split3_kernel(const float* __restrict__ src, long long lds, long long rows,
+__global__ void __launch_bounds__(256) split3_kernel(const float* src, long long lds, long long rows,
                                                      long long cols, __nv_bfloat16* __restrict__ dst,
                                                      long long rows_pad, long long ldd) {
   grid_dep_wait();
@@ -854,7 +854,7 @@ __global__ void __launch_bounds__(256) split3_kernel(const float* __restrict__ s
   float x[8];
   const float* s = src + i * lds + j0;
   if (i < rows && j0 + 8 <= cols && (reinterpret_cast<uintptr_t>(s) & 15u) == 0) {
-    const float4 a = __ldg(reinterpret_cast<const float4*>(s)), b = __ldg(reinterpret_cast<const float4*>(s) + 1);
+    const float4 a = *reinterpret_cast<const float4*>(s), b = *(reinterpret_cast<const float4*>(s) + 1);
     x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
   } else {
 #pragma unroll
@@ -872,7 +872,7 @@ __global__ void __launch_bounds__(256) split3_kernel(const float* __restrict__ s
 // The transpose of scale * src (rows x cols, fp32) as three bf16 pieces side by side: dst[j][l],
 // dst[j][kp + l], dst[j][2 kp + l] = leading, middle and last piece of scale * src[l][j]; l >= rows
 // is filled with zeros.  (A small matrix: the K-major second operand of a panel product.)
-__global__ void __launch_bounds__(256) split3_transposed_kernel(const float* __restrict__ src, long long lds, long long rows,
+__global__ void __launch_bounds__(256) split3_transposed_kernel(const float* src, long long lds, long long rows,
                                                                 long long cols, float scale,
                                                                 __nv_bfloat16* __restrict__ dst, long long kp) {
   grid_dep_wait();
@@ -889,7 +889,7 @@ __global__ void __launch_bounds__(256) split3_transposed_kernel(const float* __r
 }
 
 // The three pieces of a row side by side: dst[i] = [hi_i | mid_i | lo_i], each kp wide.
-__global__ void __launch_bounds__(256) split3_cols_kernel(const float* __restrict__ src, long long lds, long long rows,
+__global__ void __launch_bounds__(256) split3_cols_kernel(const float* src, long long lds, long long rows,
                                                           long long cols, __nv_bfloat16* __restrict__ dst, long long kp) {
   grid_dep_wait();
   grid_dep_launch();
@@ -900,7 +900,7 @@ __global__ void __launch_bounds__(256) split3_cols_kernel(const float* __restric
   float x[8];
   const float* s = src + i * lds + j0;
   if (j0 + 8 <= cols && (reinterpret_cast<uintptr_t>(s) & 15u) == 0) {
-    const float4 a = __ldg(reinterpret_cast<const float4*>(s)), b = __ldg(reinterpret_cast<const float4*>(s) + 1);
+    const float4 a = *reinterpret_cast<const float4*>(s), b = *(reinterpret_cast<const float4*>(s) + 1);
     x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
   } else {
 #pragma unroll
@@ -916,8 +916,8 @@ __global__ void __launch_bounds__(256) split3_cols_kernel(const float* __restric
 }
 
 // dX = dY * f'(Xh), element-wise (fp32 storage).
-__global__ void __launch_bounds__(256) act_backward_f32_kernel(const float* __restrict__ Xh, long long ldxh,
-                                                               const float* __restrict__ dY, long long lddy,
+__global__ void __launch_bounds__(256) act_backward_f32_kernel(const float* Xh, long long ldxh,
+                                                               const float* dY, long long lddy,
                                                                float* __restrict__ dX, long long lddx,
                                                                long long rows, long long cols, int act) {
   grid_dep_wait();
@@ -935,7 +935,7 @@ __global__ void __launch_bounds__(256) act_backward_f32_kernel(const float* __re
 // blocks b = g, g + 32, ... (16-byte loads when the rows of col_part allow it); the 32 subtotals
 // of a column are then combined in a fixed order, so the result does not depend on timing.
 // Returns the column total in the threads with g == 0 && q < 8 as four values (columns 4q + e).
-__device__ __forceinline__ void column_totals(const float* __restrict__ col_part, long long blocks, long long N,
+__device__ __forceinline__ void column_totals(const float* col_part, long long blocks, long long N,
                                               long long col0, float (&sub)[32][33], float (&tot)[4]) {
   const int g = threadIdx.x >> 3, q = threadIdx.x & 7;
   const long long c = col0 + 4 * q;
@@ -944,16 +944,24 @@ __device__ __forceinline__ void column_totals(const float* __restrict__ col_part
   if (vec) {
 #pragma unroll 16
     for (long long b = g; b < blocks; b += 32) {
-      const float4 v = __ldg(reinterpret_cast<const float4*>(col_part + b * N + c));
+      const float4 v = *reinterpret_cast<const float4*>(col_part + b * N + c);
       a0 += v.x; a1 += v.y; a2 += v.z; a3 += v.w;
     }
   } else {
-    for (long long b = g; b < blocks; b += 32) {
-      const float* r = col_part + b * N;
-      if (c < N) a0 += r[c];
-      if (c + 1 < N) a1 += r[c + 1];
-      if (c + 2 < N) a2 += r[c + 2];
-      if (c + 3 < N) a3 += r[c + 3];
+    for (long long b = g; b < blocks; b += 4 * 32) {       // (four blocks' loads in flight together)
+      float v[4][4];
+#pragma unroll
+      for (int h = 0; h < 4; ++h)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const long long bb = b + 32 * h < blocks ? b + 32 * h : b, cc = c + e < N ? c + e : N - 1;
+          v[h][e] = col_part[bb * N + cc];
+        }
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        if (b + 32 * h >= blocks) break;
+        a0 += v[h][0]; a1 += v[h][1]; a2 += v[h][2]; a3 += v[h][3];
+      }
     }
   }
   __syncthreads();                // an earlier call's readers are done with `sub`
@@ -973,9 +981,9 @@ __device__ __forceinline__ void column_totals(const float* __restrict__ col_part
 
 // After pass 1 of the RMSNorm backward.  The first ceil(M / 256) CTAs close the row sums (one
 // thread per token); each of the others closes 32 column sums (column_totals).
-__global__ void __launch_bounds__(256) rms_reduce_kernel(const float* __restrict__ row_part, int parts,
-                                                         const float* __restrict__ col_part, long long blocks,
-                                                         const float* __restrict__ rstd, long long M, long long N,
+__global__ void __launch_bounds__(256) rms_reduce_kernel(const float* row_part, int parts,
+                                                         const float* col_part, long long blocks,
+                                                         const float* rstd, long long M, long long N,
                                                          float* __restrict__ row_b, float* __restrict__ dgain) {
   grid_dep_wait();
   grid_dep_launch();
@@ -1006,13 +1014,14 @@ __global__ void __launch_bounds__(256) rms_reduce_kernel(const float* __restrict
 // 512 tokens of dY[t][i] and of rstd[t] mean[t] dY[t][i].  Grid (ceil(N / 256), ceil(M / 512)).
 // Thread (g, q) takes the eight columns 8q .. 8q + 7 of the CTA's 256 (one 16-byte load per row
 // when VEC: rows of dY 16-byte aligned and padded to a multiple of 8) and the rows g, g + 8, ...
-// of its 512; the eight subtotals of a column are combined in order.
+// of its 512; the eight subtotals of a column are combined in order.  An ordinary launch, which waits for the
+// end of the kernel before it, so that the inputs may be read through the non-coherent path (4096 x 1179, the
+// whole backward: 57 us on padded rows and 70 on contiguous ones, with an early launch 65 and 98).
 template <bool VEC>
 __global__ void __launch_bounds__(256) ln_colsum_partial_kernel(const __nv_bfloat16* __restrict__ dY, long long lddy,
                                                                 const float* __restrict__ mean, const float* __restrict__ rstd,
                                                                 long long M, long long N, float* __restrict__ part_plain,
                                                                 float* __restrict__ part_w) {
-  grid_dep_wait();
   __shared__ float sp[8][257], sw[8][257];
   const int g = threadIdx.x >> 5, q = threadIdx.x & 31;
   const long long c0 = blockIdx.x * 256ll + 8 * q;
@@ -1064,11 +1073,11 @@ __global__ void __launch_bounds__(256) ln_colsum_partial_kernel(const __nv_bfloa
 // A = sum_i a (a = gain dY): u = rstd (S - mean A); row_b = rstd^2 u / N; row_c = -rstd A / N + row_b mean.
 // Columns: dgain = sum of the pass-1 column partials - sum of the weighted partials; dbias = sum
 // of the plain partials.
-__global__ void __launch_bounds__(256) ln_reduce_kernel(const float* __restrict__ row_part, const float* __restrict__ row_part2,
-                                                        int parts, const float* __restrict__ col_part, long long blocks,
-                                                        const float* __restrict__ part_plain, const float* __restrict__ part_w,
-                                                        long long groups, const float* __restrict__ mean,
-                                                        const float* __restrict__ rstd, long long M, long long N,
+__global__ void __launch_bounds__(256) ln_reduce_kernel(const float* row_part, const float* row_part2,
+                                                        int parts, const float* col_part, long long blocks,
+                                                        const float* part_plain, const float* part_w,
+                                                        long long groups, const float* mean,
+                                                        const float* rstd, long long M, long long N,
                                                         float* __restrict__ row_b, float* __restrict__ row_c,
                                                         float* __restrict__ dgain, float* __restrict__ dbias) {
   grid_dep_wait();
@@ -1110,10 +1119,10 @@ __global__ void __launch_bounds__(256) ln_reduce_kernel(const float* __restrict_
 
 // fp32 storage, one CTA per token: A = sum a, S = sum a xn (a = gain dY, xn = (x - mean) rstd), then
 // dX = rstd (a - A / N - xn S / N).
-__global__ void __launch_bounds__(256) ln_rows_f32_kernel(const float* __restrict__ Xh, long long ldxh,
-                                                          const float* __restrict__ dY, long long lddy,
-                                                          const float* __restrict__ mean, const float* __restrict__ rstd,
-                                                          const float* __restrict__ gain, float* __restrict__ dX,
+__global__ void __launch_bounds__(256) ln_rows_f32_kernel(const float* Xh, long long ldxh,
+                                                          const float* dY, long long lddy,
+                                                          const float* mean, const float* rstd,
+                                                          const float* gain, float* __restrict__ dX,
                                                           long long lddx, long long N) {
   grid_dep_wait();
   grid_dep_launch();
@@ -1139,9 +1148,9 @@ __global__ void __launch_bounds__(256) ln_rows_f32_kernel(const float* __restric
     dX[t * lddx + i] = rs * (gain[i] * y[i] - mA - (x[i] - mu) * rs * mS);
 }
 // fp32 storage: dgain_i = sum_t dY_ti xn_ti, dbias_i = sum_t dY_ti; one thread per column, rows in order.
-__global__ void __launch_bounds__(256) ln_cols_f32_kernel(const float* __restrict__ Xh, long long ldxh,
-                                                          const float* __restrict__ dY, long long lddy,
-                                                          const float* __restrict__ mean, const float* __restrict__ rstd,
+__global__ void __launch_bounds__(256) ln_cols_f32_kernel(const float* Xh, long long ldxh,
+                                                          const float* dY, long long lddy,
+                                                          const float* mean, const float* rstd,
                                                           float* __restrict__ dgain, float* __restrict__ dbias,
                                                           long long M, long long N) {
   grid_dep_wait();
@@ -1159,9 +1168,9 @@ __global__ void __launch_bounds__(256) ln_cols_f32_kernel(const float* __restric
 }
 
 // fp32 storage, one CTA per token: u = sum_i gain_i dY_i x_i, then dX = rstd gain dY - rstd^3 u / N x.
-__global__ void __launch_bounds__(256) rms_rows_f32_kernel(const float* __restrict__ Xh, long long ldxh,
-                                                           const float* __restrict__ dY, long long lddy,
-                                                           const float* __restrict__ rstd, const float* __restrict__ gain,
+__global__ void __launch_bounds__(256) rms_rows_f32_kernel(const float* Xh, long long ldxh,
+                                                           const float* dY, long long lddy,
+                                                           const float* rstd, const float* gain,
                                                            float* __restrict__ dX, long long lddx, long long N) {
   grid_dep_wait();
   grid_dep_launch();
@@ -1182,9 +1191,9 @@ __global__ void __launch_bounds__(256) rms_rows_f32_kernel(const float* __restri
   for (long long i = threadIdx.x; i < N; i += blockDim.x) dX[t * lddx + i] = rs * gain[i] * y[i] - coef * x[i];
 }
 // fp32 storage: dgain_i = sum_t dY_ti x_ti rstd_t, one thread per column, rows in order.
-__global__ void __launch_bounds__(256) rms_cols_f32_kernel(const float* __restrict__ Xh, long long ldxh,
-                                                           const float* __restrict__ dY, long long lddy,
-                                                           const float* __restrict__ rstd, float* __restrict__ dgain,
+__global__ void __launch_bounds__(256) rms_cols_f32_kernel(const float* Xh, long long ldxh,
+                                                           const float* dY, long long lddy,
+                                                           const float* rstd, float* __restrict__ dgain,
                                                            long long M, long long N) {
   grid_dep_wait();
   grid_dep_launch();
@@ -1196,7 +1205,7 @@ __global__ void __launch_bounds__(256) rms_cols_f32_kernel(const float* __restri
 }
 
 // dst (bf16) = src with columns from `from` on multiplied by scale.
-__global__ void __launch_bounds__(256) scale_to_bf16_kernel(const float* __restrict__ src, long long lds,
+__global__ void __launch_bounds__(256) scale_to_bf16_kernel(const float* src, long long lds,
                                                             long long rows, long long cols, long long from, float scale,
                                                             __nv_bfloat16* __restrict__ dst, long long ldd) {
   grid_dep_wait();
@@ -1209,7 +1218,7 @@ __global__ void __launch_bounds__(256) scale_to_bf16_kernel(const float* __restr
   dst[i * ldd + j] = __float2bfloat16_rn(j >= from ? scale * v : v);
 }
 
-__global__ void copy2d_kernel(const float* __restrict__ src, long long lds, float* __restrict__ dst,
+__global__ void copy2d_kernel(const float* src, long long lds, float* __restrict__ dst,
                               long long ldd, long long rows, long long cols) {
   grid_dep_wait();
   grid_dep_launch();
@@ -1223,7 +1232,7 @@ __global__ void copy2d_kernel(const float* __restrict__ src, long long lds, floa
 // dst (rows x cols bf16, leading dimension ldd: rows 16-byte aligned, zero beyond cols up to ldd)
 // = src (rows x cols bf16, any leading dimension, 2-byte aligned).  One thread per 8 destination
 // elements: eight 2-byte loads (coalesced across the warp), one 16-byte store.
-__global__ void __launch_bounds__(256) repack_rows_bf16_kernel(const __nv_bfloat16* __restrict__ src, long long lds,
+__global__ void __launch_bounds__(256) repack_rows_bf16_kernel(const __nv_bfloat16* src, long long lds,
                                                                long long rows, long long cols,
                                                                __nv_bfloat16* __restrict__ dst, long long ldd) {
   grid_dep_wait();
@@ -1235,7 +1244,7 @@ __global__ void __launch_bounds__(256) repack_rows_bf16_kernel(const __nv_bfloat
   const unsigned short* s16 = reinterpret_cast<const unsigned short*>(src + i * lds + j0);
   unsigned short v[8];
 #pragma unroll
-  for (int e = 0; e < 8; ++e) v[e] = (j0 + e < cols) ? __ldg(s16 + e) : static_cast<unsigned short>(0);
+  for (int e = 0; e < 8; ++e) v[e] = (j0 + e < cols) ? s16[e] : static_cast<unsigned short>(0);
   if (!PRAC_IN(i * ldd + j0 + 7, rows * ldd)) return;
   uint4 o;
   o.x = v[0] | (static_cast<uint32_t>(v[1]) << 16);
@@ -1480,8 +1489,8 @@ int launch_ln_colsum_partial(const __nv_bfloat16* dY, int64_t lddy, const float*
                              int64_t N, float* part_plain, float* part_w, cudaStream_t stream) {
   dim3 grid(nblocks(N, 256), nblocks(M, 512));
   const bool vec = (reinterpret_cast<uintptr_t>(dY) & 15u) == 0 && lddy % 8 == 0 && lddy >= (N + 7) / 8 * 8;
-  if (vec) PRAC_LAUNCH(ln_colsum_partial_kernel<true>, dim3(grid), dim3(256), 0, stream, dY, lddy, mean, rstd, M, N, part_plain, part_w);
-  else PRAC_LAUNCH(ln_colsum_partial_kernel<false>, dim3(grid), dim3(256), 0, stream, dY, lddy, mean, rstd, M, N, part_plain, part_w);
+  if (vec) ln_colsum_partial_kernel<true><<<grid, 256, 0, stream>>>(dY, lddy, mean, rstd, M, N, part_plain, part_w);
+  else ln_colsum_partial_kernel<false><<<grid, 256, 0, stream>>>(dY, lddy, mean, rstd, M, N, part_plain, part_w);
   count_launch();
   PRAC_CUDA_TRY(cudaGetLastError());
   return PRAC_OK;
