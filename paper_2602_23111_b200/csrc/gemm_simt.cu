@@ -357,14 +357,15 @@ int launch_trans(const DevGemm& d, int ta, int tb, long long tiles, cudaStream_t
 }
 
 // CTAs of a shape that can be resident at once in clusters of `parts` (two per SM without clusters; larger
-// clusters do not fill every group of SMs: 33 of 4 and 16 of 8 at one CTA per SM).
+// clusters do not fill every group of SMs: 33 of 4 and 16 of 8 at one CTA per SM); 0 where the device has no
+// room for such a cluster (a part of a GPU may not).
 template <int TM, int TN, int SL>
 int resident_ctas(int parts, int sms) {
   using S = Shape<TM, TN, SL>;
   if (parts == 1) return 2 * sms;
   static DeviceValue cached[3];    // parts 2, 4, 8
   int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return sms; }
+  if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return 0; }
   DeviceValue& slot = cached[parts == 2 ? 0 : (parts == 4 ? 1 : 2)];
   if (slot.get(dev) > 0) return slot.get(dev);
   auto kern = gemm_simt_kernel<TM, TN, SL, false, false>;
@@ -381,7 +382,7 @@ int resident_ctas(int parts, int sms) {
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM) != cudaSuccess ||
       cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
     cudaGetLastError();
-    return sms;
+    return 0;
   }
   slot.set(dev, n * parts);
   return n * parts;
@@ -436,6 +437,7 @@ int gemm_general(const GemmArgs& g, cudaStream_t stream) {
       const long long steps = (g.K + BK * cand[c].sl * p - 1) / (BK * cand[c].sl * p);
       if (p > 1 && (steps < 2 || g.run_if != nullptr)) break;    // (an optional launch stays off the cluster barrier)
       const int fit = c == 0 ? resident_ctas<128, 128, 1>(p, sms) : (c == 1 ? resident_ctas<64, 64, 4>(p, sms) : resident_ctas<32, 32, 8>(p, sms));
+      if (fit < p) break;
       const double rounds = tiles * p > fit ? static_cast<double>(tiles * p) / fit : 1.0;     // of up to two CTAs per SM
       const double step = tiles * p <= fit / 2 ? cand[c].alone : cand[c].shared;
       const double est = rounds * (steps * step + (p == 1 ? 2.0 : (p == 2 ? 3.0 : (p == 4 ? 4.0 : 5.0))));
