@@ -8,8 +8,9 @@
 // among the thread groups of a CTA (SL slices of BK rows per step, summed through shared memory)
 // and among the CTAs of a cluster (2, 4 or 8 pieces, summed through distributed shared memory,
 // so no workspace is needed).  Both sums run in a fixed order.  Measured against the 64 x 64 tiles
-// with one serial walk over K that this replaces (fp32 layer, N = 2048, d = d_out = 512, k = r = 16):
-// compress and weight gradient 207 -> 32 us, the refit step 1089 -> 642 us.
+// with one serial walk over K that this replaced (fp32 layer, N = 2048, d = d_out = 512, k = r = 16):
+// compress and weight gradient 207 -> 32 us, the refit step 1089 -> 642 us by this alone (23 and 434 us with
+// what the launches and the rest of the fit have gained since).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -350,10 +351,9 @@ int launch_shape(DevGemm d, long long tiles, cudaStream_t stream) {
 }
 template <int TM, int TN, int SL>
 int launch_trans(const DevGemm& d, int ta, int tb, long long tiles, cudaStream_t stream) {
-  if (!ta && !tb) return launch_shape<TM, TN, SL, false, false>(d, tiles, stream);
-  if (!ta && tb) return launch_shape<TM, TN, SL, false, true>(d, tiles, stream);
-  if (ta && !tb) return launch_shape<TM, TN, SL, true, false>(d, tiles, stream);
-  return launch_shape<TM, TN, SL, true, true>(d, tiles, stream);
+  if (ta && tb) return PRAC_EINVAL;        // (nothing asks for it)
+  if (ta) return launch_shape<TM, TN, SL, true, false>(d, tiles, stream);
+  return tb ? launch_shape<TM, TN, SL, false, true>(d, tiles, stream) : launch_shape<TM, TN, SL, false, false>(d, tiles, stream);
 }
 
 // CTAs of a shape that can be resident at once in clusters of `parts` (two per SM without clusters; larger
@@ -391,6 +391,13 @@ int resident_ctas(int parts, int sms) {
 }  // namespace
 
 PRAC_BOUNDS_READER(bounds_violations_simt)
+
+#ifdef PRAC_DEBUG_BOUNDS
+// The bounds-checking build only: every product takes this tile (0, 1, 2: see `cand` below) and this number of
+// K pieces (1, 2, 4, 8) instead of those of the rule; tile < 0 gives the rule back.
+static int g_forced_tile = -1, g_forced_parts = 1;
+extern "C" void prac_debug_force_product(int tile, int parts) { g_forced_tile = tile; g_forced_parts = parts; }
+#endif
 
 int gemm_general(const GemmArgs& g, cudaStream_t stream) {
   if (g.M < 0 || g.N < 0 || g.K < 0) return PRAC_EINVAL;
@@ -445,6 +452,13 @@ int gemm_general(const GemmArgs& g, cudaStream_t stream) {
     }
   }
   if (best_t < 0.0) return PRAC_EINVAL;
+#ifdef PRAC_DEBUG_BOUNDS
+  if (g_forced_tile >= 0) {
+    best = g_forced_tile; parts = g.run_if != nullptr ? 1 : g_forced_parts;
+    const long long tm = (g.M + cand[best].tm - 1) / cand[best].tm, tn = (g.N + cand[best].tn - 1) / cand[best].tn;
+    best_tiles = symmetric ? tn * (tn + 1) / 2 : tm * tn;
+  }
+#endif
   d.parts = parts;
   d.tiles_n = static_cast<int>((g.N + cand[best].tn - 1) / cand[best].tn);
   if (best == 0) return launch_trans<128, 128, 1>(d, g.trans_a, g.trans_b, best_tiles, stream);

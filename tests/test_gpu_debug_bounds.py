@@ -100,3 +100,43 @@ def test_tiny_and_odd_shapes_stay_inside_their_buffers(dbg, shape):
     b.draw_random(seed=3, draw_counter=2)
     assert b.status() == dbg.PRAC_OK
     assert dbg.lib.prac_debug_bounds_violations() == before       # nothing stepped outside
+
+
+@pytest.mark.parametrize("parts", [1, 2, 4, 8])
+@pytest.mark.parametrize("tile", [0, 1, 2])
+def test_every_tile_and_cluster_of_the_general_product(dbg, tile, parts):
+    # The dispatch takes one of three tiles and one to eight pieces of K by estimated time; here each pair is
+    # forced, through every operand order (X P, X W^T, dY^T Z, the symmetric X^T X), on rows on and off the
+    # 16-byte grid, remainders of every tile, fewer steps than pieces, and an accumulated output.
+    # Bound: fp32 sums of at most N terms of random signs (see the general product's own tests).
+    force = dbg.lib.prac_debug_force_product
+    before = dbg.lib.prac_debug_bounds_violations()
+    g = torch.Generator(device="cuda")
+    g.manual_seed(9)
+    rel = lambda got, want: float((got.double() - want).norm() / want.norm())
+    for N, d, k, r, d_out, pad in ((1029, 133, 20, 17, 67, 1), (260, 264, 40, 24, 136, 0), (7, 9, 3, 2, 5, 0)):
+        X = torch.randn(N, d + pad, generator=g, device="cuda")[:, :d]
+        dY = torch.randn(N, d_out + pad, generator=g, device="cuda")[:, :d_out]
+        W = torch.randn(d_out, d + pad, generator=g, device="cuda")[:, :d]
+        P = torch.linalg.qr(torch.randn(d, k + r, generator=g, device="cuda", dtype=torch.float64))[0].float()
+        b = dbg.Basis(d, k, r, torch.float32)
+        b.set(P[:, :k].clone(memory_format=torch.contiguous_format), P[:, k:].clone(memory_format=torch.contiguous_format), 1.75)
+        scale = torch.ones(k + r, dtype=torch.float64, device="cuda")
+        scale[k:] = 1.75
+        force(tile, parts)
+        try:
+            Z = b.compress(X)
+            Y = b.linear_forward(X, W, want_z=False)[0]
+            Xh = b.reconstruct(Z)
+            dW = b.weight_grad(dY, Z)
+            twice = b.weight_grad(dY, Z, out=dW.clone(), accumulate=True)
+            C = b.gram(X)
+        finally:
+            force(-1, 1)
+        bound = 4 * N ** 0.5 * 2 ** -24 + 2 ** -21
+        want = (dY.double().t() @ Z.double() * scale) @ P.double().t()
+        assert rel(Z, X.double() @ P.double()) <= bound and rel(Y, X.double() @ W.double().t()) <= bound
+        assert rel(Xh, (Z.double() * scale) @ P.double().t()) <= bound
+        assert rel(dW, want) <= 2 * bound and rel(twice, 2 * want) <= 2 * bound
+        assert torch.equal(C, C.t()) and rel(C, X.double().t() @ X.double()) <= 2 * bound
+    assert dbg.lib.prac_debug_bounds_violations() == before

@@ -29,7 +29,8 @@ def _rows(n, cols, pad, g):
 
 
 # (tokens, width, k, r, outputs, columns of padding): remainders of the 32, 64 and 128 tiles and of 16-row steps,
-# one step only, products that fill the chip without pieces and products cut into eight
+# one step only, products that fill the chip and products that leave it idle (which tile and how many pieces of K
+# each takes is the dispatch's choice; every pair is forced in test_gpu_debug_bounds.py)
 @pytest.mark.parametrize("N,d,k,r,d_out,pad", [
     (1, 5, 2, 2, 1, 0), (33, 31, 3, 0, 65, 1), (130, 129, 8, 9, 127, 3), (2048, 512, 16, 16, 512, 0),
     (2049, 257, 40, 24, 511, 2), (8191, 1023, 64, 63, 1000, 1), (8192, 1024, 64, 64, 1024, 0), (700, 1024, 128, 128, 4096, 4),
