@@ -774,12 +774,16 @@ int atb_f64(const float* A, int64_t lda, const float* B, int64_t ldb, int64_t d,
   if (!ws || ws_bytes < need) return PRAC_EWORKSPACE;
   g.partial = static_cast<double*>(ws);
   g.run_if = run_if; g.run_if_mask = run_if_mask;
-  PRAC_LAUNCH(atb_f64_partial_kernel, dim3(dim3(static_cast<unsigned>(g.num_tiles), static_cast<unsigned>(g.splits))), dim3(256), 0, stream, g);
+  PRAC_LAUNCH(atb_f64_partial_kernel, dim3(static_cast<unsigned>(g.num_tiles), static_cast<unsigned>(g.splits)), dim3(256), 0, stream, g);
   count_launch();
   if (out_double)
-    PRAC_LAUNCH(reduce_partials_kernel<double>, dim3(nblocks(m * n, 256)), dim3(256), 0, stream, g.partial, g.splits, g.m, g.n, symmetric, alpha, static_cast<double*>(out), ldo, run_if, run_if_mask, static_cast<int*>(zero_after), zero_bytes / 4);
+    PRAC_LAUNCH(reduce_partials_kernel<double>, dim3(nblocks(m * n, 256)), dim3(256), 0, stream,
+                g.partial, g.splits, g.m, g.n, symmetric, alpha, static_cast<double*>(out), ldo, run_if, run_if_mask,
+                static_cast<int*>(zero_after), zero_bytes / 4);
   else
-    PRAC_LAUNCH(reduce_partials_kernel<float>, dim3(nblocks(m * n, 256)), dim3(256), 0, stream, g.partial, g.splits, g.m, g.n, symmetric, alpha, static_cast<float*>(out), ldo, run_if, run_if_mask, static_cast<int*>(zero_after), zero_bytes / 4);
+    PRAC_LAUNCH(reduce_partials_kernel<float>, dim3(nblocks(m * n, 256)), dim3(256), 0, stream,
+                g.partial, g.splits, g.m, g.n, symmetric, alpha, static_cast<float*>(out), ldo, run_if, run_if_mask,
+                static_cast<int*>(zero_after), zero_bytes / 4);
   count_launch();
   PRAC_CUDA_TRY(cudaGetLastError());
   return PRAC_OK;
@@ -923,7 +927,8 @@ int launch_copy2d_if(const float* src, int64_t lds, float* dst, int64_t ldd, int
   if (!status) return PRAC_EINVAL;
   if (rows > 0 && cols > 0) {
     const unsigned want = nblocks(rows * cols, 256);
-    PRAC_LAUNCH(copy2d_if_kernel, dim3(want < 296u ? want : 296u), dim3(256), 0, stream, src, lds, dst, ldd, rows, cols, status, run_if_mask);
+    PRAC_LAUNCH(copy2d_if_kernel, dim3(want < 296u ? want : 296u), dim3(256), 0, stream,
+                src, lds, dst, ldd, rows, cols, status, run_if_mask);
     count_launch();
   }
   PRAC_LAUNCH(clear_status_bits_kernel, dim3(1), dim3(1), 0, stream, status, clear_bits);

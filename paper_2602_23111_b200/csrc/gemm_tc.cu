@@ -2120,7 +2120,8 @@ int tc_gemm_tokens(const __nv_bfloat16* A, int64_t lda, const __nv_bfloat16* B, 
       for (int j = 0; j < c.P; ++j) r.cls_shift[j] = c.shift[j];
       const long long work = static_cast<long long>(M) * ((N + 3) / 4);
       const unsigned blocks = static_cast<unsigned>((work + 255) / 256);
-      if (type_c == ET_BF16) PRAC_LAUNCH(splitk_reduce_kernel<__nv_bfloat16>, dim3(blocks), dim3(256), 0, stream, r, static_cast<__nv_bfloat16*>(Cout));
+      if (type_c == ET_BF16) PRAC_LAUNCH(splitk_reduce_kernel<__nv_bfloat16>, dim3(blocks), dim3(256), 0, stream,
+                                         r, static_cast<__nv_bfloat16*>(Cout));
       else PRAC_LAUNCH(splitk_reduce_kernel<float>, dim3(blocks), dim3(256), 0, stream, r, static_cast<float*>(Cout));
       count_launch();
       PRAC_CUDA_TRY(cudaGetLastError());
@@ -2176,7 +2177,8 @@ int tc_gemm_tokens(const __nv_bfloat16* A, int64_t lda, const __nv_bfloat16* B, 
   if (planes) {
     if (t.tile_m % 64 != 0 || t.bn % 64 != 0) return PRAC_EINVAL;
     const dim3 pairs(static_cast<unsigned>(planes->ld / 64), static_cast<unsigned>(planes->rows_pad / 64));
-    PRAC_LAUNCH(splitk_reduce_sym_split3_kernel, dim3(pairs), dim3(threads), 0, stream, r, static_cast<float*>(Cout), planes->base, planes->rows_pad, planes->ld);
+    PRAC_LAUNCH(splitk_reduce_sym_split3_kernel, dim3(pairs), dim3(threads), 0, stream,
+                r, static_cast<float*>(Cout), planes->base, planes->rows_pad, planes->ld);
   } else if (symmetric && t.tile_m % 32 == 0 && t.bn % 32 == 0) {
     const int nblk = static_cast<int>((N + 31) / 32);
     const dim3 pairs(static_cast<unsigned>(nblk), static_cast<unsigned>(nblk));

@@ -1440,7 +1440,8 @@ int launch_make_bf16_copies(const float* P, int64_t ldp, int64_t d, int64_t s, i
                             __nv_bfloat16* Pcb, __nv_bfloat16* Pb, int64_t ldpb,
                             __nv_bfloat16* PTb, int64_t ldptb, __nv_bfloat16* P3, int64_t rows3, cudaStream_t stream) {
   dim3 grid(static_cast<unsigned>((s + 31) / 32), static_cast<unsigned>((d + 31) / 32));
-  PRAC_LAUNCH(make_bf16_copies_kernel, dim3(grid), dim3(256), 0, stream, P, ldp, d, s, Pb, ldpb, PTb, ldptb, Pcb, k, static_cast<float>(c), P3, rows3);
+  PRAC_LAUNCH(make_bf16_copies_kernel, dim3(grid), dim3(256), 0, stream,
+              P, ldp, d, s, Pb, ldpb, PTb, ldptb, Pcb, k, static_cast<float>(c), P3, rows3);
   count_launch();
   PRAC_CUDA_TRY(cudaGetLastError());
   return PRAC_OK;
@@ -1500,7 +1501,9 @@ int launch_ln_reduce(const float* row_part, const float* row_part2, int parts, c
                      const float* part_plain, const float* part_w, int64_t groups, const float* mean, const float* rstd,
                      int64_t M, int64_t N, float* row_b, float* row_c, float* dgain, float* dbias, cudaStream_t stream) {
   const unsigned ctas = nblocks(M, 256) + nblocks(N, 32);
-  PRAC_LAUNCH(ln_reduce_kernel, dim3(ctas), dim3(256), 0, stream, row_part, row_part2, parts, col_part, blocks, part_plain, part_w, groups, mean, rstd, M, N, row_b, row_c, dgain, dbias);
+  PRAC_LAUNCH(ln_reduce_kernel, dim3(ctas), dim3(256), 0, stream,
+              row_part, row_part2, parts, col_part, blocks, part_plain, part_w, groups, mean, rstd, M, N, row_b, row_c,
+              dgain, dbias);
   count_launch();
   PRAC_CUDA_TRY(cudaGetLastError());
   return PRAC_OK;
@@ -1540,7 +1543,8 @@ int launch_scale_to_bf16(const float* src, int64_t lds, int64_t rows, int64_t co
 int launch_act_backward_f32(const float* Xh, int64_t ldxh, const float* dY, int64_t lddy, float* dX, int64_t lddx,
                             int64_t rows, int64_t cols, int act, cudaStream_t stream) {
   if (rows <= 0 || cols <= 0) return PRAC_OK;
-  PRAC_LAUNCH(act_backward_f32_kernel, dim3(nblocks(rows * cols, 256)), dim3(256), 0, stream, Xh, ldxh, dY, lddy, dX, lddx, rows, cols, act);
+  PRAC_LAUNCH(act_backward_f32_kernel, dim3(nblocks(rows * cols, 256)), dim3(256), 0, stream,
+              Xh, ldxh, dY, lddy, dX, lddx, rows, cols, act);
   count_launch();
   PRAC_CUDA_TRY(cudaGetLastError());
   return PRAC_OK;
