@@ -269,17 +269,18 @@ __device__ __forceinline__ void blk_store(const double (*S)[CP], double* M, int 
 }
 
 // The 8 x 8 diagonal sub-block of a diagonal block, by one warp in registers: lane (r, c) holds
-// M[r][2c], M[r][2c + 1] (the accumulator layout of dmma_884).  Elimination without square roots: on
-// return the pivots are in pv[0..8) and their reciprocals in xi[0..8), and the strictly lower triangle
-// of M holds that of L^-1, M = L diag(pv) L^T (the elimination M[i][.] -= m M[j][.], m = M[j][i] / pv_j,
-// applied to an identity kept there too).  Only the upper triangle is read.  A pivot that is not safely
-// positive relative to the column's original squared norm is replaced by a guard value.  The
-// reciprocal is a hardware approximation refined by two Newton steps (full double accuracy).
+// M[r][2c], M[r][2c + 1] (the accumulator layout of dmma_884).  Elimination without square roots and
+// without a division: on return row r of the triangular matrix T = S L^-1, M = L diag(pv) L^T, S a diagonal
+// matrix of positive scales, is in the strictly lower part of M and S_r in `scale`; `pivot` is S_r pv_r, so that
+// M = T^-1 diag(pivot * scale) T^-T.  (An identity kept in the lower triangle is eliminated along
+// with M.)  Only the upper triangle is read.  A pivot that is not safely positive relative to the column's
+// original squared norm is replaced by a guard value.
 //
-// This is the careful form, one column at a time, for sub-blocks in which a pivot is bad.
-__device__ __noinline__ void sub_chol_guarded(double& m0, double& m1, const double* guard, double* pv_out, double* xi_out,
+// This is the careful form, one column at a time with S = 1, for sub-blocks in which a pivot is bad.
+__device__ __noinline__ void sub_chol_guarded(double& m0, double& m1, const double* guard, double& scale, double& pivot,
                                               int* dev_status, int flag_bit) {
   const int lane = threadIdx.x & 31, r = lane >> 2, c = lane & 3;
+  scale = 1.0;
 #pragma unroll 1
   for (int j = 0; j < 8; ++j) {
     const int row = j << 2;
@@ -290,9 +291,8 @@ __device__ __noinline__ void sub_chol_guarded(double& m0, double& m1, const doub
       pv = guard[j];
       if (lane == 0 && flag_bit && dev_status) atomicOr(dev_status, flag_bit);
     }
-    const double x = 1.0 / pv;
-    if (lane == 0) { pv_out[j] = pv; xi_out[j] = x; }
-    const double m = ((r & 1) ? t1 : t0) * x;                    // M[j][r] / pv
+    if (r == j) pivot = pv;
+    const double m = ((r & 1) ? t1 : t0) / pv;                   // M[j][r] / pv
     const double u0 = fma(-m, rj0, m0), u1 = fma(-m, rj1, m1);
     // U part, and L^-1 columns before j: updated; L^-1 column j starts here; the rest waits
     const int l0 = 2 * c, l1 = 2 * c + 1;
@@ -303,37 +303,47 @@ __device__ __noinline__ void sub_chol_guarded(double& m0, double& m1, const doub
   }
 }
 
-// The same without the test in the dependent chain (pivot -> reciprocal -> multipliers -> next pivot, about
-// 165 cycles per column; two columns per step through their 2 x 2 determinant took the same: the step is
-// bound by the instructions it issues as much as by the chain).  1 / pv = x0 (1 + e + e^2 + ..),
-// e = 1 - pv x0: the hardware's x0 is good to 20 bits, so the terms up to e^2 leave a relative error
-// below 2^-60.  Returns whether all pivots were good; where not, the caller repeats the sub-block in the
-// careful form.
-__device__ __forceinline__ bool sub_chol(double& m0, double& m1, const double* guard, double* pv_out, double* xi_out) {
+// The same with neither a division nor a test in the dependent chain.  Column j turns every later row r into
+// (pv_j M[r] - M[j][r] M[j]) 2^-e, e the exponent of the new scale: rows keep a common scale S in [1, 2) instead
+// of being divided by the pivot, and a column is a shuffle and three operations (with a reciprocal
+// approximation and its refinement in the chain it took 165 cycles).  Returns whether all pivots were good; where
+// not, the caller repeats the sub-block in the careful form.
+__device__ __forceinline__ bool sub_chol(double& m0, double& m1, const double* guard, double& scale, double& pivot) {
   const int lane = threadIdx.x & 31, r = lane >> 2, c = lane & 3;
+  const int l0 = 2 * c, l1 = 2 * c + 1;
   bool good = true;
+  double S = 1.0;
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const int row = j << 2;
     const double pv = __shfl_sync(0xffffffffu, (j & 1) ? m1 : m0, row | (j >> 1));
+    good = good && pv > guard[j] * S;                            // (false for NaN)
+    if (r == j) { scale = S; pivot = pv; }
+    if (j == 7) break;
     const double rj0 = __shfl_sync(0xffffffffu, m0, row | c), rj1 = __shfl_sync(0xffffffffu, m1, row | c);
     const double t0 = __shfl_sync(0xffffffffu, m0, row | (r >> 1)), t1 = __shfl_sync(0xffffffffu, m1, row | (r >> 1));
-    good = good && pv > guard[j];                                // (false for NaN)
-    double x0;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x0) : "d"(pv));
-    const double e = fma(-pv, x0, 1.0);
-    const double corr = fma(e, e, e);
-    const double q0 = ((r & 1) ? t1 : t0) * x0;
-    const double m = fma(q0, corr, q0);                          // M[j][r] / pv
-    if (lane == 0) { pv_out[j] = pv; xi_out[j] = fma(x0, corr, x0); }
-    const double u0 = fma(-m, rj0, m0), u1 = fma(-m, rj1, m1);
-    const int l0 = 2 * c, l1 = 2 * c + 1;
-    const double n0 = (l0 >= r || l0 < j) ? u0 : ((l0 == j) ? -m : m0);
-    const double n1 = (l1 >= r || l1 < j) ? u1 : ((l1 == j) ? -m : m1);
+    const double t = (r & 1) ? t1 : t0;                          // M[j][r]
+    const double Sp = S * pv;
+    // 2^-e with e the exponent of Sp (a good pivot is a positive normal number)
+    const double two = __hiloint2double(0x7fe00000 - (__double2hiint(Sp) & 0x7ff00000), 0);
+    const double u0 = fma(pv, m0, -(t * rj0)) * two, u1 = fma(pv, m1, -(t * rj1)) * two;
+    const double start = -(t * S) * two;                         // column j of T begins (its diagonal entry is S)
+    S = Sp * two;
+    const double n0 = (l0 >= r || l0 < j) ? u0 : ((l0 == j) ? start : m0);
+    const double n1 = (l1 >= r || l1 < j) ? u1 : ((l1 == j) ? start : m1);
     m0 = r > j ? n0 : m0;
     m1 = r > j ? n1 : m1;
   }
   return good;
+}
+
+// 1 / x for a positive normal x: 1 / x = x0 (1 + e + e^2 + ..), e = 1 - x x0; the hardware's x0 is good to 20 bits, so the
+// terms up to e^2 leave a relative error below 2^-60.
+__device__ __forceinline__ double rcp_f64(double x) {
+  double x0;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x0) : "d"(x));
+  const double e = fma(-x, x0, 1.0);
+  return fma(x0, fma(e, e, e), x0);
 }
 
 // The 256 threads that compute (the chain's CTA has more, see chol_inv_kernel).
@@ -349,62 +359,75 @@ __device__ __forceinline__ void bar_arrive(int id, int threads) {
 }
 __device__ __forceinline__ void main_sync() { bar_sync(1, CHOL_MAIN); }
 
+// What a diagonal block's factorisation leaves in shared memory beside the block: limits below which a pivot is
+// replaced, scaled pivots, their inverse square roots.
+struct CholDiag { double guard[CB], pi[CB], rs[CB]; };
+__device__ __forceinline__ double pivot_guard(double diagonal_on_entry) {
+  return diagonal_on_entry > 0.0 ? 1e-13 * diagonal_on_entry : 1.0;
+}
+
 // In shared memory: D (CB x CB, symmetric positive definite on entry, upper triangle used) -> I = R^-1
-// (upper), where R^T R = D, by the 256 main threads.  The chain of 32 dependent column steps is what this costs, so
+// (upper), where R^T R = D, by the 256 main threads, which have met at a barrier since D and x.guard were written.  The
+// chain of 32 dependent column steps is what this costs, so
 // it runs in one warp's registers, eight columns at a time (one block barrier per column over all
 // 256 threads took 330 cycles each); the other 8 x 8 tiles are brought up to date on the fp64 tensor
-// cores by the other warps, one tile each, beside the next sub-block's chain.  With T = L_ss^-1 of sub-block s, U_q = T D_sq, V_q = diag(1/pv) U_q:
-// D_pq -= V_p^T U_q, and the same elimination applied to an identity (E) gives the block rows of L^-1:
-// Lin_sc = T E_sc (E_ss = 1), E_pc -= V_p^T Lin_sc.  R^-1 = (L^-1)^T diag(1/sqrt(pv)).
-// W: scratch, rows 0..7 U, 8..15 V (columns 8 q ..), 16..23 T, two in turn, 24..31 warp 0's own U and V.  Dinv: R^-1 goes there (global memory) too.
-__device__ void blk_chol_inv(double (*D)[CP], double (*I)[CP], double (*Lin)[CP], double (*E)[CP], double (*W)[CP],
-                             double* Dinv, const double* diag0, int n, int j0, int* dev_status, int flag_bit) {
-  __shared__ double guard_sh[CB], pv_sh[CB], xi_sh[CB];
+// cores by the other warps, one tile each, beside the next sub-block's chain.  With T = S L_ss^-1 of sub-block s (sub_chol),
+// pi = pivot * scale, U_q = T D_sq, V_q = diag(1/pi) U_q:
+// D_pq -= V_p^T U_q, and the same elimination applied to an identity (E) gives the block rows of S L^-1:
+// Lin_sc = T E_sc (E_ss = 1), E_pc -= V_p^T Lin_sc.  R^-1 = (S L^-1)^T diag(1/sqrt(pi)).
+// W: scratch, rows 0..7 U, 8..15 V (columns 8 q ..), 16..23 T, two in turn.  emit(r, c, v0, v1): elements (r, c), (r, c + 1) of
+// R^-1, which are written to I too.
+template <typename Emit>
+__device__ __forceinline__ void blk_chol_inv(double (*D)[CP], double (*I)[CP], double (*Lin)[CP], double (*E)[CP], double (*W)[CP],
+                                             CholDiag& x, int* dev_status, int flag_bit, Emit emit) {
   static_assert(CB == 32, "four sub-blocks of eight columns");
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31, g = lane >> 2, q4 = lane & 3;
-  double (*U)[CP] = W; double (*V)[CP] = W + 8; double (*own)[CP] = W + 24;
-  if (t < CB) {
-    const double d0 = (j0 + t < n) ? diag0[j0 + t] : 1.0;
-    guard_sh[t] = d0 > 0.0 ? 1e-13 * d0 : 1.0;
-  }
+  double (*U)[CP] = W; double (*V)[CP] = W + 8; double (*T)[CP] = W + 16;
   double m0 = 0.0, m1 = 0.0;
-  main_sync();
   if (warp == 0) { m0 = D[g][2 * q4]; m1 = D[g][2 * q4 + 1]; }
 #pragma unroll 1
   for (int s = 0; s < CB / 8; ++s) {
     const int o = 8 * s;
     const int tc = 8 * (s & 1);                    // T of this sub-block: W[16 ..][tc ..]
-    double (*T)[CP] = W + 16;
+    double t0 = 0.0, t1 = 0.0, pi = 1.0;
     if (warp == 0) {
       const double k0 = m0, k1 = m1;
-      if (!sub_chol(m0, m1, guard_sh + o, pv_sh + o, xi_sh + o)) {     // (the lanes agree)
+      double scale = 1.0, pivot = 1.0;
+      if (!sub_chol(m0, m1, x.guard + o, scale, pivot)) {     // (the lanes agree)
         m0 = k0; m1 = k1;
-        sub_chol_guarded(m0, m1, guard_sh + o, pv_sh + o, xi_sh + o, dev_status, flag_bit);
+        sub_chol_guarded(m0, m1, x.guard + o, scale, pivot, dev_status, flag_bit);
       }
-      const double t0 = 2 * q4 < g ? m0 : (2 * q4 == g ? 1.0 : 0.0), t1 = 2 * q4 + 1 < g ? m1 : (2 * q4 + 1 == g ? 1.0 : 0.0);
+      t0 = 2 * q4 < g ? m0 : (2 * q4 == g ? scale : 0.0);
+      t1 = 2 * q4 + 1 < g ? m1 : (2 * q4 + 1 == g ? scale : 0.0);
+      pi = pivot * scale;
       T[g][tc + 2 * q4] = t0; T[g][tc + 2 * q4 + 1] = t1;
       Lin[o + g][o + 2 * q4] = t0; Lin[o + g][o + 2 * q4 + 1] = t1;
+      if (q4 == 0) x.pi[o + g] = pi;
     }
     main_sync();
     if (warp == 0) {
-      // the next diagonal sub-block, on its own: U and V of block column s + 1 (the others make them again)
+      // the next diagonal sub-block, on its own and in registers (the others make U and V of block column s + 1
+      // again): a fragment of A may name its columns in any order that B's rows follow, so T goes in as it lies;
+      // U comes back with its rows over the lanes and is turned by shuffles
       if (s + 1 < CB / 8) {
         const int p = o + 8;
         double acc[2] = {0.0, 0.0};
-#pragma unroll
-        for (int kk = 0; kk < 2; ++kk) dmma_884(acc, T[g][tc + 4 * kk + q4], D[o + 4 * kk + q4][p + g]);
-        const double x = xi_sh[o + g];
-        own[g][2 * q4] = acc[0]; own[g][2 * q4 + 1] = acc[1];
-        own[g][8 + 2 * q4] = x * acc[0]; own[g][8 + 2 * q4 + 1] = x * acc[1];
-        __syncwarp();
+        dmma_884(acc, t0, D[o + 2 * q4][p + g]);
+        dmma_884(acc, t1, D[o + 2 * q4 + 1][p + g]);
+        const double xi = rcp_f64(pi);
         double upd[2] = {0.0, 0.0};
 #pragma unroll
-        for (int kk = 0; kk < 2; ++kk) dmma_884(upd, own[4 * kk + q4][8 + g], own[4 * kk + q4][g]);
+        for (int kk = 0; kk < 2; ++kk) {
+          const int from = ((4 * kk + q4) << 2) | (g >> 1);
+          const double u0 = __shfl_sync(0xffffffffu, acc[0], from), u1 = __shfl_sync(0xffffffffu, acc[1], from);
+          const double u = (g & 1) ? u1 : u0;      // U[4 kk + q4][g]
+          dmma_884(upd, u * __shfl_sync(0xffffffffu, xi, (4 * kk + q4) << 2), u);
+        }
         m0 = D[p + g][p + 2 * q4] - upd[0];
         m1 = D[p + g][p + 2 * q4 + 1] - upd[1];
-        __syncwarp();
       }
     } else {
+      if (warp == 7 && lane < 8) x.rs[o + lane] = rsqrt(x.pi[o + lane]);
       // three tiles: U_q, q > s, and Lin_sc, c < s
       if (warp < 4) {
         const int q = warp - 1 < s ? warp - 1 : warp;
@@ -415,9 +438,9 @@ __device__ void blk_chol_inv(double (*D)[CP], double (*I)[CP], double (*Lin)[CP]
         if (q < s) {
           Lin[o + g][8 * q + 2 * q4] = acc[0]; Lin[o + g][8 * q + 2 * q4 + 1] = acc[1];
         } else {
-          const double x = xi_sh[o + g];
+          const double xi = rcp_f64(x.pi[o + g]);
           U[g][8 * q + 2 * q4] = acc[0]; U[g][8 * q + 2 * q4 + 1] = acc[1];
-          V[g][8 * q + 2 * q4] = x * acc[0]; V[g][8 * q + 2 * q4 + 1] = x * acc[1];
+          V[g][8 * q + 2 * q4] = xi * acc[0]; V[g][8 * q + 2 * q4 + 1] = xi * acc[1];
         }
       }
       bar_sync(8, CHOL_MAIN - 32);
@@ -447,18 +470,13 @@ __device__ void blk_chol_inv(double (*D)[CP], double (*I)[CP], double (*Lin)[CP]
     }
   }
   main_sync();
-  {
-    const int c = t % CB;                      // the same column for all of a thread's elements
-    const double scale = rsqrt(pv_sh[c]);
 #pragma unroll
-    for (int e = 0; e < CB * CB / CHOL_MAIN; ++e) {
-      const int r = (t + CHOL_MAIN * e) / CB;
-      const double v = (r <= c) ? Lin[c][r] * scale : 0.0;
-      I[r][c] = v;
-      Dinv[r * CB + c] = v;
-    }
+  for (int e = 0; e < CB * CB / 2 / CHOL_MAIN; ++e) {
+    const int r = (t + CHOL_MAIN * e) / (CB / 2), c = 2 * (t % (CB / 2));
+    const double v0 = r <= c ? Lin[c][r] * x.rs[c] : 0.0, v1 = r <= c + 1 ? Lin[c + 1][r] * x.rs[c + 1] : 0.0;
+    *reinterpret_cast<double2*>(&I[r][c]) = make_double2(v0, v1);
+    emit(r, c, v0, v1);
   }
-  main_sync();
 }
 
 // Up to three blocks fetched in one round trip: all of a thread's loads are issued before the first store.
@@ -546,8 +564,9 @@ __device__ __forceinline__ bool chol_wait(CholSync* sy, const unsigned* word, un
 // leaves; nothing asynchronous is in flight here, so the early exit is clean.
 __global__ void __launch_bounds__(CHOL_MAIN + CHOL_HELP) chol_inv_kernel(const CholArgs a) {
   if (a.run_if_mask && pass_is_off(a.dev_status, a.run_if_mask)) return;
-  extern __shared__ double chol_smem[];
+  extern __shared__ __align__(16) double chol_smem[];
   __shared__ int ok_sh[2];
+  __shared__ CholDiag diag;
   double (*S0)[CP] = reinterpret_cast<double (*)[CP]>(chol_smem);
   double (*S1)[CP] = S0 + CB;
   double (*S2)[CP] = S1 + CB;
@@ -619,7 +638,15 @@ __global__ void __launch_bounds__(CHOL_MAIN + CHOL_HELP) chol_inv_kernel(const C
         main_sync();
       }
       if (j + 1 < nb) bar_arrive(4, CHOL_MAIN + CHOL_HELP);
-      blk_chol_inv(D, S1, S2, S3, S5, a.Dinv + static_cast<long long>(j) * CB * CB, a.diag0, n, j * CB, a.dev_status, a.flag_bit);
+      if (threadIdx.x < CB) {                      // (warp 0, which alone reads the limits)
+        const int i = j * CB + threadIdx.x;
+        diag.guard[threadIdx.x] = pivot_guard(i < n ? a.diag0[i] : 1.0);
+        __syncwarp();
+      }
+      double* const inv = a.Dinv + static_cast<long long>(j) * CB * CB;
+      blk_chol_inv(D, S1, S2, S3, S5, diag, a.dev_status, a.flag_bit,
+                   [&](int r, int c, double v0, double v1) { *reinterpret_cast<double2*>(&inv[r * CB + c]) = make_double2(v0, v1); });
+      main_sync();
       bar_arrive(2 + 4 * (j & 1), CHOL_MAIN + CHOL_HELP);
     }
     return;
@@ -715,6 +742,272 @@ __global__ void __launch_bounds__(CHOL_MAIN + CHOL_HELP) chol_inv_kernel(const C
     }
     if (worker == static_cast<int>(workers) - 1) { chol_emit(a, S1, j, j); sync(); }
   }
+}
+
+// ------------------------------------------------------------------ the same on one cluster, up to 16 blocks of columns
+// Shared memory of another CTA of the cluster.
+__device__ __forceinline__ uint32_t cluster_addr(const void* own, unsigned rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(own))), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ double2 cluster_ld(uint32_t addr) {
+  double2 v;
+  asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void cluster_st(uint32_t addr, double x, double y) {
+  asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(addr), "d"(x), "d"(y) : "memory");
+}
+__device__ __forceinline__ void cluster_st_flag(uint32_t addr, int v) {
+  asm volatile("st.release.cluster.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ int ld_flag(const int* own) {
+  int v;
+  asm volatile("ld.acquire.cluster.shared::cta.s32 %0, [%1];" : "=r"(v)
+               : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(own))) : "memory");
+  return v;
+}
+__device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+constexpr int CC_MAX = 16;                       // blocks of columns = CTAs of the cluster
+constexpr int CC_GROUPS = 2;                     // groups of 256 threads in a CTA
+// What the CTAs tell one another; every word is written by one CTA and only grows.
+struct ChainWords {
+  int row_done[CC_MAX];      // [x]: blocks (c, x), c < row_done[x], of R are final in CTA x
+  int inv_done[CC_MAX];      // [x]: 8 when the inverse of diagonal block x is final in CTA x (x before this one: stored here by CTA x's eight warps)
+  int abort;                 // a wait gave up
+};
+
+// Column blocks of G and block rows of the inverse stay in shared memory for the whole factorisation: CTA q of
+// the cluster holds the blocks (p, q), p <= q, of G, which become those of R, and row q of X = R^-1.  Step c, once R_cc^-1
+// is known: the CTAs right of c form R_cq = R_cc^-T G_cq and subtract R_cp^T R_cq from their blocks (p, q), p > c; the others
+// close X_qc = X_qc R_cc^-1 and subtract X_qc R_cx from their running sums X_qx, x > c.  The blocks R_cx of another CTA are
+// fetched from its shared memory when its flag says that they are final; nothing is ever overwritten that another
+// CTA may still want.  CTA c + 1, whose diagonal block the chain waits for, has nothing else to do in step c: R_cc^-1 is
+// stored into its shared memory as it is formed, and two products later it factors.
+//
+// The chain of diagonal blocks is what this costs.  A factorisation whose CTAs met through flags in global memory
+// (chol_inv_kernel) took 13 400 cycles a block, most of them the way of a block through L2 and back.
+//
+// Every wait on another CTA is bounded; a CTA that gives up tells the others, and all of them meet at the
+// cluster's barrier before any leaves, so that nobody's shared memory goes away under a reader.
+__global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const CholArgs a) {
+  grid_dep_wait();
+  if (a.run_if_mask && pass_is_off(a.dev_status, a.run_if_mask)) return;
+  extern __shared__ __align__(16) double chol_smem[];
+  __shared__ CholDiag diag;
+  __shared__ ChainWords words;
+  typedef double (*Blk)[CP];
+  const int n = a.n, nb = a.nb, q = static_cast<int>(blockIdx.x);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, group = tid >> 8, gt = tid & 255;
+  const int g = lane >> 2, q4 = lane & 3;
+  auto block = [&](int i) { return reinterpret_cast<Blk>(chol_smem + static_cast<size_t>(i) * CB * CP); };
+  auto col = [&](int p) { return block(p); };                 // (p, q) of G, then of R
+  auto inv = [&](int x) { return block(x + 1); };             // (q, x) of R^-1, x >= q
+  Blk const Lin = block(nb + 1), E = block(nb + 2), W = block(nb + 3), Dprev = block(nb + 4), Dfar = block(nb + 5);
+  Blk const stage = block(nb + 6 + group);
+  bool fail = false;
+
+  if (tid < static_cast<int>(sizeof(words) / sizeof(int))) reinterpret_cast<int*>(&words)[tid] = 0;
+  __syncthreads();
+  cluster_arrive();
+  // this CTA's column of G, padded with the identity
+  for (int idx = tid; idx < (q + 1) * CB * CB; idx += 256 * CC_GROUPS) {
+    const int i = idx / CB, j = idx % CB;
+    col(i / CB)[i % CB][j] = ld_pad(a.G, n, i, q * CB + j);
+  }
+  for (int idx = tid; idx < (nb - 1 - q) * CB * CP; idx += 256 * CC_GROUPS)      // the running sums
+    inv(q + 1)[idx / CP][idx % CP] = 0.0;
+  if (group == 1) chol_emit_zeros(a, q, nb);
+  cluster_wait();
+  __syncthreads();
+  if (tid < CB) diag.guard[tid] = pivot_guard(col(q)[tid][tid]);
+  __syncthreads();
+
+  auto give_up = [&]() {
+    fail = true;
+    for (int x = 0; x < nb; ++x) cluster_st_flag(cluster_addr(&words.abort, x), 1);
+  };
+  // One lane of a warp polls a word of this CTA's shared memory; where it gives up the caller carries on with what it
+  // has, until the CTA next meets and leaves together.
+  auto wait_word = [&](const int* word, int target) {
+    if (lane == 0 && !fail) {
+      unsigned polls = 0;
+      while (ld_flag(word) < target) {
+        if (++polls >= a.poll_limit) { give_up(); break; }
+        if ((polls & 63u) == 0u && ld_flag(&words.abort)) { fail = true; break; }
+      }
+    }
+    __syncwarp();
+  };
+  // the pairs (row, 2 columns) of a block that a thread of a group moves
+  auto pull = [&](uint32_t from, double2 (&v)[2]) {
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+      v[e] = cluster_ld(from + (((gt + 256 * e) >> 4) * CP + 2 * (gt & 15)) * 8);
+  };
+  auto put = [&](Blk to, const double2 (&v)[2]) {
+#pragma unroll
+    for (int e = 0; e < 2; ++e) *reinterpret_cast<double2*>(&to[(gt + 256 * e) >> 4][2 * (gt & 15)]) = v[e];
+  };
+
+  for (int c = 0; c < nb; ++c) {
+    if (c == q) {
+      if (group == 0) {
+        const bool next = q + 1 < nb;
+        const uint32_t far = next ? cluster_addr(Dprev, q + 1) : 0u;
+        blk_chol_inv(col(q), inv(q), Lin, E, W, diag, a.dev_status, a.flag_bit, [&](int r, int cc, double v0, double v1) {
+          if (next) cluster_st(far + (r * CP + cc) * 8, v0, v1);
+        });
+        // (each warp says that its part is there: inv_done counts them)
+        __syncwarp();
+        if (next && lane == 0) {
+          asm volatile("red.release.cluster.shared::cluster.add.u32 [%0], 1;" ::"r"(cluster_addr(&words.inv_done[q], q + 1)) : "memory");
+        }
+      }
+      __syncthreads();
+      // the CTA after this one counts the eight warps above, the others wait for this word
+      if (warp == 8 && lane < nb && lane != q && lane != q + 1) cluster_st_flag(cluster_addr(&words.inv_done[q], lane), 8);
+    } else {
+      // ---- R_cc^-1, then this CTA's own block of step c
+      Blk D = Dfar;
+      wait_word(&words.inv_done[c], 8);
+      if (c == q - 1) {
+        D = Dprev;
+      } else {
+        const int r = tid >> 4, cc = 2 * (tid & 15);
+        const double2 v = cluster_ld(cluster_addr(&block(c + 1)[r][cc], c));
+        *reinterpret_cast<double2*>(&Dfar[r][cc]) = v;
+        __syncthreads();
+      }
+      const int r0 = (warp >> 2) * 8, c0 = (warp & 3) * 8;    // a tile per warp
+      double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+      Blk const mine = c < q ? col(c) : inv(c);
+      // (R_cc^-1 is upper triangular: the products end where it does)
+      const int ks_end = c < q ? 2 * (warp >> 2) + 2 : 2 * (warp & 3) + 2;
+#pragma unroll
+      for (int ks = 0; ks < CB / 4; ++ks) {
+        if (ks >= ks_end) break;
+        const double x = c < q ? D[ks * 4 + q4][r0 + g] : mine[r0 + g][ks * 4 + q4];
+        const double y = c < q ? mine[ks * 4 + q4][c0 + g] : D[ks * 4 + q4][c0 + g];
+        dmma_884(acc[ks & 1], x, y);
+      }
+      __syncthreads();
+      *reinterpret_cast<double2*>(&mine[r0 + g][c0 + 2 * q4]) = make_double2(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
+    }
+    // every thread leaves here if one has given up
+    if (__syncthreads_or(fail)) { fail = true; break; }
+
+    if (c < q) {
+      if (warp == 15 && lane < nb && lane != q) cluster_st_flag(cluster_addr(&words.row_done[q], lane), c + 1);
+      Blk const R = col(c);
+      if (c == q - 1) {
+        // the diagonal block, at once: the upper 8 x 8 tiles, by the threads that factor it next
+        if (group == 0) {
+          for (int u = warp; u < 10; u += 8) {
+            int p = 0, left = u;
+            while (left >= 4 - p) { left -= 4 - p; ++p; }
+            const int r0 = 8 * p, c0 = 8 * (p + left);
+            double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+#pragma unroll
+            for (int ks = 0; ks < CB / 4; ++ks) dmma_884(acc[ks & 1], R[ks * 4 + q4][r0 + g], R[ks * 4 + q4][c0 + g]);
+            double2* o = reinterpret_cast<double2*>(&col(q)[r0 + g][c0 + 2 * q4]);
+            const double2 old = *o;
+            *o = make_double2(old.x - (acc[0][0] + acc[1][0]), old.y - (acc[0][1] + acc[1][1]));
+          }
+          main_sync();
+        }
+      } else {
+        // blocks (p, q), c < p <= q, dealt to the groups, (q, q) first: it needs nobody else's block
+        if (group == 0) blk_mm(col(q), R, R, 1);
+        double2 v[2];
+        int p = c + 1 + (1 - group);
+        if (p < q) { wait_word(&words.row_done[p], c + 1); pull(cluster_addr(R, p), v); }
+        for (; p < q; p += CC_GROUPS) {
+          bar_sync(1 + group, 256);            // the block before this one is done with
+          put(stage, v);
+          bar_sync(1 + group, 256);
+          if (p + CC_GROUPS < q) { wait_word(&words.row_done[p + CC_GROUPS], c + 1); pull(cluster_addr(R, p + CC_GROUPS), v); }
+          blk_mm(col(p), stage, R, 1);
+        }
+      }
+    } else {
+      // row q of the inverse: X_qx -= X_qc R_cx, x > c
+      Blk const X = inv(c);
+      double2 v[2];
+      int x = c + 1 + group;
+      if (x < nb) { wait_word(&words.row_done[x], c + 1); pull(cluster_addr(block(c), x), v); }
+      if (group == 1) chol_emit(a, X, q, c);
+      for (; x < nb; x += CC_GROUPS) {
+        bar_sync(1 + group, 256);
+        put(stage, v);
+        bar_sync(1 + group, 256);
+        if (x + CC_GROUPS < nb) { wait_word(&words.row_done[x + CC_GROUPS], c + 1); pull(cluster_addr(block(c), x + CC_GROUPS), v); }
+        blk_mm(inv(x), X, stage, 3);
+      }
+    }
+    // (the next step reads what the other group has brought up to date; the diagonal block is group 0's own)
+    if (c != q - 1) __syncthreads();
+  }
+  if (fail && lane == 0 && a.dev_status) atomicOr(a.dev_status, DEV_WAIT_EXPIRED);
+  cluster_arrive();
+  cluster_wait();
+}
+
+size_t chol_cluster_smem(int nb) {
+  const size_t need = static_cast<size_t>(nb + 6 + CC_GROUPS) * CB * CP * 8;
+  return need > static_cast<size_t>(CHOL_SMEM_ASK) ? need : static_cast<size_t>(CHOL_SMEM_ASK);
+}
+
+void chol_cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2], int nb, cudaStream_t stream) {
+  cfg = {};
+  cfg.gridDim = dim3(nb);
+  cfg.blockDim = dim3(256 * CC_GROUPS);
+  cfg.dynamicSmemBytes = chol_cluster_smem(nb);
+  cfg.stream = stream;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = nb;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1] = dependent_launch_attr();
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+}
+
+// Whether the current device can place a cluster of nb CTAs of chol_cluster_kernel (asked once per device and size).
+bool chol_cluster_fits(int nb) {
+  if (nb < 1 || nb > CC_MAX) return false;
+  static DeviceValue known[CC_MAX + 1];          // 1: no, 2: yes
+  static DeviceOnce attrs;
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) { (void)cudaGetLastError(); return false; }
+  const int v = known[nb].get(dev);
+  if (v != 0) return v == 2;
+  bool ok = true;
+  if (!attrs.done(dev)) {
+    ok = cudaFuncSetAttribute(chol_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(chol_cluster_smem(CC_MAX))) == cudaSuccess &&
+         cudaFuncSetAttribute(chol_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    if (ok) attrs.mark(dev);
+  }
+  if (ok) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    chol_cluster_config(cfg, attr, nb, nullptr);
+    int clusters = 0;
+    ok = cudaOccupancyMaxActiveClusters(&clusters, chol_cluster_kernel, &cfg) == cudaSuccess && clusters >= 1;
+  }
+  if (!ok) (void)cudaGetLastError();
+  known[nb].set(dev, ok ? 2 : 1);
+  return ok;
 }
 
 cudaError_t chol_smem_attr() {
@@ -859,30 +1152,37 @@ int cholqr_pass(const float* Vin, int64_t ldin, float* Vout, int64_t ldout, int6
   const bool tensor = run_if_mask == 0 && c.tensor && tc_init() == PRAC_OK && aligned16(Vout) && (ldout % 4) == 0;
   a.Rt3 = tensor ? c.Rt3 : nullptr;
   a.kp = static_cast<int>(c.kp);
-  const int rem = a.nb - 1;
-  // one group of 256 threads per task of the busiest step (trailing blocks plus the products of the
-  // inverse), two groups per CTA
-  int want = rem * (rem + 1) / 2;
-  for (int j = 1; j < a.nb; ++j) {
-    const int w = a.nb - j;
-    const int tasks = (w - 1) * w / 2 + j * w;
-    if (tasks > want) want = tasks;
+  if (chol_cluster_fits(a.nb)) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    chol_cluster_config(cfg, attr, a.nb, stream);
+    PRAC_CUDA_TRY(cudaLaunchKernelEx(&cfg, chol_cluster_kernel, a));
+  } else {
+    const int rem = a.nb - 1;
+    // one group of 256 threads per task of the busiest step (trailing blocks plus the products of the
+    // inverse), two groups per CTA
+    int want = rem * (rem + 1) / 2;
+    for (int j = 1; j < a.nb; ++j) {
+      const int w = a.nb - j;
+      const int tasks = (w - 1) * w / 2 + j * w;
+      if (tasks > want) want = tasks;
+    }
+    int grid = (want < 1 ? 1 : (want + 1) / 2) + 1;    // at least one CTA of workers, and CTA 0, which walks the diagonal
+    // ... and at most a quarter of the SMs, an SM each: a transformer block fits the bases of its four
+    // distinct inputs side by side (four streams), and factorisations whose CTAs share SMs hold one
+    // another up (their waits are as long as the slowest CTA)
+    {
+      const int sms = tc_num_sms();
+      const int quarter = sms >= 8 ? sms / 4 : 2;
+      if (grid > quarter) grid = quarter;
+    }
+    const int smem = CHOL_SMEM_ASK;
+    void* args[] = {const_cast<CholArgs*>(&a)};
+    PRAC_CUDA_TRY(chol_smem_attr());
+    // cooperative launch: CTAs wait for one another, so all have to be resident
+    PRAC_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(chol_inv_kernel), dim3(grid), dim3(CHOL_MAIN + CHOL_HELP), args,
+                                              smem, stream));
   }
-  int grid = (want < 1 ? 1 : (want + 1) / 2) + 1;    // at least one CTA of workers, and CTA 0, which walks the diagonal
-  // ... and at most a quarter of the SMs, an SM each: a transformer block fits the bases of its four
-  // distinct inputs side by side (four streams), and factorisations whose CTAs share SMs hold one
-  // another up (their waits are as long as the slowest CTA)
-  {
-    const int sms = tc_num_sms();
-    const int quarter = sms >= 8 ? sms / 4 : 2;
-    if (grid > quarter) grid = quarter;
-  }
-  const int smem = CHOL_SMEM_ASK;
-  void* args[] = {const_cast<CholArgs*>(&a)};
-  PRAC_CUDA_TRY(chol_smem_attr());
-  // cooperative launch: CTAs wait for one another, so all have to be resident
-  PRAC_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(chol_inv_kernel), dim3(grid), dim3(CHOL_MAIN + CHOL_HELP), args,
-                                            smem, stream));
   count_launch();
   if (tensor) {
     st = launch_split3_cols(Vin, ldin, d, n, c.V3, c.kp, stream);
