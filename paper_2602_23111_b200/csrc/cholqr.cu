@@ -1,7 +1,7 @@
 // Orthonormalisation of tall fp32 panels by Cholesky-QR, three launches per pass:
-//   1. G = V^T V accumulated in double over slices of the rows (atb_f64_partial_kernel) and
-//      summed in a fixed order (reduce_partials_kernel);
-//   2. R = chol(G) and R^-1 in one cooperative kernel (chol_inv_kernel), all in double;
+//   1. G = V^T V accumulated in double over slices of the rows that are summed in a fixed order (atb_f64_kernel);
+//   2. R = chol(G) and R^-1 in one kernel, all in double: a cluster up to 512 columns (chol_cluster_kernel), a cooperative
+//      launch above (chol_inv_kernel);
 //   3. V_out = V_in * R^-1: on the tensor cores for panels big enough to fill their tiles (both
 //      operands as three bf16 pieces, six chained cross terms: fp32 accuracy), else a general
 //      fp32 GEMM.
@@ -28,18 +28,90 @@ struct AtbArgs {
   const float* B; long long ldb;   // d x n
   int m, n;
   long long d;
-  int splits;                      // row slices
-  int tiles_m, tiles_n, num_tiles;
-  int symmetric;                   // A == B, m == n: only tiles reaching the upper triangle
-  double* partial;                 // [splits][m][n]
+  int tiles_n;
+  int symmetric;                   // A == B, m == n: only tiles reaching the upper triangle, mirrored
+  double alpha;
+  void* out; long long ldo;
+  int out_double;                  // out is double, else float
+  int next_early;                  // the next kernel may be set up from the start of this one
   const int* run_if;               // optional: the kernel does nothing unless *run_if & run_if_mask
   int run_if_mask;
+  int* zero_words; int zero_count; // words that the next kernel on the stream expects zeroed
 };
 
 // Kernels of an optional pass are always launched and look at a device word to see whether
 // they have anything to do (the host does not wait for the device to find out).
 __device__ __forceinline__ bool pass_is_off(const int* run_if, int mask) {
   return run_if != nullptr && (*reinterpret_cast<const volatile int*>(run_if) & mask) == 0;
+}
+
+// Shared memory of another CTA of the cluster.
+__device__ __forceinline__ uint32_t cluster_addr(const void* own, unsigned rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(own))), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ double2 cluster_ld(uint32_t addr) {
+  double2 v;
+  asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ double cluster_ld1(uint32_t addr) {
+  double v;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr) : "memory");
+  return v;
+}
+// (the store's 16 bytes are counted on the barrier when they have arrived)
+__device__ __forceinline__ void cluster_st_async(uint32_t addr, double2 v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%0], {%1, %2}, [%3];" ::"r"(addr), "d"(v.x), "d"(v.y), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void cluster_st_flag(uint32_t addr, int v) {
+  asm volatile("st.release.cluster.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+// A barrier for one event: an arrival, or, where bytes > 0, that many bytes stored by cluster_st_async.
+__device__ __forceinline__ void cluster_bar_init(uint64_t* own, unsigned bytes) {
+  const uint32_t b = static_cast<uint32_t>(__cvta_generic_to_shared(own));
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b) : "memory");
+  if (bytes) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cluster_bar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ bool cluster_try_wait(uint64_t* own) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred P;\n\t"
+      "mbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 P, [%1], 0;\n\t"
+      "selp.b32 %0, 1, 0, P;\n\t}"
+      : "=r"(ok) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(own))) : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ bool cluster_try_wait_acquire(uint64_t* own) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred P;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 P, [%1], 0;\n\t"
+      "selp.b32 %0, 1, 0, P;\n\t}"
+      : "=r"(ok) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(own))) : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ bool cluster_try_wait_rows(uint64_t* own) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred P;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 P, [%1], 0;\n\t"
+      "selp.b32 %0, 1, 0, P;\n\t}"
+      : "=r"(ok) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(own))) : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 __device__ __forceinline__ void atb_tile(const AtbArgs& g, int tile, int& ti, int& tj) {
@@ -60,125 +132,112 @@ __device__ __forceinline__ void dmma_884(double (&d)[2], double a, double b) {
                : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
 }
 
-// A 64 x 64 output tile over one slice of the rows: 16 rows at a time are widened to double in
-// shared memory (the next 16 are already on their way in registers), warp w multiplies 16 columns
-// of A (w / 2) by 32 columns of B (w % 2) on the fp64 tensor cores: six fragment loads for eight
-// products (the kernel waits on its shared-memory loads; 8 x 64 per warp took nine).
-__global__ void __launch_bounds__(256) atb_f64_partial_kernel(const AtbArgs g) {
+// A 64 x 64 output tile by one cluster: each CTA takes a slice of the rows, 16 at a time, three chunks ahead of the
+// products by asynchronous copies; warp w multiplies 16 columns
+// of A (w / 2) by 32 columns of B (w % 2) on the fp64 tensor cores: six fragment loads, widened to double, for eight
+// products.  Then every CTA adds up its rows of the
+// slices' tiles from the others' shared memory, in the order of the slices, and writes them.  (Slices that went through
+// global memory, 15 MB of them at 320 columns, took a second kernel of 8 us.)  The loops are short on purpose: most of these
+// launches last a few microseconds, and an SM fetches instructions that it has not seen at 270 cycles per 128 bytes.
+constexpr int AT_STAGES = 4;
+constexpr int AT_P = AT_T + 8;      // pitch of a row in shared memory: what four rows of a fragment load read lies in 32 banks
+__global__ void __launch_bounds__(256) atb_f64_kernel(const AtbArgs g) {
   grid_dep_wait();
-  __shared__ double As[AT_K][AT_T + 2];
-  __shared__ double Bs[AT_K][AT_T + 2];
+  if (g.next_early) grid_dep_launch();
+  __shared__ __align__(16) double tile[AT_T * AT_P];        // the chunks in flight (fp32), then the slice's tile
+  static_assert(AT_STAGES * 2 * AT_K * AT_P * sizeof(float) <= sizeof(tile), "the tile takes the place of the chunks");
   if (pass_is_off(g.run_if, g.run_if_mask)) return;
+  float* const raw = reinterpret_cast<float*>(tile);
   int ti, tj;
   atb_tile(g, blockIdx.x, ti, tj);
-  const int split = blockIdx.y;
-  const long long r0 = g.d * split / g.splits, r1 = g.d * (split + 1) / g.splits;
+  const int rank = blockIdx.y, slices = gridDim.y;          // (the cluster is 1 x slices)
+  const int r0 = static_cast<int>(g.d * rank / slices), r1 = static_cast<int>(g.d * (rank + 1) / slices);
   const int t = threadIdx.x;
   const int warp = t >> 5, lane = t & 31, gq = lane >> 2, q4 = lane & 3;
   const int m0 = ti * AT_T, n0 = tj * AT_T;
   const int wa = (warp >> 1) * 16, wb = (warp & 1) * 32;   // this warp's columns of A and of B within the tile
+  if (blockIdx.x == 0 && rank == 0)
+    for (int i = t; i < g.zero_count; i += 256) g.zero_words[i] = 0;
   double acc[2][4][2];
 #pragma unroll
   for (int h = 0; h < 2; ++h)
 #pragma unroll
     for (int c = 0; c < 4; ++c) { acc[h][c][0] = 0.0; acc[h][c][1] = 0.0; }
-  // staging: row lr of the chunk, columns lc, lc + 16, lc + 32, lc + 48: the 16 threads of a row write
-  // 16 consecutive doubles per store (one shared-memory wavefront per row; four columns per thread
-  // side by side made every store an eight-way bank conflict)
-  const int lr = t >> 4, lc = t & 15;
-  // two chunks of 16 rows are on their way in registers while a third is multiplied (one was not
-  // enough to cover the loads' latency: the long slices of a wide panel took 2 us per chunk)
-  float ra[2][4], rb[2][4];
-  auto fetch = [&](long long k0, float (&fa)[4], float (&fb)[4]) {
-    const long long row = k0 + lr;
-    const bool in_k = row < r1;
+  // a thread copies column t % 64 of four rows of A's chunk and of B's (past the slice, or the matrix: zeros)
+  const int lr = t >> 6, lc = t & 63;
+  const bool in_a = m0 + lc < g.m, in_b = n0 + lc < g.n;
+  const float* pa = g.A + static_cast<long long>(r0 + lr) * g.lda + (in_a ? m0 + lc : 0);
+  const float* pb = g.B + static_cast<long long>(r0 + lr) * g.ldb + (in_b ? n0 + lc : 0);
+  const uint32_t to = static_cast<uint32_t>(__cvta_generic_to_shared(raw)) + (lr * AT_P + lc) * 4;
+  int next = r0 + lr;                                       // this thread's next row
+  auto fetch = [&](int stage) {
+    const uint32_t dst = to + stage * (2 * AT_K * AT_P * 4);
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int ca = m0 + lc + 16 * e, cb = n0 + lc + 16 * e;
-      fa[e] = (in_k && ca < g.m && PRAC_IN(row * g.lda + ca, (g.d - 1) * g.lda + g.m)) ? g.A[row * g.lda + ca] : 0.f;
-      fb[e] = (in_k && cb < g.n && PRAC_IN(row * g.ldb + cb, (g.d - 1) * g.ldb + g.n)) ? g.B[row * g.ldb + cb] : 0.f;
+    for (int e = 0; e < AT_K / 4; ++e) {
+      const bool in = next < r1;
+      const bool ok_a = in && in_a && PRAC_IN(pa - g.A, (g.d - 1) * g.lda + g.m), ok_b = in && in_b && PRAC_IN(pb - g.B, (g.d - 1) * g.ldb + g.n);
+      const float* const sa = ok_a ? pa : g.A;
+      const float* const sb = ok_b ? pb : g.B;
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + e * (4 * AT_P * 4)), "l"(sa), "r"(ok_a ? 4 : 0) : "memory");
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + (AT_K + 4 * e) * (AT_P * 4)), "l"(sb), "r"(ok_b ? 4 : 0) : "memory");
+      pa += 4 * g.lda; pb += 4 * g.ldb; next += 4;
     }
+    asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  fetch(r0, ra[0], rb[0]);
-  fetch(r0 + AT_K, ra[1], rb[1]);
-  int cur = 0;
-  for (long long k0 = r0; k0 < r1; k0 += AT_K, cur ^= 1) {
-    // (cur is 0, 1, 0, ...: both branches below are the same code on the two register sets)
-    if (cur == 0) {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        As[lr][lc + 16 * e] = static_cast<double>(ra[0][e]);
-        Bs[lr][lc + 16 * e] = static_cast<double>(rb[0][e]);
-      }
-    } else {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        As[lr][lc + 16 * e] = static_cast<double>(ra[1][e]);
-        Bs[lr][lc + 16 * e] = static_cast<double>(rb[1][e]);
-      }
-    }
-    __syncthreads();
-    if (cur == 0) fetch(k0 + 2 * AT_K, ra[0], rb[0]);
-    else fetch(k0 + 2 * AT_K, ra[1], rb[1]);
-#pragma unroll
+#pragma unroll 1
+  for (int s = 0; s < AT_STAGES - 1; ++s) fetch(s);
+  int stage = 0;
+#pragma unroll 1
+  for (int k0 = r0; k0 < r1; k0 += AT_K) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(AT_STAGES - 2) : "memory");
+    __syncthreads();                 // everybody's part of this chunk is there, and the chunk before it has been read
+    fetch((stage + AT_STAGES - 1) % AT_STAGES);
+    const float* const As = raw + stage * (2 * AT_K * AT_P) + q4 * AT_P + gq;
+#pragma unroll 2
     for (int kk = 0; kk < AT_K / 4; ++kk) {
-      const double a0 = As[kk * 4 + q4][wa + gq], a1 = As[kk * 4 + q4][wa + 8 + gq];
+      const float* const a = As + kk * 4 * AT_P + wa;
+      const float* const b = As + (AT_K + kk * 4) * AT_P + wb;
+      const double a0 = a[0], a1 = a[8];
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        const double bv = Bs[kk * 4 + q4][wb + c * 8 + gq];
+        const double bv = b[c * 8];
         dmma_884(acc[0][c], a0, bv);
         dmma_884(acc[1][c], a1, bv);
       }
     }
-    __syncthreads();
+    stage = (stage + 1) % AT_STAGES;
   }
-  double* out = g.partial + static_cast<long long>(split) * g.m * g.n;
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int gi = m0 + wa + h * 8 + gq;
-    if (gi >= g.m) continue;
+  for (int h = 0; h < 2; ++h)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const int gj = n0 + wb + c * 8 + 2 * q4 + i;
-        if (gj < g.n && PRAC_IN(static_cast<long long>(gi) * g.n + gj, static_cast<long long>(g.m) * g.n))
-          out[static_cast<long long>(gi) * g.n + gj] = acc[h][c][i];
-      }
+    for (int c = 0; c < 4; ++c)
+      *reinterpret_cast<double2*>(&tile[(wa + h * 8 + gq) * AT_P + wb + c * 8 + 2 * q4]) = make_double2(acc[h][c][0], acc[h][c][1]);
+  cluster_arrive();
+  cluster_wait();
+  // rows [64 rank / slices, 64 (rank + 1) / slices) of the tile
+  const int rows = AT_T / slices;
+#pragma unroll 1
+  for (int idx = t; idx < rows * AT_T; idx += 256) {
+    const int r = rows * rank + idx / AT_T, c = idx % AT_T;
+    const int i = m0 + r, j = n0 + c;
+    double v = 0.0;
+#pragma unroll 4
+    for (int s = 0; s < slices; ++s) v += cluster_ld1(cluster_addr(&tile[r * AT_P + c], s));
+    v *= g.alpha;
+    if (i >= g.m || j >= g.n || (g.symmetric && i > j)) continue;
+    const int copies = g.symmetric && i != j ? 2 : 1;
+#pragma unroll 1
+    for (int e = 0; e < copies; ++e) {
+      const long long o = e ? static_cast<long long>(j) * g.ldo + i : static_cast<long long>(i) * g.ldo + j;
+      if (!PRAC_IN(o, static_cast<long long>(g.m - 1) * g.ldo + g.n)) continue;
+      if (g.out_double) static_cast<double*>(g.out)[o] = v;
+      else static_cast<float*>(g.out)[o] = static_cast<float>(v);
     }
   }
-}
-
-// out[i][j] = alpha * sum_s partial[s][i][j], slices added in order.  symmetric: entries
-// below the diagonal are read from their mirror image (tiles below the diagonal were
-// not computed).  TOut = float or double.
-template <typename TOut>
-__global__ void reduce_partials_kernel(const double* partial, int splits, int m, int n,
-                                       int symmetric, double alpha, TOut* __restrict__ out, long long ldo,
-                                       const int* run_if, int run_if_mask, int* zero_words, int zero_count) {
-  grid_dep_wait();
-  if (pass_is_off(run_if, run_if_mask)) return;
-  // state that the next kernel on the stream expects zeroed (its grid-barrier counter)
-  if (blockIdx.x == 0 && static_cast<int>(threadIdx.x) < zero_count) zero_words[threadIdx.x] = 0;
-  const long long idx = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
-  if (idx >= static_cast<long long>(m) * n) return;
-  const int i = static_cast<int>(idx / n), j = static_cast<int>(idx % n);
-  const long long src = (symmetric && i > j) ? static_cast<long long>(j) * n + i : static_cast<long long>(i) * n + j;
-  // (eight loads in flight at a time: with many slices and few entries, as for the Rayleigh-Ritz
-  // matrix, the kernel is a chain of loads otherwise; the slices are still added one by one, in order)
-  const long long mn = static_cast<long long>(m) * n;
-  double s = 0.0;
-  int sp = 0;
-  for (; sp + 8 <= splits; sp += 8) {
-    double v[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = partial[(sp + e) * mn + src];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) s += v[e];
-  }
-  for (; sp < splits; ++sp) s += partial[sp * mn + src];
-  if (PRAC_IN(static_cast<long long>(i) * ldo + j, static_cast<long long>(m - 1) * ldo + n))
-    out[static_cast<long long>(i) * ldo + j] = static_cast<TOut>(alpha * s);
+  cluster_arrive();                  // (nobody's tile goes away under a reader)
+  cluster_wait();
 }
 
 // ------------------------------------------------------------------ Cholesky + inverse, one launch
@@ -268,84 +327,6 @@ __device__ __forceinline__ void blk_store(const double (*S)[CP], double* M, int 
   }
 }
 
-// The 8 x 8 diagonal sub-block of a diagonal block, by one warp in registers: lane (r, c) holds
-// M[r][2c], M[r][2c + 1] (the accumulator layout of dmma_884).  Elimination without square roots and
-// without a division: on return row r of the triangular matrix T = S L^-1, M = L diag(pv) L^T, S a diagonal
-// matrix of positive scales, is in the strictly lower part of M and S_r in `scale`; `pivot` is S_r pv_r, so that
-// M = T^-1 diag(pivot * scale) T^-T.  (An identity kept in the lower triangle is eliminated along
-// with M.)  Only the upper triangle is read.  A pivot that is not safely positive relative to the column's
-// original squared norm is replaced by a guard value.
-//
-// This is the careful form, one column at a time with S = 1, for sub-blocks in which a pivot is bad.
-__device__ __noinline__ void sub_chol_guarded(double& m0, double& m1, const double* guard, double& scale, double& pivot,
-                                              int* dev_status, int flag_bit) {
-  const int lane = threadIdx.x & 31, r = lane >> 2, c = lane & 3;
-  scale = 1.0;
-#pragma unroll 1
-  for (int j = 0; j < 8; ++j) {
-    const int row = j << 2;
-    double pv = __shfl_sync(0xffffffffu, (j & 1) ? m1 : m0, row | (j >> 1));
-    const double rj0 = __shfl_sync(0xffffffffu, m0, row | c), rj1 = __shfl_sync(0xffffffffu, m1, row | c);
-    const double t0 = __shfl_sync(0xffffffffu, m0, row | (r >> 1)), t1 = __shfl_sync(0xffffffffu, m1, row | (r >> 1));
-    if (!(pv > guard[j])) {                                      // warp-uniform
-      pv = guard[j];
-      if (lane == 0 && flag_bit && dev_status) atomicOr(dev_status, flag_bit);
-    }
-    if (r == j) pivot = pv;
-    const double m = ((r & 1) ? t1 : t0) / pv;                   // M[j][r] / pv
-    const double u0 = fma(-m, rj0, m0), u1 = fma(-m, rj1, m1);
-    // U part, and L^-1 columns before j: updated; L^-1 column j starts here; the rest waits
-    const int l0 = 2 * c, l1 = 2 * c + 1;
-    const double n0 = (l0 >= r || l0 < j) ? u0 : ((l0 == j) ? -m : m0);
-    const double n1 = (l1 >= r || l1 < j) ? u1 : ((l1 == j) ? -m : m1);
-    m0 = r > j ? n0 : m0;
-    m1 = r > j ? n1 : m1;
-  }
-}
-
-// The same with neither a division nor a test in the dependent chain.  Column j turns every later row r into
-// (pv_j M[r] - M[j][r] M[j]) 2^-e, e the exponent of the new scale: rows keep a common scale S in [1, 2) instead
-// of being divided by the pivot, and a column is a shuffle and three operations (with a reciprocal
-// approximation and its refinement in the chain it took 165 cycles).  Returns whether all pivots were good; where
-// not, the caller repeats the sub-block in the careful form.
-__device__ __forceinline__ bool sub_chol(double& m0, double& m1, const double* guard, double& scale, double& pivot) {
-  const int lane = threadIdx.x & 31, r = lane >> 2, c = lane & 3;
-  const int l0 = 2 * c, l1 = 2 * c + 1;
-  bool good = true;
-  double S = 1.0;
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const int row = j << 2;
-    const double pv = __shfl_sync(0xffffffffu, (j & 1) ? m1 : m0, row | (j >> 1));
-    good = good && pv > guard[j] * S;                            // (false for NaN)
-    if (r == j) { scale = S; pivot = pv; }
-    if (j == 7) break;
-    const double rj0 = __shfl_sync(0xffffffffu, m0, row | c), rj1 = __shfl_sync(0xffffffffu, m1, row | c);
-    const double t0 = __shfl_sync(0xffffffffu, m0, row | (r >> 1)), t1 = __shfl_sync(0xffffffffu, m1, row | (r >> 1));
-    const double t = (r & 1) ? t1 : t0;                          // M[j][r]
-    const double Sp = S * pv;
-    // 2^-e with e the exponent of Sp (a good pivot is a positive normal number)
-    const double two = __hiloint2double(0x7fe00000 - (__double2hiint(Sp) & 0x7ff00000), 0);
-    const double u0 = fma(pv, m0, -(t * rj0)) * two, u1 = fma(pv, m1, -(t * rj1)) * two;
-    const double start = -(t * S) * two;                         // column j of T begins (its diagonal entry is S)
-    S = Sp * two;
-    const double n0 = (l0 >= r || l0 < j) ? u0 : ((l0 == j) ? start : m0);
-    const double n1 = (l1 >= r || l1 < j) ? u1 : ((l1 == j) ? start : m1);
-    m0 = r > j ? n0 : m0;
-    m1 = r > j ? n1 : m1;
-  }
-  return good;
-}
-
-// 1 / x for a positive normal x: 1 / x = x0 (1 + e + e^2 + ..), e = 1 - x x0; the hardware's x0 is good to 20 bits, so the
-// terms up to e^2 leave a relative error below 2^-60.
-__device__ __forceinline__ double rcp_f64(double x) {
-  double x0;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x0) : "d"(x));
-  const double e = fma(-x, x0, 1.0);
-  return fma(x0, fma(e, e, e), x0);
-}
-
 // The 256 threads that compute (the chain's CTA has more, see chol_inv_kernel).
 constexpr int CHOL_MAIN = 256, CHOL_HELP = 256;
 // (a warp has to be converged at these barriers)
@@ -359,124 +340,155 @@ __device__ __forceinline__ void bar_arrive(int id, int threads) {
 }
 __device__ __forceinline__ void main_sync() { bar_sync(1, CHOL_MAIN); }
 
-// What a diagonal block's factorisation leaves in shared memory beside the block: limits below which a pivot is
-// replaced, scaled pivots, their inverse square roots.
-struct CholDiag { double guard[CB], pi[CB], rs[CB]; };
 __device__ __forceinline__ double pivot_guard(double diagonal_on_entry) {
   return diagonal_on_entry > 0.0 ? 1e-13 * diagonal_on_entry : 1.0;
 }
 
-// In shared memory: D (CB x CB, symmetric positive definite on entry, upper triangle used) -> I = R^-1
-// (upper), where R^T R = D, by the 256 main threads, which have met at a barrier since D and x.guard were written.  The
-// chain of 32 dependent column steps is what this costs, so
-// it runs in one warp's registers, eight columns at a time (one block barrier per column over all
-// 256 threads took 330 cycles each); the other 8 x 8 tiles are brought up to date on the fp64 tensor
-// cores by the other warps, one tile each, beside the next sub-block's chain.  With T = S L_ss^-1 of sub-block s (sub_chol),
-// pi = pivot * scale, U_q = T D_sq, V_q = diag(1/pi) U_q:
-// D_pq -= V_p^T U_q, and the same elimination applied to an identity (E) gives the block rows of S L^-1:
-// Lin_sc = T E_sc (E_ss = 1), E_pc -= V_p^T Lin_sc.  R^-1 = (S L^-1)^T diag(1/sqrt(pi)).
-// W: scratch, rows 0..7 U, 8..15 V (columns 8 q ..), 16..23 T, two in turn.  emit(r, c, v0, v1): elements (r, c), (r, c + 1) of
-// R^-1, which are written to I too.
-template <typename Emit>
-__device__ __forceinline__ void blk_chol_inv(double (*D)[CP], double (*I)[CP], double (*Lin)[CP], double (*E)[CP], double (*W)[CP],
-                                             CholDiag& x, int* dev_status, int flag_bit, Emit emit) {
+// Where a diagonal block is factored, all in shared memory.  D: the block (upper triangle); guard: limits below which a
+// pivot is replaced.  Lin: the block rows of R^-T, D = R^T R (zero right of the diagonal tiles on entry).  E: the
+// identity under the same elimination.  W: eight rows of R at a time, rows 0..7 and 8..15 in turn.
+struct CholBlock { double (*D)[CP]; double (*Lin)[CP]; double (*E)[CP]; double (*W)[CP]; const double* guard; };
+
+// The column of a sub-block's row that a lane carries through the elimination: tile `lane / 8` of four (the
+// identity, the tiles of D right of the diagonal, those of E left of it), column lane % 8.
+struct CholLane { int column; bool unit, of_d; };
+__device__ __forceinline__ CholLane chol_lane(int s) {
+  const int lane = threadIdx.x & 31, i = lane >> 3;
+  CholLane l;
+  l.unit = i == 0;
+  l.of_d = i > 0 && s + i < CB / 8;
+  l.column = 8 * (l.unit ? s : (l.of_d ? s + i : s + i - CB / 8)) + (lane & 7);
+  return l;
+}
+__device__ __forceinline__ double chol_lane_load(const CholBlock& b, const CholLane& l, int s, int k) {
+  if (l.unit) return (threadIdx.x & 7) == k ? 1.0 : 0.0;
+  return (l.of_d ? b.D : b.E)[8 * s + k][l.column];
+}
+__device__ __forceinline__ double* chol_lane_out(const CholBlock& b, const CholLane& l, int s) {
+  return l.of_d ? &b.W[8 * (s & 1)][l.column] : &b.Lin[8 * s][l.column];
+}
+
+// Sub-block s in the careful form, for one in which a pivot is not safely positive relative to the
+// column's original squared norm: such a pivot is replaced by a guard value (and reported).  One warp; the
+// diagonal tile is overwritten.
+__device__ __noinline__ void sub_chol_guarded(const CholBlock b, int s, int* dev_status, int flag_bit) {
+  const int lane = threadIdx.x & 31, o = 8 * s;
+  const CholLane l = chol_lane(s);
+  double* const out = chol_lane_out(b, l, s);
+  double rhs[8];
+  for (int k = 0; k < 8; ++k) rhs[k] = chol_lane_load(b, l, s, k);
+  for (int j = 0; j < 8; ++j) {
+    __syncwarp();
+    double pv = b.D[o + j][o + j];
+    if (!(pv > b.guard[o + j])) {
+      pv = b.guard[o + j];
+      if (lane == 0 && flag_bit && dev_status) atomicOr(dev_status, flag_bit);
+    }
+    for (int r = j + 1; r < 8; ++r) rhs[r] = fma(-(b.D[o + j][o + r] / pv), rhs[j], rhs[r]);
+    for (int i = lane; i < 64; i += 32) {
+      const int r = i >> 3, c = i & 7;
+      if (r > j && c >= r) b.D[o + r][o + c] = fma(-(b.D[o + j][o + r] / pv), b.D[o + j][o + c], b.D[o + r][o + c]);
+    }
+    out[j * CP] = rhs[j] * rsqrt(pv);
+  }
+}
+
+// The same without the tests.  Every lane eliminates the 8 x 8 tile in its own registers (no exchange between the
+// dependent steps: pivot, reciprocal, multiplier, next pivot; with the tile spread over the lanes and rows
+// passed by shuffles a column took 165 cycles, here 115 with its loads and stores) and takes its own column along, so that the
+// whole block row s of R and of R^-T comes out with it.  The reciprocal and the square root refine the
+// hardware's approximations x0, y0 of 20 bits: 1 / x = x0 (1 + e + e^2 + ..), e = 1 - x x0, and x^-1/2 = y0 (1 + e / 2 +
+// 3 e^2 / 8 + ..), e = 1 - x y0^2, with a relative error below 2^-58.  Returns whether all pivots were good.
+__device__ __forceinline__ bool sub_chol(const CholBlock& b, int s) {
+  const int o = 8 * s;
+  const CholLane l = chol_lane(s);
+  double* const out = chol_lane_out(b, l, s);
+  double m[8][8], rhs[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+#pragma unroll
+    for (int j = i & ~1; j < 8; j += 2) {
+      const double2 v = *reinterpret_cast<const double2*>(&b.D[o + i][o + j]);
+      if (j >= i) m[i][j] = v.x;
+      m[i][j + 1] = v.y;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 8; ++k) rhs[k] = chol_lane_load(b, l, s, k);
+  bool good = true;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const double pv = m[j][j];
+    double x0, y0;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x0) : "d"(pv));
+    const double e = fma(-pv, x0, 1.0), corr = fma(e, e, e);
+#pragma unroll
+    for (int r = j + 1; r < 8; ++r) {
+      const double q = m[j][r] * x0, f = fma(q, corr, q);         // m[j][r] / pivot
+#pragma unroll
+      for (int c = r; c < 8; ++c) m[r][c] = fma(-f, m[j][c], m[r][c]);
+      rhs[r] = fma(-f, rhs[j], rhs[r]);
+    }
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(pv));
+    const double h = fma(-(pv * y0), y0, 1.0);
+    out[j * CP] = rhs[j] * fma(y0, h * fma(0.375, h, 0.5), y0);
+    good = good && pv > b.guard[o + j];                           // (false for NaN)
+  }
+  return good;
+}
+
+// C (8 x 8 tile) = [C] - R_p^T B_q, the k = 8 rows of a sub-block.
+__device__ __forceinline__ void sub_update(double (*C)[CP], int p, int q, const double (*R)[CP], const double (*B)[CP], bool fresh) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, q4 = lane & 3;
+  double2* const o = reinterpret_cast<double2*>(&C[8 * p + g][8 * q + 2 * q4]);
+  const double2 old = *o;
+  double a0[2] = {0.0, 0.0}, a1[2] = {0.0, 0.0};
+  dmma_884(a0, R[q4][8 * p + g], B[q4][8 * q + g]);
+  dmma_884(a1, R[4 + q4][8 * p + g], B[4 + q4][8 * q + g]);
+  *o = make_double2((fresh ? 0.0 : old.x) - (a0[0] + a1[0]), (fresh ? 0.0 : old.y) - (a0[1] + a1[1]));
+}
+
+// D (CB x CB, symmetric positive definite on entry, upper triangle used) -> Lin = R^-T (lower), where R^T R = D, by
+// the 256 main threads, which have met at a barrier since D and the limits were written.  The
+// chain of 32 dependent column steps is what this costs, so one warp walks it, eight columns at a time, each lane on
+// its own (sub_chol); the other warps bring the 8 x 8 tiles below up to date on the fp64 tensor cores, those of the
+// next row first.  With R_s the eight rows of R from sub-block s: D_pq -= R_sp^T R_sq, and the same elimination applied
+// to an identity (E) gives the block rows of R^-T: E_pc -= R_sp^T Lin_sc.
+// rows_done(s): rows 8 s .. 8 s + 7 of Lin, final, are visible to warps 4..7, which call it (after the last, warps 0..3).
+template <typename RowsDone>
+__device__ __forceinline__ void blk_chol_inv(const CholBlock& b, int* dev_status, int flag_bit, RowsDone rows_done) {
   static_assert(CB == 32, "four sub-blocks of eight columns");
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31, g = lane >> 2, q4 = lane & 3;
-  double (*U)[CP] = W; double (*V)[CP] = W + 8; double (*T)[CP] = W + 16;
-  double m0 = 0.0, m1 = 0.0;
-  if (warp == 0) { m0 = D[g][2 * q4]; m1 = D[g][2 * q4 + 1]; }
+  const int warp = threadIdx.x >> 5;
 #pragma unroll 1
   for (int s = 0; s < CB / 8; ++s) {
-    const int o = 8 * s;
-    const int tc = 8 * (s & 1);                    // T of this sub-block: W[16 ..][tc ..]
-    double t0 = 0.0, t1 = 0.0, pi = 1.0;
-    if (warp == 0) {
-      const double k0 = m0, k1 = m1;
-      double scale = 1.0, pivot = 1.0;
-      if (!sub_chol(m0, m1, x.guard + o, scale, pivot)) {     // (the lanes agree)
-        m0 = k0; m1 = k1;
-        sub_chol_guarded(m0, m1, x.guard + o, scale, pivot, dev_status, flag_bit);
-      }
-      t0 = 2 * q4 < g ? m0 : (2 * q4 == g ? scale : 0.0);
-      t1 = 2 * q4 + 1 < g ? m1 : (2 * q4 + 1 == g ? scale : 0.0);
-      pi = pivot * scale;
-      T[g][tc + 2 * q4] = t0; T[g][tc + 2 * q4 + 1] = t1;
-      Lin[o + g][o + 2 * q4] = t0; Lin[o + g][o + 2 * q4 + 1] = t1;
-      if (q4 == 0) x.pi[o + g] = pi;
-    }
+    double (*R)[CP] = b.W + 8 * (s & 1);
+    const double (*L)[CP] = b.Lin + 8 * s;
+    if (warp == 0 && !sub_chol(b, s)) sub_chol_guarded(b, s, dev_status, flag_bit);     // (the lanes agree)
     main_sync();
-    if (warp == 0) {
-      // the next diagonal sub-block, on its own and in registers (the others make U and V of block column s + 1
-      // again): a fragment of A may name its columns in any order that B's rows follow, so T goes in as it lies;
-      // U comes back with its rows over the lanes and is turned by shuffles
-      if (s + 1 < CB / 8) {
-        const int p = o + 8;
-        double acc[2] = {0.0, 0.0};
-        dmma_884(acc, t0, D[o + 2 * q4][p + g]);
-        dmma_884(acc, t1, D[o + 2 * q4 + 1][p + g]);
-        const double xi = rcp_f64(pi);
-        double upd[2] = {0.0, 0.0};
-#pragma unroll
-        for (int kk = 0; kk < 2; ++kk) {
-          const int from = ((4 * kk + q4) << 2) | (g >> 1);
-          const double u0 = __shfl_sync(0xffffffffu, acc[0], from), u1 = __shfl_sync(0xffffffffu, acc[1], from);
-          const double u = (g & 1) ? u1 : u0;      // U[4 kk + q4][g]
-          dmma_884(upd, u * __shfl_sync(0xffffffffu, xi, (4 * kk + q4) << 2), u);
-        }
-        m0 = D[p + g][p + 2 * q4] - upd[0];
-        m1 = D[p + g][p + 2 * q4 + 1] - upd[1];
-      }
+    if (s + 1 == CB / 8) break;
+    // row s + 1, the four tiles that the next sub-block starts from: its part of D (warp 0 the diagonal tile) and of E
+    if (warp < 4) {
+      const int q = s + 1 + warp;
+      const bool of_d = q < CB / 8;
+      sub_update(of_d ? b.D : b.E, s + 1, of_d ? q : q - CB / 8, R, of_d ? R : L, q - CB / 8 == s);   // (E_ps starts from zero)
+      bar_sync(8, 128);
     } else {
-      if (warp == 7 && lane < 8) x.rs[o + lane] = rsqrt(x.pi[o + lane]);
-      // three tiles: U_q, q > s, and Lin_sc, c < s
-      if (warp < 4) {
-        const int q = warp - 1 < s ? warp - 1 : warp;
-        double (*B)[CP] = q < s ? E : D;
-        double acc[2] = {0.0, 0.0};
-#pragma unroll
-        for (int kk = 0; kk < 2; ++kk) dmma_884(acc, T[g][tc + 4 * kk + q4], B[o + 4 * kk + q4][8 * q + g]);
-        if (q < s) {
-          Lin[o + g][8 * q + 2 * q4] = acc[0]; Lin[o + g][8 * q + 2 * q4 + 1] = acc[1];
-        } else {
-          const double xi = rcp_f64(x.pi[o + g]);
-          U[g][8 * q + 2 * q4] = acc[0]; U[g][8 * q + 2 * q4 + 1] = acc[1];
-          V[g][8 * q + 2 * q4] = xi * acc[0]; V[g][8 * q + 2 * q4 + 1] = xi * acc[1];
-        }
-      }
-      bar_sync(8, CHOL_MAIN - 32);
-      // trailing tiles D_pq (s < p <= q, without the one warp 0 has) and E_pc (c <= s < p), in one list
-      const int rest = CB / 8 - 1 - s, nd = rest * (rest + 1) / 2 - 1, ne = rest * (s + 1);
-      for (int u = warp - 1; u < nd + ne; u += 7) {
-        double acc[2] = {0.0, 0.0};
-        int p, q;
-        if (u < nd) {                              // tile u + 1 of the upper triangle, by rows (tile 0 is warp 0's)
-          int left = u + 1;
-          p = s + 1;
+      rows_done(s);
+      // the rows below, beside the next sub-block's chain
+      const int rest = CB / 8 - 2 - s, nd = rest * (rest + 1) / 2, ne = rest * (s + 1);
+      for (int u = warp - 4; u < nd + ne; u += 4) {
+        if (u < nd) {
+          int p = s + 2, left = u;
           while (left >= CB / 8 - p) { left -= CB / 8 - p; ++p; }
-          q = p + left;
+          sub_update(b.D, p, p + left, R, R, false);
         } else {
-          p = s + 1 + (u - nd) / (s + 1);
-          q = (u - nd) % (s + 1);
+          const int c = (u - nd) % (s + 1);
+          sub_update(b.E, s + 2 + (u - nd) / (s + 1), c, R, L, c == s);
         }
-        double (*B)[CP] = u < nd ? U : Lin + o;
-        double (*C)[CP] = u < nd ? D : E;
-#pragma unroll
-        for (int kk = 0; kk < 2; ++kk) dmma_884(acc, V[4 * kk + q4][8 * p + g], B[4 * kk + q4][8 * q + g]);
-        double* o0 = &C[8 * p + g][8 * q + 2 * q4];
-        const bool fresh = u >= nd && q == s;      // (E_ps starts from zero)
-        o0[0] = (fresh ? 0.0 : o0[0]) - acc[0];
-        o0[1] = (fresh ? 0.0 : o0[1]) - acc[1];
       }
     }
   }
-  main_sync();
-#pragma unroll
-  for (int e = 0; e < CB * CB / 2 / CHOL_MAIN; ++e) {
-    const int r = (t + CHOL_MAIN * e) / (CB / 2), c = 2 * (t % (CB / 2));
-    const double v0 = r <= c ? Lin[c][r] * x.rs[c] : 0.0, v1 = r <= c + 1 ? Lin[c + 1][r] * x.rs[c + 1] : 0.0;
-    *reinterpret_cast<double2*>(&I[r][c]) = make_double2(v0, v1);
-    emit(r, c, v0, v1);
-  }
+  if (warp < 4) rows_done(CB / 8 - 1);
 }
 
 // Up to three blocks fetched in one round trip: all of a thread's loads are issued before the first store.
@@ -500,16 +512,16 @@ __device__ __forceinline__ void blk_load3(double (*A)[CP], const double* MA, int
 }
 
 // Block (p, q), p <= q, of the result R^-1, from shared memory into the outputs (see CholArgs): the fp32
-// matrix, or the transposed matrix as three bf16 pieces.
-__device__ __forceinline__ void chol_emit(const CholArgs& a, const double (*S)[CP], int p, int q) {
+// matrix, or the transposed matrix as three bf16 pieces.  transposed: S holds the block's transpose.
+__device__ __forceinline__ void chol_emit(const CholArgs& a, const double (*S)[CP], int p, int q, bool transposed = false) {
   for (int idx = group_tid(); idx < CB * CB; idx += 256) {
     if (!a.Rt3) {
       const int i = p * CB + idx / CB, j = q * CB + idx % CB;
-      if (i < a.n && j < a.n) a.Rinv[static_cast<long long>(i) * a.ldr + j] = static_cast<float>(S[idx / CB][idx % CB]);
+      if (i < a.n && j < a.n) a.Rinv[static_cast<long long>(i) * a.ldr + j] = static_cast<float>(transposed ? S[idx % CB][idx / CB] : S[idx / CB][idx % CB]);
     } else {
       const int j = q * CB + idx / CB, l = p * CB + idx % CB;
       if (j < a.n && l < a.kp) {
-        float x = l < a.n ? static_cast<float>(S[idx % CB][idx / CB]) : 0.f;
+        float x = l < a.n ? static_cast<float>(transposed ? S[idx / CB][idx % CB] : S[idx % CB][idx / CB]) : 0.f;
         __nv_bfloat16* o = a.Rt3 + static_cast<long long>(j) * 3 * a.kp + l;
         const __nv_bfloat16 hi = __float2bfloat16_rn(x);
         x -= __bfloat162float(hi);
@@ -566,7 +578,7 @@ __global__ void __launch_bounds__(CHOL_MAIN + CHOL_HELP) chol_inv_kernel(const C
   if (a.run_if_mask && pass_is_off(a.dev_status, a.run_if_mask)) return;
   extern __shared__ __align__(16) double chol_smem[];
   __shared__ int ok_sh[2];
-  __shared__ CholDiag diag;
+  __shared__ double guard[CB];
   double (*S0)[CP] = reinterpret_cast<double (*)[CP]>(chol_smem);
   double (*S1)[CP] = S0 + CB;
   double (*S2)[CP] = S1 + CB;
@@ -640,12 +652,15 @@ __global__ void __launch_bounds__(CHOL_MAIN + CHOL_HELP) chol_inv_kernel(const C
       if (j + 1 < nb) bar_arrive(4, CHOL_MAIN + CHOL_HELP);
       if (threadIdx.x < CB) {                      // (warp 0, which alone reads the limits)
         const int i = j * CB + threadIdx.x;
-        diag.guard[threadIdx.x] = pivot_guard(i < n ? a.diag0[i] : 1.0);
+        guard[threadIdx.x] = pivot_guard(i < n ? a.diag0[i] : 1.0);
         __syncwarp();
       }
       double* const inv = a.Dinv + static_cast<long long>(j) * CB * CB;
-      blk_chol_inv(D, S1, S2, S3, S5, diag, a.dev_status, a.flag_bit,
-                   [&](int r, int c, double v0, double v1) { *reinterpret_cast<double2*>(&inv[r * CB + c]) = make_double2(v0, v1); });
+      blk_chol_inv(CholBlock{D, S2, S3, S5, guard}, a.dev_status, a.flag_bit, [](int) {});
+      for (int idx = threadIdx.x; idx < CB * CB; idx += CHOL_MAIN) {
+        const int r = idx / CB, c = idx % CB;
+        inv[idx] = S1[r][c] = r <= c ? S2[c][r] : 0.0;
+      }
       main_sync();
       bar_arrive(2 + 4 * (j & 1), CHOL_MAIN + CHOL_HELP);
     }
@@ -745,65 +760,37 @@ __global__ void __launch_bounds__(CHOL_MAIN + CHOL_HELP) chol_inv_kernel(const C
 }
 
 // ------------------------------------------------------------------ the same on one cluster, up to 16 blocks of columns
-// Shared memory of another CTA of the cluster.
-__device__ __forceinline__ uint32_t cluster_addr(const void* own, unsigned rank) {
-  uint32_t r;
-  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(own))), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ double2 cluster_ld(uint32_t addr) {
-  double2 v;
-  asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(addr) : "memory");
-  return v;
-}
-__device__ __forceinline__ void cluster_st(uint32_t addr, double x, double y) {
-  asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(addr), "d"(x), "d"(y) : "memory");
-}
-__device__ __forceinline__ void cluster_st_flag(uint32_t addr, int v) {
-  asm volatile("st.release.cluster.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
-__device__ __forceinline__ int ld_flag(const int* own) {
-  int v;
-  asm volatile("ld.acquire.cluster.shared::cta.s32 %0, [%1];" : "=r"(v)
-               : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(own))) : "memory");
-  return v;
-}
-__device__ __forceinline__ void cluster_arrive() {
-  __syncwarp();
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait() {
-  __syncwarp();
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
 constexpr int CC_MAX = 16;                       // blocks of columns = CTAs of the cluster
 constexpr int CC_GROUPS = 2;                     // groups of 256 threads in a CTA
-// What the CTAs tell one another; every word is written by one CTA and only grows.
+// What the CTAs tell one another: barriers in the shared memory of the CTA that waits, each for one event.
 struct ChainWords {
-  int row_done[CC_MAX];      // [x]: blocks (c, x), c < row_done[x], of R are final in CTA x
-  int inv_done[CC_MAX];      // [x]: 8 when the inverse of diagonal block x is final in CTA x (x before this one: stored here by CTA x's eight warps)
-  int abort;                 // a wait gave up
+  uint64_t row[CC_MAX][CC_MAX];   // [c][x]: block (c, x) of R is final in CTA x
+  uint64_t diag[CC_MAX];          // [c]: R_cc^-T is final in CTA c
+  uint64_t band[CB / 8];          // rows 8 s .. 8 s + 7 of R_cc^-T from the CTA before this one have arrived here
+  int abort;                      // a wait gave up
 };
 
 // Column blocks of G and block rows of the inverse stay in shared memory for the whole factorisation: CTA q of
-// the cluster holds the blocks (p, q), p <= q, of G, which become those of R, and row q of X = R^-1.  Step c, once R_cc^-1
+// the cluster holds the blocks (p, q), p <= q, of G, which become those of R, and row q of X = R^-1 (its diagonal block
+// transposed).  Step c, once R_cc^-1
 // is known: the CTAs right of c form R_cq = R_cc^-T G_cq and subtract R_cp^T R_cq from their blocks (p, q), p > c; the others
 // close X_qc = X_qc R_cc^-1 and subtract X_qc R_cx from their running sums X_qx, x > c.  The blocks R_cx of another CTA are
-// fetched from its shared memory when its flag says that they are final; nothing is ever overwritten that another
-// CTA may still want.  CTA c + 1, whose diagonal block the chain waits for, has nothing else to do in step c: R_cc^-1 is
-// stored into its shared memory as it is formed, and two products later it factors.
+// fetched from its shared memory when it has said that they are final; nothing is ever overwritten that another
+// CTA may still want.  CTA c + 1, whose diagonal block the chain waits for, has nothing else to do in step c: the rows of
+// R_cc^-T are stored into its shared memory as they are formed, eight at a time, and its threads form the same rows of
+// R_c,c+1 and take their part off the diagonal block while the next eight are on their way.
 //
 // The chain of diagonal blocks is what this costs.  A factorisation whose CTAs met through flags in global memory
 // (chol_inv_kernel) took 13 400 cycles a block, most of them the way of a block through L2 and back.
 //
 // Every wait on another CTA is bounded; a CTA that gives up tells the others, and all of them meet at the
 // cluster's barrier before any leaves, so that nobody's shared memory goes away under a reader.
+//
+// A CTA walks most of this code once, with its instructions not in the SM's cache yet (see sub_chol).  So every CTA
+// first runs the chain's part of a step on an identity, before it waits for the kernel that makes G.
 __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const CholArgs a) {
-  grid_dep_wait();
-  if (a.run_if_mask && pass_is_off(a.dev_status, a.run_if_mask)) return;
   extern __shared__ __align__(16) double chol_smem[];
-  __shared__ CholDiag diag;
+  __shared__ double guard[CB];
   __shared__ ChainWords words;
   typedef double (*Blk)[CP];
   const int n = a.n, nb = a.nb, q = static_cast<int>(blockIdx.x);
@@ -812,38 +799,39 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
   auto block = [&](int i) { return reinterpret_cast<Blk>(chol_smem + static_cast<size_t>(i) * CB * CP); };
   auto col = [&](int p) { return block(p); };                 // (p, q) of G, then of R
   auto inv = [&](int x) { return block(x + 1); };             // (q, x) of R^-1, x >= q
-  Blk const Lin = block(nb + 1), E = block(nb + 2), W = block(nb + 3), Dprev = block(nb + 4), Dfar = block(nb + 5);
-  Blk const stage = block(nb + 6 + group);
+  Blk const W = block(nb + 1), Dprev = block(nb + 2), Dfar = block(nb + 3);
+  Blk const stage = block(nb + 4 + group);
+  Blk const E = block(nb + 4);                                // (group 0's: it factors or it fetches)
   bool fail = false;
 
-  if (tid < static_cast<int>(sizeof(words) / sizeof(int))) reinterpret_cast<int*>(&words)[tid] = 0;
-  __syncthreads();
-  cluster_arrive();
-  // this CTA's column of G, padded with the identity
-  for (int idx = tid; idx < (q + 1) * CB * CB; idx += 256 * CC_GROUPS) {
-    const int i = idx / CB, j = idx % CB;
-    col(i / CB)[i % CB][j] = ld_pad(a.G, n, i, q * CB + j);
-  }
-  for (int idx = tid; idx < (nb - 1 - q) * CB * CP; idx += 256 * CC_GROUPS)      // the running sums
-    inv(q + 1)[idx / CP][idx % CP] = 0.0;
-  if (group == 1) chol_emit_zeros(a, q, nb);
-  cluster_wait();
-  __syncthreads();
-  if (tid < CB) diag.guard[tid] = pivot_guard(col(q)[tid][tid]);
-  __syncthreads();
-
-  auto give_up = [&]() {
-    fail = true;
-    for (int x = 0; x < nb; ++x) cluster_st_flag(cluster_addr(&words.abort, x), 1);
+  // Every lane waits for a barrier of its own (or none): cheap polls, and one that acquires (it takes 400 cycles) once
+  // all of them are through.  Where a lane gives up the caller carries on with what it has, until the CTA next meets and leaves together.
+  auto wait_for = [&](uint64_t* bar) {
+    if (bar != nullptr && !fail) {
+      unsigned polls = 0;
+      while (!cluster_try_wait(bar)) {
+        if (++polls >= a.poll_limit) {
+          fail = true;
+          for (int x = 0; x < nb; ++x) cluster_st_flag(cluster_addr(&words.abort, x), 1);
+          break;
+        }
+        if ((polls & 63u) == 0u && *reinterpret_cast<volatile int*>(&words.abort)) { fail = true; break; }
+      }
+    }
+    __syncwarp();
+    if (bar != nullptr && !fail) (void)cluster_try_wait_acquire(bar);
+    __syncwarp();
   };
-  // One lane of a warp polls a word of this CTA's shared memory; where it gives up the caller carries on with what it
-  // has, until the CTA next meets and leaves together.
-  auto wait_word = [&](const int* word, int target) {
+  // (what arrives by cluster_st_async is visible to who has seen its barrier complete)
+  auto wait_rows = [&](uint64_t* bar) {
     if (lane == 0 && !fail) {
       unsigned polls = 0;
-      while (ld_flag(word) < target) {
-        if (++polls >= a.poll_limit) { give_up(); break; }
-        if ((polls & 63u) == 0u && ld_flag(&words.abort)) { fail = true; break; }
+      while (!cluster_try_wait_rows(bar)) {
+        if (++polls >= a.poll_limit || ((polls & 63u) == 0u && *reinterpret_cast<volatile int*>(&words.abort))) {
+          fail = true;
+          for (int x = 0; x < nb; ++x) cluster_st_flag(cluster_addr(&words.abort, x), 1);
+          break;
+        }
       }
     }
     __syncwarp();
@@ -859,111 +847,194 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
     for (int e = 0; e < 2; ++e) *reinterpret_cast<double2*>(&to[(gt + 256 * e) >> 4][2 * (gt & 15)]) = v[e];
   };
 
-  for (int c = 0; c < nb; ++c) {
-    if (c == q) {
-      if (group == 0) {
-        const bool next = q + 1 < nb;
-        const uint32_t far = next ? cluster_addr(Dprev, q + 1) : 0u;
-        blk_chol_inv(col(q), inv(q), Lin, E, W, diag, a.dev_status, a.flag_bit, [&](int r, int cc, double v0, double v1) {
-          if (next) cluster_st(far + (r * CP + cc) * 8, v0, v1);
-        });
-        // (each warp says that its part is there: inv_done counts them)
-        __syncwarp();
-        if (next && lane == 0) {
-          asm volatile("red.release.cluster.shared::cluster.add.u32 [%0], 1;" ::"r"(cluster_addr(&words.inv_done[q], q + 1)) : "memory");
+  // c = -2: the dry run (an optional pass, which is nearly always off, goes without, and so do one or
+  // two blocks, whose CTAs the product before does not keep waiting for long enough); c = -1: set-up, and CTA 0
+  // factors its block; then the steps
+  for (int c = a.run_if_mask || nb <= 2 ? -1 : -2; c < nb; ++c) {
+    const bool dry = c == -2;
+    if (c < 0) {
+      const int rows = dry ? 0 : n;              // (the dry run reads and writes no global memory)
+      if (!dry) {
+        grid_dep_wait();
+        if (a.run_if_mask && pass_is_off(a.dev_status, a.run_if_mask)) return;
+      }
+      if (!dry) {
+        if (tid < CC_MAX * CC_MAX) cluster_bar_init(&words.row[0][0] + tid, 0);
+        else if (tid < CC_MAX * CC_MAX + CC_MAX) cluster_bar_init(&words.diag[tid - CC_MAX * CC_MAX], 0);
+        else if (tid < CC_MAX * CC_MAX + CC_MAX + CB / 8) {
+          const int s = tid - CC_MAX * CC_MAX - CC_MAX;
+          cluster_bar_init(&words.band[s], q > 0 ? 8 * 8 * (s + 1) * 8 : 0);      // eight rows up to the diagonal tile, in bytes
+        }
+        if (tid == 511) words.abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      }
+      __syncthreads();
+      cluster_arrive();
+      // this CTA's column of G, padded with the identity
+      for (int i0 = tid / CB; i0 < (q + 1) * CB; i0 += 8 * (256 * CC_GROUPS / CB)) {       // (eight loads in flight)
+        double v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const int i = i0 + e * (256 * CC_GROUPS / CB), j = q * CB + tid % CB;
+          v[e] = i == j ? 1.0 : 0.0;
+          if (i < rows && j < rows) v[e] = __ldcg(&a.G[static_cast<long long>(i) * n + j]);
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const int i = i0 + e * (256 * CC_GROUPS / CB);
+          if (i < (q + 1) * CB) col(i / CB)[i % CB][tid % CB] = v[e];
+        }
+      }
+      for (int idx = tid; idx < (nb - q) * CB * CP; idx += 256 * CC_GROUPS)      // the running sums
+        inv(q)[0][idx] = 0.0;
+      if (group == 1 && !dry) chol_emit_zeros(a, q, nb);
+      cluster_wait();
+      __syncthreads();
+      if (tid < CB) guard[tid] = dry ? 1e-13 : pivot_guard(col(q)[tid][tid]);
+      if (dry) {
+        for (int idx = tid; idx < CB * CB; idx += 256 * CC_GROUPS) {
+          const int i = idx / CB, j = idx % CB;
+          Dprev[i][j] = block(nb + 4)[i][j] = i == j ? 1.0 : 0.0;
+          block(nb + 5)[i][j] = i == j ? 2.0 : 0.0;
         }
       }
       __syncthreads();
-      // the CTA after this one counts the eight warps above, the others wait for this word
-      if (warp == 8 && lane < nb && lane != q && lane != q + 1) cluster_st_flag(cluster_addr(&words.inv_done[q], lane), 8);
-    } else {
-      // ---- R_cc^-1, then this CTA's own block of step c
-      Blk D = Dfar;
-      wait_word(&words.inv_done[c], 8);
-      if (c == q - 1) {
-        D = Dprev;
-      } else {
-        const int r = tid >> 4, cc = 2 * (tid & 15);
-        const double2 v = cluster_ld(cluster_addr(&block(c + 1)[r][cc], c));
-        *reinterpret_cast<double2*>(&Dfar[r][cc]) = v;
-        __syncthreads();
-      }
-      const int r0 = (warp >> 2) * 8, c0 = (warp & 3) * 8;    // a tile per warp
-      double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-      Blk const mine = c < q ? col(c) : inv(c);
-      // (R_cc^-1 is upper triangular: the products end where it does)
-      const int ks_end = c < q ? 2 * (warp >> 2) + 2 : 2 * (warp & 3) + 2;
-#pragma unroll
-      for (int ks = 0; ks < CB / 4; ++ks) {
-        if (ks >= ks_end) break;
-        const double x = c < q ? D[ks * 4 + q4][r0 + g] : mine[r0 + g][ks * 4 + q4];
-        const double y = c < q ? mine[ks * 4 + q4][c0 + g] : D[ks * 4 + q4][c0 + g];
-        dmma_884(acc[ks & 1], x, y);
-      }
-      __syncthreads();
-      *reinterpret_cast<double2*>(&mine[r0 + g][c0 + 2 * q4]) = make_double2(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
     }
-    // every thread leaves here if one has given up
-    if (__syncthreads_or(fail)) { fail = true; break; }
 
-    if (c < q) {
-      if (warp == 15 && lane < nb && lane != q) cluster_st_flag(cluster_addr(&words.row_done[q], lane), c + 1);
-      Blk const R = col(c);
-      if (c == q - 1) {
-        // the diagonal block, at once: the upper 8 x 8 tiles, by the threads that factor it next
-        if (group == 0) {
-          for (int u = warp; u < 10; u += 8) {
-            int p = 0, left = u;
-            while (left >= 4 - p) { left -= 4 - p; ++p; }
-            const int r0 = 8 * p, c0 = 8 * (p + left);
-            double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-#pragma unroll
-            for (int ks = 0; ks < CB / 4; ++ks) dmma_884(acc[ks & 1], R[ks * 4 + q4][r0 + g], R[ks * 4 + q4][c0 + g]);
-            double2* o = reinterpret_cast<double2*>(&col(q)[r0 + g][c0 + 2 * q4]);
-            const double2 old = *o;
-            *o = make_double2(old.x - (acc[0][0] + acc[1][0]), old.y - (acc[0][1] + acc[1][1]));
+    if (dry || c == q - 1) {
+      // ---- the chain: block (c, q) of R and the diagonal block, by rows of R_cc^-T as they come; then the factorisation
+      Blk const Dq = dry ? block(nb + 5) : col(q), Rbuf = Dfar;
+      if (c == -1) {
+        // (CTA 0: nothing to take off)
+      } else if (group == 1) {
+        for (int s = (warp >> 2) & 1; s < CB / 8; s += 2) {
+          if (!dry) wait_rows(&words.band[s]);
+          Blk const mine = dry ? block(nb + 4) : col(c);
+          const int r0 = 8 * s, c0 = 8 * (warp & 3);
+          double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+#pragma unroll 2
+          for (int ks = 0; ks < 2 * s + 2; ks += 2) {
+            dmma_884(acc[0], Dprev[r0 + g][ks * 4 + q4], mine[ks * 4 + q4][c0 + g]);
+            dmma_884(acc[1], Dprev[r0 + g][ks * 4 + 4 + q4], mine[ks * 4 + 4 + q4][c0 + g]);
           }
-          main_sync();
+          *reinterpret_cast<double2*>(&Rbuf[r0 + g][c0 + 2 * q4]) = make_double2(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
+          bar_arrive(9 + s, 128 + 256);
         }
       } else {
-        // blocks (p, q), c < p <= q, dealt to the groups, (q, q) first: it needs nobody else's block
-        if (group == 0) blk_mm(col(q), R, R, 1);
-        double2 v[2];
-        int p = c + 1 + (1 - group);
-        if (p < q) { wait_word(&words.row_done[p], c + 1); pull(cluster_addr(R, p), v); }
-        for (; p < q; p += CC_GROUPS) {
-          bar_sync(1 + group, 256);            // the block before this one is done with
-          put(stage, v);
-          bar_sync(1 + group, 256);
-          if (p + CC_GROUPS < q) { wait_word(&words.row_done[p + CC_GROUPS], c + 1); pull(cluster_addr(R, p + CC_GROUPS), v); }
-          blk_mm(col(p), stage, R, 1);
+        // a tile of the upper triangle per warp, two for the last two
+        const int u0 = warp, u1 = warp >= 6 ? warp + 2 : -1;
+        auto tile = [](int u, int& p, int& x) {
+          p = 0;
+          while (u >= 4 - p) { u -= 4 - p; ++p; }
+          x = p + u;
+        };
+        int p0, x0, p1 = 0, x1 = 0;
+        tile(u0, p0, x0);
+        if (u1 >= 0) tile(u1, p1, x1);
+        double acc[2][2][2] = {};
+#pragma unroll 1
+        for (int s = 0; s < CB / 8; ++s) {
+          bar_sync(9 + s, 128 + 256);
+          const double (*R)[CP] = Rbuf + 8 * s;
+          dmma_884(acc[0][0], R[q4][8 * p0 + g], R[q4][8 * x0 + g]);
+          dmma_884(acc[0][1], R[4 + q4][8 * p0 + g], R[4 + q4][8 * x0 + g]);
+          if (u1 >= 0) {
+            dmma_884(acc[1][0], R[q4][8 * p1 + g], R[q4][8 * x1 + g]);
+            dmma_884(acc[1][1], R[4 + q4][8 * p1 + g], R[4 + q4][8 * x1 + g]);
+          }
         }
+        double2* o = reinterpret_cast<double2*>(&Dq[8 * p0 + g][8 * x0 + 2 * q4]);
+        double2 old = *o;
+        *o = make_double2(old.x - (acc[0][0][0] + acc[0][1][0]), old.y - (acc[0][0][1] + acc[0][1][1]));
+        if (u1 >= 0) {
+          o = reinterpret_cast<double2*>(&Dq[8 * p1 + g][8 * x1 + 2 * q4]);
+          old = *o;
+          *o = make_double2(old.x - (acc[1][0][0] + acc[1][1][0]), old.y - (acc[1][0][1] + acc[1][1][1]));
+        }
+        main_sync();
       }
-    } else {
-      // row q of the inverse: X_qx -= X_qc R_cx, x > c
-      Blk const X = inv(c);
+      if (group == 0) {
+        Blk const Lin = dry ? block(nb) : inv(q);
+        const bool next = !dry && q + 1 < nb;
+        const uint32_t far = next ? cluster_addr(Dprev, q + 1) : 0u, far_bar = next ? cluster_addr(words.band, q + 1) : 0u;
+        blk_chol_inv(CholBlock{Dq, Lin, E, W, guard}, dry ? nullptr : a.dev_status, a.flag_bit, [&](int s) {
+          const int i = tid & 127, r = 8 * s + (i & 7), cc = 2 * (i >> 3);
+          if (next && cc < 8 * (s + 1)) cluster_st_async(far + (r * CP + cc) * 8, *reinterpret_cast<const double2*>(&Lin[r][cc]), far_bar + 8 * s);
+        });
+      } else if (!dry && c >= 0) {
+        bar_sync(2, 256);                        // (Rbuf is complete)
+        double2 v[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) v[e] = *reinterpret_cast<const double2*>(&Rbuf[(gt + 256 * e) >> 4][2 * (gt & 15)]);
+        put(col(c), v);
+        bar_sync(2, 256);
+        if (warp == 15 && lane < nb && lane != q) cluster_bar_arrive(cluster_addr(&words.row[c][q], lane));
+      }
+      // every thread leaves here if one has given up
+      if (__syncthreads_or(fail)) { fail = true; break; }
+      if (!dry && warp == 8 && lane < nb && lane != q) cluster_bar_arrive(cluster_addr(&words.diag[q], lane));
+    }
+    if (dry || (c >= 0 && c != q - 1)) {
+      const bool left = c < q;
+      Blk const own = dry ? block(nb + 5) : (left ? col(c) : inv(c));
+      // ---- R_cc^-T, then this CTA's own block of step c
+      if (c != q) {
+        if (!dry) wait_for(lane == 0 ? &words.diag[c] : nullptr);
+        {
+          const int r = tid >> 4, cc = 2 * (tid & 15);
+          const double2 v = cluster_ld(cluster_addr(&(dry ? Dprev : block(c + 1))[r][cc], dry ? q : c));
+          *reinterpret_cast<double2*>(&Dfar[r][cc]) = v;
+        }
+        __syncthreads();
+        const int r0 = (warp >> 2) * 8, c0 = (warp & 3) * 8;    // a tile per warp
+        double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+        // (R_cc^-T is lower triangular: the products end where it does)
+        const int ks_end = left ? 2 * (warp >> 2) + 2 : 2 * (warp & 3) + 2;
+#pragma unroll 2
+        for (int ks = 0; ks < ks_end; ks += 2) {
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const int k = (ks + e) * 4 + q4;
+            dmma_884(acc[e], left ? Dfar[r0 + g][k] : own[r0 + g][k], left ? own[k][c0 + g] : Dfar[c0 + g][k]);
+          }
+        }
+        __syncthreads();
+        *reinterpret_cast<double2*>(&own[r0 + g][c0 + 2 * q4]) = make_double2(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
+        if (__syncthreads_or(fail)) { fail = true; break; }
+        if (!dry && left && warp == 15 && lane < nb && lane != q) cluster_bar_arrive(cluster_addr(&words.row[c][q], lane));
+      }
+      // ---- the blocks it brings up to date, dealt to the groups: (p, q), c < p <= q, of G, (q, q) first, which needs nobody
+      // else's block; or (q, x), x > c, of the inverse
+      if (left && !dry && group == 0) blk_mm(col(q), own, own, 1);
+      if (!left && group == 1) chol_emit(a, own, q, c, c == q);
+      const int first = dry ? 0 : c + 1 + (left ? 1 - group : group), end = dry ? 1 : (left ? q : nb);
+      Blk const from = dry ? Dprev : block(c);
       double2 v[2];
-      int x = c + 1 + group;
-      if (x < nb) { wait_word(&words.row_done[x], c + 1); pull(cluster_addr(block(c), x), v); }
-      if (group == 1) chol_emit(a, X, q, c);
-      for (; x < nb; x += CC_GROUPS) {
-        bar_sync(1 + group, 256);
+      if (first < end) {
+        const int mine = first + CC_GROUPS * lane;
+        if (!dry) wait_for(mine < end ? &words.row[c][mine] : nullptr);
+        pull(cluster_addr(from, dry ? q : first), v);
+      }
+      for (int x = first; x < end; x += CC_GROUPS) {
+        bar_sync(1 + group, 256);            // the block before this one is done with
         put(stage, v);
         bar_sync(1 + group, 256);
-        if (x + CC_GROUPS < nb) { wait_word(&words.row_done[x + CC_GROUPS], c + 1); pull(cluster_addr(block(c), x + CC_GROUPS), v); }
-        blk_mm(inv(x), X, stage, 3);
+        if (x + CC_GROUPS < end) pull(cluster_addr(from, x + CC_GROUPS), v);
+        Blk const C = dry ? Dfar : (left ? col(x) : inv(x));
+        if (left) blk_mm(C, stage, own, 1);
+        else blk_mm(C, own, stage, c == q ? 1 : 3);
       }
+      __syncthreads();
     }
-    // (the next step reads what the other group has brought up to date; the diagonal block is group 0's own)
-    if (c != q - 1) __syncthreads();
   }
   if (fail && lane == 0 && a.dev_status) atomicOr(a.dev_status, DEV_WAIT_EXPIRED);
   cluster_arrive();
   cluster_wait();
+  if (fail) for (int i = 0; i < 64; ++i) __nanosleep(1000);      // rows may still be on their way from the CTA before
 }
 
 size_t chol_cluster_smem(int nb) {
-  const size_t need = static_cast<size_t>(nb + 6 + CC_GROUPS) * CB * CP * 8;
+  const size_t need = static_cast<size_t>(nb + 4 + CC_GROUPS) * CB * CP * 8;
   return need > static_cast<size_t>(CHOL_SMEM_ASK) ? need : static_cast<size_t>(CHOL_SMEM_ASK);
 }
 
@@ -1021,16 +1092,51 @@ cudaError_t chol_smem_attr() {
   return e;
 }
 
-int pick_row_splits(int num_tiles, int64_t d) {
+void atb_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2], int tiles, int slices, cudaStream_t stream) {
+  cfg = {};
+  cfg.gridDim = dim3(tiles, slices);
+  cfg.blockDim = dim3(256);
+  cfg.stream = stream;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 1;
+  attr[0].val.clusterDim.y = slices;
+  attr[0].val.clusterDim.z = 1;
+  attr[1] = dependent_launch_attr();
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+}
+
+// Slices of the rows = CTAs of a tile's cluster: what lets the busiest SM go through the fewest chunks of 16 rows, two
+// chunks' time for every doubling (the sum over the slices).  Clusters do not fill every SM before one of them takes a
+// second CTA: 15 clusters of 8 ran side by side (2048 x 320 symmetric, 17 us), 16 did not (2048 x 256 by 256, 26 us).  16 is
+// more than the portable cluster size: only where the device can place it.
+int atb_slices(int tiles, int64_t d) {
+  static DeviceValue wide;                       // 1: no, 2: yes
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) { (void)cudaGetLastError(); return 8; }
+  int w = wide.get(dev);
+  if (w == 0) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    atb_config(cfg, attr, 1, 16, nullptr);
+    int clusters = 0;
+    const bool ok = cudaFuncSetAttribute(atb_f64_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&clusters, atb_f64_kernel, &cfg) == cudaSuccess && clusters >= 1;
+    if (!ok) (void)cudaGetLastError();
+    w = ok ? 2 : 1;
+    wide.set(dev, w);
+  }
   tc_init();
-  int sms = tc_num_sms();
-  if (sms <= 0) sms = 148;
-  int s = (2 * sms) / (num_tiles > 0 ? num_tiles : 1);
-  const int64_t max_by_rows = d / 64 > 0 ? d / 64 : 1;
-  if (s > max_by_rows) s = static_cast<int>(max_by_rows);
-  if (s < 1) s = 1;
-  if (s > 64) s = 64;
-  return s;
+  const int sms = tc_num_sms() > 0 ? tc_num_sms() : 148;
+  int best = 1;
+  long long least = -1;
+  for (int s = 1, doublings = 0; s <= (w == 2 ? 16 : 8); s *= 2, ++doublings) {
+    const int room = s <= 4 ? sms : (s == 8 ? sms * 13 / 16 : sms * 3 / 4);
+    const long long per_sm = (static_cast<long long>(tiles) * s + room - 1) / room;
+    const long long cost = per_sm * ((d + AT_K * s - 1) / (AT_K * s)) + 2 * doublings;
+    if (least < 0 || cost < least) { least = cost; best = s; }
+  }
+  return best;
 }
 
 }  // namespace
@@ -1038,53 +1144,33 @@ int pick_row_splits(int num_tiles, int64_t d) {
 PRAC_BOUNDS_READER(bounds_violations_cholqr)
 
 // ------------------------------------------------------------------ host side
-namespace {
-int atb_tiles(int64_t m, int64_t n, int symmetric) {
-  const int tm = static_cast<int>((m + AT_T - 1) / AT_T), tn = static_cast<int>((n + AT_T - 1) / AT_T);
-  return symmetric ? tn * (tn + 1) / 2 : tm * tn;
-}
-}  // namespace
-
-size_t atb_ws_bytes(int64_t m, int64_t n, int64_t d, int symmetric) {
-  if (m <= 0 || n <= 0 || d <= 0) return 0;
-  return static_cast<size_t>(pick_row_splits(atb_tiles(m, n, symmetric), d)) * m * n * sizeof(double);
-}
-
 int atb_f64(const float* A, int64_t lda, const float* B, int64_t ldb, int64_t d, int64_t m, int64_t n,
-            int symmetric, double alpha, void* out, int64_t ldo, int out_double, void* ws, size_t ws_bytes,
-            cudaStream_t stream, const int* run_if, int run_if_mask, void* zero_after, int zero_bytes) {
+            int symmetric, double alpha, void* out, int64_t ldo, int out_double, cudaStream_t stream, const int* run_if,
+            int run_if_mask, void* zero_words, int zero_bytes, bool next_early) {
   if (m <= 0 || n <= 0) return PRAC_OK;
   if (d <= 0 || (symmetric && (A != B || m != n))) return PRAC_EINVAL;
   AtbArgs g{};
   g.A = A; g.lda = lda; g.B = B; g.ldb = ldb;
   g.m = static_cast<int>(m); g.n = static_cast<int>(n); g.d = d;
-  g.tiles_m = static_cast<int>((m + AT_T - 1) / AT_T);
+  const int tiles_m = static_cast<int>((m + AT_T - 1) / AT_T);
   g.tiles_n = static_cast<int>((n + AT_T - 1) / AT_T);
   g.symmetric = symmetric;
-  g.num_tiles = atb_tiles(m, n, symmetric);
-  g.splits = pick_row_splits(g.num_tiles, d);
-  const size_t need = static_cast<size_t>(g.splits) * m * n * sizeof(double);
-  if (!ws || ws_bytes < need) return PRAC_EWORKSPACE;
-  g.partial = static_cast<double*>(ws);
+  g.alpha = alpha;
+  g.out = out; g.ldo = ldo; g.out_double = out_double;
+  g.next_early = next_early ? 1 : 0;
   g.run_if = run_if; g.run_if_mask = run_if_mask;
-  PRAC_LAUNCH(atb_f64_partial_kernel, dim3(static_cast<unsigned>(g.num_tiles), static_cast<unsigned>(g.splits)), dim3(256), 0, stream, g);
+  g.zero_words = static_cast<int*>(zero_words); g.zero_count = zero_bytes / 4;
+  const int tiles = symmetric ? g.tiles_n * (g.tiles_n + 1) / 2 : tiles_m * g.tiles_n;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[2];
+  atb_config(cfg, attr, tiles, atb_slices(tiles, d), stream);
+  PRAC_CUDA_TRY(cudaLaunchKernelEx(&cfg, atb_f64_kernel, g));
   count_launch();
-  if (out_double)
-    PRAC_LAUNCH(reduce_partials_kernel<double>, dim3(nblocks(m * n, 256)), dim3(256), 0, stream,
-                g.partial, g.splits, g.m, g.n, symmetric, alpha, static_cast<double*>(out), ldo, run_if, run_if_mask,
-                static_cast<int*>(zero_after), zero_bytes / 4);
-  else
-    PRAC_LAUNCH(reduce_partials_kernel<float>, dim3(nblocks(m * n, 256)), dim3(256), 0, stream,
-                g.partial, g.splits, g.m, g.n, symmetric, alpha, static_cast<float*>(out), ldo, run_if, run_if_mask,
-                static_cast<int*>(zero_after), zero_bytes / 4);
-  count_launch();
-  PRAC_CUDA_TRY(cudaGetLastError());
   return PRAC_OK;
 }
 
 // Workspace of one Cholesky-QR pass on n columns (all 256-byte aligned):
-//   G n*n double | R n*n double | X n*n double | Dinv nb*CB*CB double | diag0 n double | Rinv n*n float |
-//   slices of the transposed product
+//   G n*n double | R n*n double | X n*n double | Dinv nb*CB*CB double | diag0 n double | Rinv n*n float
 namespace {
 // Both operands as three bf16 pieces, side by side in rows of 3 kp: the segments of the chained
 // product mid*mid, lo*hi, hi*lo, mid*hi, hi*mid, hi*hi: everything down to 2^-24 of the product, the
@@ -1099,7 +1185,7 @@ TcSegments six_cross_terms(int64_t kp) {
   return segs;
 }
 
-struct CholWs { double* G; double* R; double* X; double* Dinv; double* diag0; float* Rinv; void* part; size_t part_bytes; size_t bytes;
+struct CholWs { double* G; double* R; double* X; double* Dinv; double* diag0; float* Rinv; size_t bytes;
                 __nv_bfloat16* V3; __nv_bfloat16* Rt3; int64_t kp; bool tensor; CholSync* sync; };
 // V R^-1 runs on the tensor cores (operands as three bf16 pieces each, six cross terms: fp32
 // accuracy) when the panel is big enough to fill their tiles.
@@ -1111,8 +1197,6 @@ CholWs carve_chol(void* ws, int64_t n, int64_t d) {
   auto take = [&](size_t b) { size_t o = off; off += (b + 255) / 256 * 256; return o; };
   const size_t oG = take(n * n * 8), oRR = take(n * n * 8), oX = take(n * n * 8), oD = take(nb * CB * CB * 8), o0 = take(n * 8);
   const size_t oR = take(n * n * 4);
-  c.part_bytes = atb_ws_bytes(n, n, d, 1);
-  const size_t oP = take(c.part_bytes);
   c.tensor = vr_on_tensor_cores(n, d);
   c.kp = (n + 63) / 64 * 64;
   const size_t oV3 = take(c.tensor ? static_cast<size_t>(d) * 3 * c.kp * 2 : 0);
@@ -1122,7 +1206,7 @@ CholWs carve_chol(void* ws, int64_t n, int64_t d) {
   c.sync = reinterpret_cast<CholSync*>(b + oBar);
   c.G = reinterpret_cast<double*>(b + oG); c.R = reinterpret_cast<double*>(b + oRR); c.X = reinterpret_cast<double*>(b + oX);
   c.Dinv = reinterpret_cast<double*>(b + oD); c.diag0 = reinterpret_cast<double*>(b + o0);
-  c.Rinv = reinterpret_cast<float*>(b + oR); c.part = b + oP;
+  c.Rinv = reinterpret_cast<float*>(b + oR);
   c.V3 = reinterpret_cast<__nv_bfloat16*>(b + oV3); c.Rt3 = reinterpret_cast<__nv_bfloat16*>(b + oR3);
   c.bytes = off;
   return c;
@@ -1139,9 +1223,10 @@ int cholqr_pass(const float* Vin, int64_t ldin, float* Vout, int64_t ldout, int6
   const CholWs c = carve_chol(ws, n, d);
   if (ws == nullptr || ws_bytes < c.bytes) return PRAC_EWORKSPACE;
   const int* run_if = run_if_mask ? dev_status : nullptr;
-  // (the reduction kernel also zeroes the grid-barrier state of the factorisation that follows it)
-  int st = atb_f64(Vin, ldin, Vin, ldin, d, n, n, 1, 1.0, c.G, n, 1, c.part, c.part_bytes, stream, run_if, run_if_mask,
-                   c.sync, static_cast<int>(sizeof(CholSync)));
+  // (the product's kernel also zeroes the state of the factorisation that follows it)
+  const int64_t nb = (n + CB - 1) / CB;
+  int st = atb_f64(Vin, ldin, Vin, ldin, d, n, n, 1, 1.0, c.G, n, 1, stream, run_if, run_if_mask,
+                   c.sync, static_cast<int>(sizeof(CholSync)), nb <= CC_MAX);
   if (st != PRAC_OK) return st;
   CholArgs a{};
   a.G = c.G; a.R = c.R; a.Dinv = c.Dinv; a.X = c.X; a.diag0 = c.diag0; a.Rinv = c.Rinv; a.ldr = n;

@@ -269,14 +269,13 @@ int launch_gaussian(uint64_t seed, uint64_t draw_counter, int64_t d, int64_t r, 
 // out (m x n, leading dimension ldo, double if out_double else float) = alpha * A^T B for fp32
 // A (d x m, lda) and B (d x n, ldb), accumulated in double over row slices that are summed in a
 // fixed order.  symmetric != 0 (A == B, m == n) computes the upper tiles and mirrors them.
-// ws >= atb_ws_bytes(m, n, d, symmetric).
-size_t atb_ws_bytes(int64_t m, int64_t n, int64_t d, int symmetric);
-// run_if != nullptr: both kernels return at once unless *run_if & run_if_mask (a device word).
-// zero_after: up to 1 KB (a multiple of 4 bytes) that the second kernel sets to zero.
+// run_if != nullptr: the kernel returns at once unless *run_if & run_if_mask (a device word).
+// zero_words: up to 1 KB (a multiple of 4 bytes) that the kernel sets to zero.  next_early: the next kernel on the
+// stream, a small grid, may be set up from the start of this one.
 int atb_f64(const float* A, int64_t lda, const float* B, int64_t ldb, int64_t d, int64_t m, int64_t n,
-            int symmetric, double alpha, void* out, int64_t ldo, int out_double, void* ws, size_t ws_bytes,
-            cudaStream_t stream, const int* run_if = nullptr, int run_if_mask = 0, void* zero_after = nullptr,
-            int zero_bytes = 0);
+            int symmetric, double alpha, void* out, int64_t ldo, int out_double, cudaStream_t stream,
+            const int* run_if = nullptr, int run_if_mask = 0, void* zero_words = nullptr, int zero_bytes = 0,
+            bool next_early = false);
 
 // One Cholesky-QR pass: Vout (d x n, ldout) = Vin (d x n, ldin) R^-1 with R^T R = Vin^T Vin, the
 // Gram matrix accumulated and factored in double.  R has a positive diagonal.  Vout != Vin.

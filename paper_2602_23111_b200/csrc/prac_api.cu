@@ -113,7 +113,7 @@ RitzWindow ritz_window(int64_t k, int64_t ell) {
   return win;
 }
 
-struct FitLayout { size_t C, V, Y, T2, Bj, Wsel, T, chol, jac, atb, Cs, Vs, mm, mm3, part, xpack, total; size_t mm3_bytes; int64_t ldxp; int64_t nj, wcols, kp, ldcs, ldvs; size_t chol_bytes, jac_bytes, atb_bytes, mm_bytes, part_bytes; };
+struct FitLayout { size_t C, V, Y, T2, Bj, Wsel, T, chol, jac, Cs, Vs, mm, mm3, part, xpack, total; size_t mm3_bytes; int64_t ldxp; int64_t nj, wcols, kp, ldcs, ldvs; size_t chol_bytes, jac_bytes, mm_bytes, part_bytes; };
 FitLayout fit_layout(const prac_params* p, int64_t N) {
   FitLayout L{};
   const int64_t d = p->d, k = p->k, r = p->r, ell = panel_cols(p);
@@ -128,16 +128,12 @@ FitLayout fit_layout(const prac_params* p, int64_t N) {
   L.Bj = c.take(static_cast<size_t>(L.nj) * L.nj * 8);
   L.Wsel = c.take(static_cast<size_t>(L.nj) * (k > 0 ? k : 1) * 4);
   L.T = c.take(static_cast<size_t>(k > 0 ? k : 1) * (r > 0 ? r : 1) * 4);
-  // the row-slice count, hence the scratch, is not monotone in the panel width: size for both
   const size_t chol_ell = cholqr_ws_bytes(ell, d), chol_r = cholqr_ws_bytes(r, d), chol_k = cholqr_ws_bytes(k, d);
   L.chol_bytes = chol_ell > chol_r ? chol_ell : chol_r;
   if (chol_k > L.chol_bytes) L.chol_bytes = chol_k;      // the warm refresh orthonormalises d x k panels
   L.chol = c.take(L.chol_bytes);
   L.jac_bytes = jacobi_ws_bytes(L.nj);
   L.jac = c.take(L.jac_bytes);
-  const size_t atb_rr = atb_ws_bytes(win.n, win.n, d, 0), atb_pr = atb_ws_bytes(k, r, d, 0);
-  L.atb_bytes = atb_rr > atb_pr ? atb_rr : atb_pr;
-  L.atb = c.take(L.atb_bytes);
   L.kp = round_up(d, 64);
   L.ldcs = round_up(d, 64);
   L.ldvs = round_up(ell > 0 ? ell : 1, 64);
@@ -446,7 +442,7 @@ int fit_principal_impl(prac_basis* b, const void* X, int64_t N, int64_t ldx, uin
   const float* Yb = Y + win.first;
   st_code = apply_gram(b, L, w, Yb, ell, win.n, V, win.n, st);
   if (st_code != PRAC_OK) return st_code;
-  st_code = atb_f64(Yb, ell, V, win.n, d, win.n, win.n, 0, 1.0, Bj, win.n, 1, w + L.atb, L.atb_bytes, st);
+  st_code = atb_f64(Yb, ell, V, win.n, d, win.n, win.n, 0, 1.0, Bj, win.n, 1, st);
   if (st_code != PRAC_OK) return st_code;
   st_code = jacobi_topk(Bj, win.n, win.n, win.w, Wsel, w + L.jac, L.jac_bytes, b->status, st);
   if (st_code != PRAC_OK) return st_code;
@@ -601,7 +597,7 @@ int prac_draw_random(prac_basis* b, uint64_t seed, uint64_t draw_counter, void* 
     const int reps = (8 * k > d) ? 2 : 1;
     for (int rep = 0; rep < reps; ++rep) {
       // T = U^T S ;  S -= U T
-      sc = atb_f64(b->P, s, S, r, d, k, r, 0, 1.0, T, r, 0, w + L.atb, L.atb_bytes, st);
+      sc = atb_f64(b->P, s, S, r, d, k, r, 0, 1.0, T, r, 0, st);
       if (sc != PRAC_OK) return sc;
       sc = panel_mm3(b->P, s, T, r, d, k, r, -1.f, S, r, 1, w + L.mm3, L.mm3_bytes, b->status, st);
       if (sc != PRAC_OK) return sc;

@@ -1,0 +1,48 @@
+"""The factorisation inside Cholesky-QR at the sizes where its kernel changes: blocks of 32 columns (one block, a last
+block of one column or one short), clusters above the portable eight CTAs, the kernel for more than 512 columns, and a
+panel whose rank ends inside a block.  Through prac_draw_random without a principal part, which orthonormalises a
+Gaussian block: its thin QR factor with positive diagonal is unique.
+
+Bounds: each column of Q to 1e-4 (fp32 panel, R exact to double), and the orthonormality that rounding Q to fp32 leaves,
+||Q^T Q - I||_F of about n 2^-24 with a constant of order one (8.5e-6 measured at 512 columns)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import prac_oracle as orc
+from paper_2602_23111_b200 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def f64(t):
+    return t.detach().to(torch.float32).cpu().numpy().astype(np.float64)
+
+
+@pytest.mark.parametrize("r", [1, 8, 31, 32, 33, 65, 256, 257, 320, 511, 512, 513, 640])
+def test_random_basis_is_the_unique_qr_factor(r):
+    from paper_2602_23111_b200 import api
+    d = max(256, 2 * r + 19)
+    b = api.Basis(d, 0, r, torch.float32)
+    b.draw_random(seed=11, draw_counter=5)
+    assert b.status() == api.PRAC_OK
+    Q = f64(b.projection()[0])
+    Q0 = orc.random_basis(np.zeros((d, 0)), orc.gaussian_draw(11, 5, d, r))
+    assert np.max(np.linalg.norm(Q - Q0, axis=0)) <= 1e-4
+    assert np.linalg.norm(Q.T @ Q - np.eye(r)) <= max(1e-5, 2e-5 * r / 512)
+    b.draw_random(seed=11, draw_counter=5)
+    assert np.array_equal(f64(b.projection()[0]), Q)          # sums in a fixed order, whoever is first
+
+
+@pytest.mark.parametrize("k, rank", [(256, 100), (128, 33), (64, 64)])
+def test_panel_whose_rank_ends_inside_a_block(k, rank):
+    # pivots are replaced from column `rank` on, in every block after it; the extra pass makes the rest orthonormal
+    from paper_2602_23111_b200 import api
+    N, d = 700, 640
+    X = inputs.make_planted(N, d, rank, seed=31, dtype="f32", exact_rank=True)
+    b = api.Basis(d, k, 8, torch.float32)
+    b.fit(X.cuda(), seed=6)
+    assert b.status() == api.PRAC_OK
+    U, X64 = f64(b.get()[0]), f64(X)
+    assert np.linalg.norm(U.T @ U - np.eye(k)) <= 1e-5
+    assert np.linalg.norm(X64 - X64 @ U @ U.T) <= 1e-4 * np.linalg.norm(X64)
