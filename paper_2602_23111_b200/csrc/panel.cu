@@ -101,19 +101,29 @@ constexpr int JAC_MAX_SWEEPS = 30;
 // The sweep that confirms is one of seven or eight on a power law.)
 // Sweeps that run out are an error only where a cosine of 1e-4 is left (JAC_FAIL_COS2).
 constexpr float JAC_DONE_COS2 = 1e-13f, JAC_FAIL_COS2 = 1e-8f;
+// A finishing step (jacobi_finish) is tried after a sweep that met cosines up to JAC_NEAR; it turns all pairs at once where no
+// angle is above JAC_STEP_ANGLE, and is the last one where none is above JAC_LAST_ANGLE: what it leaves is of the order
+// of the angles' squares, n 4e-10 at most.
+constexpr int JAC_MAX_FINISH = 8;
+constexpr float JAC_NEAR_COS2 = 1e-4f, JAC_STEP_ANGLE = 0.02f, JAC_LAST_ANGLE = 2e-5f;
 struct JacobiInfo {
   GridBarrierState bar;             // zeroed before the launch
   int sweeps;
   double inv_scale;                 // 1 / largest diagonal entry of B (written by jacobi_prepare_kernel)
   int rotations[JAC_MAX_SWEEPS];    // rotations applied in each outer sweep
   int max_cos2[JAC_MAX_SWEEPS];     // largest squared cosine rotated away in each sweep (float bits)
+  int fin_cos2[JAC_MAX_FINISH], fin_angle[JAC_MAX_FINISH];   // the same, and the largest angle, of each finishing step
+  double norms[128];                // squared norms of the columns in a finishing step
 };
 
 // Pair i of step `step` of the round-robin schedule on m (even) items, as p < q.
 __device__ __forceinline__ void rr_pair(int m, int step, int i, int& p, int& q) {
   int a, b;
   if (i == 0) { a = m - 1; b = step; }
-  else { a = (step + i) % (m - 1); b = (step - i + (m - 1)) % (m - 1); }
+  else {                       // (modulo m - 1, without a division: it is on the way from one visit to the next)
+    a = step + i; if (a >= m - 1) a -= m - 1;
+    b = step - i; if (b < 0) b += m - 1;
+  }
   p = a < b ? a : b;
   q = a < b ? b : a;
 }
@@ -507,8 +517,7 @@ __global__ void __launch_bounds__(256) jacobi_gram_kernel(double* At, int n, int
 // holds the 2 x 2 block where pairs u and v meet and works out both pairs' angles itself, so a round
 // is one barrier of two warps.  ROWS other threads hold one row each of the sixteen columns in registers
 // and apply the rounds in double as their angles are published: the update costs nothing beyond the
-// rounds, and no column passes through shared memory.  n = 128: 112 -> 61 us a sweep; of a visit's 7800
-// cycles the rounds take 500 each, forming G 900, the columns' way to the next CTA (store, barrier, load) 2600.
+// rounds.
 // (With G in fp32 and the rotations of G not on the unit circle a round takes 360 cycles, but the diagonal of
 // G then drifts by more than the columns of a cluster differ by: 18 to 30 sweeps there instead of 7 to 14.)
 //
@@ -517,11 +526,15 @@ __global__ void __launch_bounds__(256) jacobi_gram_kernel(double* At, int n, int
 // visit the 64 pairs that cross the two blocks ((i, 8 + y[i]), y moving up by one).  After the last
 // round every item is back in its place.
 //
-// CLUSTER: the whole grid is one thread-block cluster and the CTAs meet at the hardware cluster
-// barrier, whose release / acquire also orders their global-memory traffic; every CTA runs the same
+// CLUSTER: the whole grid is one thread-block cluster.  The columns never leave its shared memory: after a visit the
+// row threads store them where the next visit wants them, in the second buffer of the CTA before or after this one, whose
+// mbarrier counts their bytes (a visit's columns through global memory: 2350 cycles from the last round to the next Gram
+// matrix, and 1350 to form it from loads that go to L2, of 7400).  A buffer is free when it is stored to again two visits
+// later: the columns that this CTA needed meanwhile came from its two neighbours' visit after they had read it.  Only at the
+// end of a sweep do the CTAs meet at the hardware cluster barrier: every CTA runs the same
 // number of steps and sweeps (the stopping test reads values that are final before the barrier it
 // follows), so each barrier is reached by all of them.  Otherwise a cooperative launch with the
-// bounded software barrier.
+// bounded software barrier, the columns in global memory.
 constexpr int JS_G_THREADS = 256;      // form the Gram matrix; the first 64 walk the rounds
 constexpr int JS_R_THREADS = 64;
 constexpr int JS_MAX_ROWS = 256;
@@ -544,15 +557,167 @@ __device__ __forceinline__ void stream_pair(bool full, int is, int u, int& a, in
   b = is - u; if (b < 0) b += JG_M - 1;
 }
 
-// a' = c a + o b, b' = c b - o a make the columns orthogonal: with d = |b|^2 - |a|^2 and g = 2 a.b the
-// tangent of the smaller such angle is sign(d) g / (|d| + |(d, g)|).  (The hardware's approximations:
-// the angle only has to shrink the inner product.)
+// a' = c a + o b, b' = c b - o a make the columns orthogonal: with d = |b|^2 - |a|^2 and g = 2 a.b the smaller such angle has
+// cos 2t = |d| / |(d, g)|, sin 2t = sign(d) g / |(d, g)|; c = sqrt((1 + cos 2t) / 2), o = -sin 2t / (2 c).  (The hardware's
+// approximations, two in a row: the angle only has to shrink the inner product.  A shift of |d| by 1e-18 keeps the angle of
+// two zero columns zero.)
 __device__ __forceinline__ float2 stream_angle(double aa, double bb, double ab) {
   const float d = static_cast<float>(bb - aa), g = 2.f * static_cast<float>(ab);
-  const float q = fmaf(d, d, fmaf(g, g, 1e-36f));
-  const float t = copysignf(1.f, d) * g * rcp_approx(fmaf(q, rsqrt_fast(q), fabsf(d)));
-  const float c = rsqrt_fast(fmaf(t, t, 1.f));
-  return make_float2(c, -c * t);
+  const float ad = fabsf(d) + 1e-18f;
+  const float ih = rsqrt_fast(fmaf(ad, ad, g * g));
+  const float c2 = fmaf(0.5f * ad, ih, 0.5f);
+  const float rc = rsqrt_fast(c2);
+  return make_float2(c2 * rc, -0.5f * copysignf(1.f, d) * g * ih * rc);
+}
+
+// Where block X of m (even) is in step `step` of the round-robin schedule: CTA and slot (0: the lower block of the pair).
+__device__ __forceinline__ void rr_where(int m, int step, int X, int& cta, int& slot) {
+  int partner;
+  if (X == m - 1) { cta = 0; partner = step; }
+  else if (X == step) { cta = 0; partner = m - 1; }
+  else {
+    int d = X - step;
+    if (d < 0) d += m - 1;
+    const bool first = d <= m / 2 - 1;
+    cta = first ? d : m - 1 - d;
+    partner = first ? step - cta : step + cta;
+    if (partner < 0) partner += m - 1;
+    if (partner >= m - 1) partner -= m - 1;
+  }
+  slot = X < partner ? 0 : 1;
+}
+
+__device__ __forceinline__ uint32_t cluster_smem(const void* own, int cta) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(own))), "r"(cta));
+  return r;
+}
+__device__ __forceinline__ double cluster_ld(uint32_t addr) {
+  double v;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void cluster_barrier() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// A finishing step on the columns of all CTAs (16 each; up to ROWS of them), once they are nearly orthogonal:
+// the whole Gram matrix, and then either nothing more (no cosine is left above the level of fp32), or, where every pair's
+// rotation angle g_ij / (g_jj - g_ii) is small, all rotations at once to first order, A <- A (I + T), or nothing because
+// columns of nearly equal norm still turn by large angles.  Pairs that are orthogonal already are left alone, however
+// close their norms.  It takes some 12 000 cycles at 128 columns, where a sweep takes 100 000, and it converges as the
+// sweeps do at the end, quadratically.  Called by all threads of all CTAs; returns 0: no step, 1: one step, 2: converged,
+// -1: a barrier gave up.
+// cols: this CTA's columns in shared memory (CLUSTER), else they are in At, as the next sweep's first step pairs them.  The
+// norms pass through info.
+template <bool CLUSTER, int ROWS>
+__device__ __noinline__ int jacobi_finish(double (*cols)[ROWS + 2], double* At, int n, double (*T)[ROWS + 2], double (*Gp)[ROWS + 2],
+                                          double scale2, JacobiInfo* info, int attempt, unsigned& bar, unsigned poll_limit) {
+  __shared__ double norms[ROWS];
+  __shared__ int worst[2];
+  constexpr int WARPS = (JS_G_THREADS + ROWS) / 32;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q4 = lane & 3;
+  const int ctas = gridDim.x, rank = blockIdx.x;
+  // column e of CTA c: where it starts in At
+  auto column = [&](int c, int e) {
+    int I, J;
+    rr_pair(2 * ctas, 0, c, I, J);
+    return At + static_cast<long long>(e < JG_B ? I * JG_B + e : J * JG_B + e - JG_B) * n;
+  };
+  auto meet = [&]() {
+    if (CLUSTER) { cluster_barrier(); return true; }
+    return grid_barrier(&info->bar, ++bar * gridDim.x, poll_limit);
+  };
+  // ---- Gp[i][j] = column i of this CTA times column j of all
+  for (int job = warp; job < 2 * ctas; job += WARPS) {
+    const int e = 8 * (job & 1) + g;
+    const uint32_t other = CLUSTER ? cluster_smem(&cols[e][q4], job >> 1) : 0u;
+    const double* const in_mem = CLUSTER ? nullptr : column(job >> 1, e) + q4;
+    const double* const own0 = CLUSTER ? &cols[g][q4] : column(rank, g) + q4;
+    const double* const own1 = CLUSTER ? &cols[8 + g][q4] : column(rank, 8 + g) + q4;
+    double acc0[2] = {0.0, 0.0}, acc1[2] = {0.0, 0.0};
+#pragma unroll 8
+    for (int ks = 0; ks < ROWS / 4; ++ks) {
+      double a0, a1, b;
+      if (CLUSTER) {
+        b = cluster_ld(other + ks * 32);
+        a0 = own0[4 * ks]; a1 = own1[4 * ks];
+      } else {                         // (n is a multiple of 16)
+        const bool in = 4 * ks < n;
+        b = in ? __ldcg(in_mem + 4 * ks) : 0.0;
+        a0 = in ? __ldcg(own0 + 4 * ks) : 0.0; a1 = in ? __ldcg(own1 + 4 * ks) : 0.0;
+      }
+      dmma_884(acc0, a0, b);
+      dmma_884(acc1, a1, b);
+    }
+#pragma unroll
+    for (int e2 = 0; e2 < 2; ++e2) {
+      Gp[g][8 * job + 2 * q4 + e2] = acc0[e2] * scale2;
+      Gp[8 + g][8 * job + 2 * q4 + e2] = acc1[e2] * scale2;
+    }
+  }
+  if (threadIdx.x < 2) worst[threadIdx.x] = 0;
+  __syncthreads();
+  if (threadIdx.x < JG_M) info->norms[JG_M * rank + threadIdx.x] = Gp[threadIdx.x][JG_M * rank + threadIdx.x];
+  if (!meet()) return -1;
+  for (int j = threadIdx.x; j < n; j += blockDim.x) norms[j] = __ldcg(&info->norms[j]);
+  __syncthreads();
+  // ---- T: the angle by which column j of this CTA takes up column i
+  float cos2 = 0.f, angle = 0.f;
+  for (int idx = threadIdx.x; idx < JG_M * n; idx += blockDim.x) {
+    const int j = idx / n, i = idx % n, jj = JG_M * rank + j;
+    const double v = Gp[j][i], di = norms[i], dj = norms[jj];
+    const float c2 = i == jj ? 0.f : static_cast<float>(v * v / (di * dj));
+    double t = 0.0;
+    if (c2 > 1e-14f) {
+      t = v / (dj - di);
+      cos2 = fmaxf(cos2, fminf(c2, 1.f));
+      angle = fmaxf(angle, fminf(fabsf(static_cast<float>(t)), 1e30f));
+    }
+    T[j][i] = t;
+  }
+  const int w0 = __reduce_max_sync(0xffffffffu, __float_as_int(cos2)), w1 = __reduce_max_sync(0xffffffffu, __float_as_int(angle));
+  if (lane == 0) { atomicMax(&worst[0], w0); atomicMax(&worst[1], w1); }   // (non-negative floats order as ints)
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    atomicMax(&info->fin_cos2[attempt], worst[0]);
+    atomicMax(&info->fin_angle[attempt], worst[1]);
+  }
+  if (!meet()) return -1;
+  cos2 = __int_as_float(*reinterpret_cast<volatile int*>(&info->fin_cos2[attempt]));
+  angle = __int_as_float(*reinterpret_cast<volatile int*>(&info->fin_angle[attempt]));
+  if (cos2 < JAC_DONE_COS2) return 2;
+  if (!(angle <= JAC_STEP_ANGLE)) return 0;
+  // ---- columns of this CTA += all columns times T, eight rows at a time, into Gp
+  for (int band = warp; 8 * band < n; band += WARPS) {
+    double acc0[2] = {0.0, 0.0}, acc1[2] = {0.0, 0.0};
+    const int r = 8 * band + g;
+    for (int c = 0; c < ctas; ++c) {
+      const uint32_t other = CLUSTER ? cluster_smem(&cols[q4][r], c) : 0u;
+#pragma unroll
+      for (int ks = 0; ks < JG_M / 4; ++ks) {
+        const double a = CLUSTER ? cluster_ld(other + ks * 4 * (ROWS + 2) * 8) : __ldcg(column(c, 4 * ks + q4) + r);
+        dmma_884(acc0, a, T[g][JG_M * c + 4 * ks + q4]);
+        dmma_884(acc1, a, T[8 + g][JG_M * c + 4 * ks + q4]);
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const int e = 8 * (h >> 1) + 2 * q4 + (h & 1);
+      const double old = CLUSTER ? cols[e][r] : __ldcg(column(rank, e) + r);
+      Gp[e][r] = old + (h < 2 ? acc0[h] : acc1[h - 2]);
+    }
+  }
+  if (!meet()) return -1;              // (nobody reads the old columns any more)
+  for (int idx = threadIdx.x; idx < JG_M * n; idx += blockDim.x) {
+    const int e = idx / n, r = idx % n;
+    if (CLUSTER) cols[e][r] = Gp[e][r];
+    else column(rank, e)[r] = Gp[e][r];
+  }
+  if (!meet()) return -1;
+  return angle <= JAC_LAST_ANGLE ? 2 : 1;
 }
 
 template <bool CLUSTER, int ROWS>   // ROWS = 128 or 256 >= n
@@ -563,6 +728,10 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
   __shared__ double G[2][JG_M][JG_P];
   __shared__ float2 coef[JG_M][JG_B];            // every round of the visit, per pair: c, o
   __shared__ double2 unit[ROWS / 32][2][JG_B];   // two rounds of them on the unit circle, per row warp
+  // CLUSTER: the sixteen columns of this visit and of the next, which the CTAs of this visit store here
+  extern __shared__ __align__(16) double jacobi_cols[];
+  __shared__ uint64_t arrived[2];                // all of a buffer's columns are there
+  typedef double (*Cols)[ROWS + 2];
   const int b = JG_B;
   const int nb = n / b;                          // even: n is a multiple of 16
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -574,12 +743,32 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
   bool alive = true, converged = false;
   float mc2 = 1.f;
   int sweep = 0;
+  unsigned visit = 0;
+  bool late = false;
+  int attempt = 0, refused = 0;
+  if (CLUSTER) {
+    if (threadIdx.x < 2)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(&arrived[threadIdx.x]))) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    int I, J;
+    rr_pair(nb, 0, blockIdx.x, I, J);
+    for (int e = warp; e < JG_M; e += (JS_G_THREADS + ROWS) / 32)
+      for (int r = lane; r < ROWS; r += 32)
+        reinterpret_cast<Cols>(jacobi_cols)[e][r] = r < n ? __ldcg(At + static_cast<long long>((e < b ? I * b + e : J * b + e - b)) * n + r) : 0.0;
+    __syncthreads();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");      // (every CTA of the cluster has started)
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
   for (; alive && sweep < max_sweeps && !converged; ++sweep) {
     for (int step = 0; alive && step < nb - 1; ++step) {
       int I, J;
       rr_pair(nb, step, blockIdx.x, I, J);
       double* const colI = At + static_cast<long long>(I) * b * n;
       double* const colJ = At + static_cast<long long>(J) * b * n;
+      const unsigned turn = visit & 1;
+      Cols const here = reinterpret_cast<Cols>(jacobi_cols) + turn * JG_M, there = reinterpret_cast<Cols>(jacobi_cols) + (turn ^ 1) * JG_M;
+      if (CLUSTER && threadIdx.x == 0)
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(&arrived[turn ^ 1]))), "n"(JG_M * ROWS * 8) : "memory");
       const bool full = step == 0;
       const int rounds = full ? JG_M - 1 : JG_B;
       if (row_thread) {
@@ -588,8 +777,13 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
         double x[JG_M];
 #pragma unroll
         for (int e = 0; e < JG_B; ++e) {
-          x[e] = r < n ? __ldcg(colI + e * n + r) : 0.0;
-          x[JG_B + e] = r < n ? __ldcg(colJ + e * n + r) : 0.0;
+          if (CLUSTER) {
+            x[e] = here[e][r];
+            x[JG_B + e] = here[JG_B + e][r];
+          } else {
+            x[e] = r < n ? __ldcg(colI + e * n + r) : 0.0;
+            x[JG_B + e] = r < n ? __ldcg(colJ + e * n + r) : 0.0;
+          }
         }
         auto rotate = [&](const double2 co, int a, int bq) {
           const double xa = x[a], xb = x[bq];
@@ -631,7 +825,20 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
           }
           __syncwarp();
         }
-        if (r < n) {
+        if (CLUSTER) {
+          const int next = step + 1 < nb - 1 ? step + 1 : 0;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            int cta, slot;
+            rr_where(nb, next, h ? J : I, cta, slot);
+            uint32_t to, bar;
+            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(&there[JG_B * slot][r]))), "r"(cta));
+            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(bar) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(&arrived[turn ^ 1]))), "r"(cta));
+#pragma unroll
+            for (int e = 0; e < JG_B; ++e)
+              asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f64 [%0], %1, [%2];" ::"r"(to + e * (ROWS + 2) * 8), "d"(x[JG_B * h + e]), "r"(bar) : "memory");
+          }
+        } else if (r < n) {
 #pragma unroll
           for (int e = 0; e < JG_B; ++e) {
             colI[e * n + r] = x[e];
@@ -648,10 +855,16 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
           for (int h = 0; h < ROWS / 128; ++h) {
             const int r = (warp + 8 * h) * 16 + 4 * q4;
             const double2 zero = make_double2(0.0, 0.0);
-            const double2* p0 = reinterpret_cast<const double2*>(colI + g * n + r);
-            const double2* p1 = reinterpret_cast<const double2*>(colJ + g * n + r);
-            v[h][0] = r < n ? __ldcg(p0) : zero; v[h][1] = r < n ? __ldcg(p0 + 1) : zero;
-            v[h][2] = r < n ? __ldcg(p1) : zero; v[h][3] = r < n ? __ldcg(p1 + 1) : zero;
+            if (CLUSTER) {
+              const double2* p0 = reinterpret_cast<const double2*>(&here[g][r]);
+              const double2* p1 = reinterpret_cast<const double2*>(&here[JG_B + g][r]);
+              v[h][0] = p0[0]; v[h][1] = p0[1]; v[h][2] = p1[0]; v[h][3] = p1[1];
+            } else {
+              const double2* p0 = reinterpret_cast<const double2*>(colI + g * n + r);
+              const double2* p1 = reinterpret_cast<const double2*>(colJ + g * n + r);
+              v[h][0] = r < n ? __ldcg(p0) : zero; v[h][1] = r < n ? __ldcg(p0 + 1) : zero;
+              v[h][2] = r < n ? __ldcg(p1) : zero; v[h][3] = r < n ? __ldcg(p1 + 1) : zero;
+            }
           }
 #pragma unroll
           for (int h = 0; h < ROWS / 128; ++h) {
@@ -743,9 +956,28 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
         }
       }
       if (CLUSTER) {
+        // (the whole CTA has to be through with this visit's angles; and warps that polled meanwhile would slow those that
+        // work: a round 457 -> 540 cycles)
+        __syncthreads();
+        if (lane == 0 && !late) {
+          const uint32_t bar_addr = static_cast<uint32_t>(__cvta_generic_to_shared(&arrived[turn ^ 1]));
+          unsigned polls = 0, ok = 0;
+          while (true) {
+            asm volatile(
+                "{\n\t.reg .pred P;\n\t"
+                "mbarrier.try_wait.parity.shared::cta.b64 P, [%1], %2;\n\t"
+                "selp.b32 %0, 1, 0, P;\n\t}"
+                : "=r"(ok) : "r"(bar_addr), "r"((visit >> 1) & 1u) : "memory");
+            if (ok) break;
+            if (++polls >= poll_limit) { late = true; break; }    // (it carries on with what it has: everybody meets below)
+          }
+        }
         __syncwarp();
-        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        ++visit;
+        if (step == nb - 2) {          // the sweep's largest cosine is complete
+          asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+          asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        }
       } else {
         alive = grid_barrier(&info->bar, ++bar * nctas, poll_limit);
       }
@@ -753,7 +985,25 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
     if (alive) {
       mc2 = __int_as_float(*reinterpret_cast<volatile int*>(&info->max_cos2[sweep]));
       converged = mc2 < JAC_DONE_COS2;
+      if (ROWS == 128) {               // (128 columns: 449 -> 391 us in all; a step's two matrices of 256 columns do not fit beside the buffers)
+        while (alive && !converged && mc2 < JAC_NEAR_COS2 && attempt < JAC_MAX_FINISH && refused < 3) {
+          Cols const buf = reinterpret_cast<Cols>(jacobi_cols);
+          const int r = jacobi_finish<CLUSTER, ROWS>(buf + (visit & 1) * JG_M, At, n, buf + ((visit & 1) ^ 1) * JG_M, buf + 2 * JG_M,
+                                                     inv_scale * inv_scale, info, attempt++, bar, poll_limit);
+          alive = r >= 0;
+          converged = r == 2;
+          if (r == 0) { ++refused; break; }
+        }
+      }
     }
+  }
+  if (CLUSTER) {                       // (the columns lie as the next sweep's first step has them)
+    int I, J;
+    rr_pair(nb, 0, blockIdx.x, I, J);
+    for (int e = warp; e < JG_M; e += (JS_G_THREADS + ROWS) / 32)
+      for (int r = lane; r < n; r += 32)
+        At[static_cast<long long>((e < b ? I * b + e : J * b + e - b)) * n + r] = (reinterpret_cast<Cols>(jacobi_cols) + (visit & 1) * JG_M)[e][r];
+    if (late && dev_status) atomicOr(dev_status, DEV_WAIT_EXPIRED);
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     info->sweeps = sweep;
@@ -1381,11 +1631,13 @@ int jacobi_topk(const double* B, int64_t ldb, int64_t ell, int64_t k, float* Wse
     void (*const on_grid)(double*, int, int, JacobiInfo*, int*, unsigned) =
         n <= 128 ? jacobi_stream_kernel<false, 128> : jacobi_stream_kernel<false, 256>;
     const unsigned threads = JS_G_THREADS + (n <= 128 ? 128 : 256);
+    const int cols_smem = (n <= 128 ? 3 : 2) * JG_M * ((n <= 128 ? 128 : 256) + 2) * 8;
     bool as_cluster = poll_limit == GRID_BARRIER_POLLS;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = cols_smem;
     cfg.stream = stream;
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = grid;
@@ -1394,6 +1646,14 @@ int jacobi_topk(const double* B, int64_t ldb, int64_t ell, int64_t k, float* Wse
     attr[1] = dependent_launch_attr();
     cfg.attrs = attr;
     cfg.numAttrs = 2;
+    if (as_cluster) {
+      static DeviceOnce smem_attr[2];
+      DeviceOnce& once = smem_attr[n <= 128 ? 0 : 1];
+      if (!once.done(dev)) {
+        PRAC_CUDA_TRY(cudaFuncSetAttribute(on_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, cols_smem));
+        once.mark(dev);
+      }
+    }
     if (as_cluster && grid > 8) {
       static DeviceOnce wide_attr;
       if (!wide_attr.done(dev)) {
@@ -1416,7 +1676,13 @@ int jacobi_topk(const double* B, int64_t ldb, int64_t ell, int64_t k, float* Wse
       PRAC_CUDA_TRY(cudaLaunchKernelEx(&cfg, on_cluster, at, ni, max_sweeps, info, dev_status, poll_limit));
     } else {
       void* sargs[] = {&at, &ni, &max_sweeps, &info, &dev_status, &poll_limit};
-      PRAC_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(on_grid), dim3(grid), dim3(threads), sargs, 0, stream));
+      static DeviceOnce grid_attr;
+      if (n <= 128 && !grid_attr.done(dev)) {
+        PRAC_CUDA_TRY(cudaFuncSetAttribute(on_grid, cudaFuncAttributeMaxDynamicSharedMemorySize, cols_smem));
+        grid_attr.mark(dev);
+      }
+      PRAC_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(on_grid), dim3(grid), dim3(threads), sargs,
+                                                n <= 128 ? cols_smem : 0, stream));   // (a finishing step's two matrices)
     }
   } else if (gram) {
     void* gargs[] = {&at, &ni, &max_sweeps, &tol, &info, &dev_status, &poll_limit};
