@@ -847,10 +847,9 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
     for (int e = 0; e < 2; ++e) *reinterpret_cast<double2*>(&to[(gt + 256 * e) >> 4][2 * (gt & 15)]) = v[e];
   };
 
-  // c = -2: the dry run (an optional pass, which is nearly always off, goes without, and so do one or
-  // two blocks, whose CTAs the product before does not keep waiting for long enough); c = -1: set-up, and CTA 0
+  // c = -2: the dry run (an optional pass, which is nearly always off, goes without); c = -1: set-up, and CTA 0
   // factors its block; then the steps
-  for (int c = a.run_if_mask || nb <= 2 ? -1 : -2; c < nb; ++c) {
+  for (int c = a.run_if_mask ? -1 : -2; c < nb; ++c) {
     const bool dry = c == -2;
     if (c < 0) {
       const int rows = dry ? 0 : n;              // (the dry run reads and writes no global memory)
