@@ -101,18 +101,18 @@ constexpr int JAC_MAX_SWEEPS = 30;
 // The sweep that confirms is one of seven or eight on a power law.)
 // Sweeps that run out are an error only where a cosine of 1e-4 is left (JAC_FAIL_COS2).
 constexpr float JAC_DONE_COS2 = 1e-13f, JAC_FAIL_COS2 = 1e-8f;
-// A finishing step (jacobi_finish) is tried after a sweep that met cosines up to JAC_NEAR; it turns all pairs at once where no
-// angle is above JAC_STEP_ANGLE, and is the last one where none is above JAC_LAST_ANGLE: what it leaves is of the order
-// of the angles' squares, n 4e-10 at most.
+// A finishing step (jacobi_finish) is tried after a sweep that met cosines up to JAC_NEAR; it turns all columns at once where
+// no column's angles add up to more than JAC_STEP_TURN, by a rotation that is orthogonal to JAC_TURN_REST, and is the
+// last one where they add up to no more than JAC_LAST_TURN.
 constexpr int JAC_MAX_FINISH = 8;
-constexpr float JAC_NEAR_COS2 = 1e-4f, JAC_STEP_ANGLE = 0.02f, JAC_LAST_ANGLE = 2e-5f;
+constexpr float JAC_NEAR_COS2 = 1e-4f, JAC_STEP_TURN = 0.2f, JAC_TURN_REST = 1e-12f, JAC_LAST_TURN = 2e-5f;
 struct JacobiInfo {
   GridBarrierState bar;             // zeroed before the launch
   int sweeps;
   double inv_scale;                 // 1 / largest diagonal entry of B (written by jacobi_prepare_kernel)
   int rotations[JAC_MAX_SWEEPS];    // rotations applied in each outer sweep
   int max_cos2[JAC_MAX_SWEEPS];     // largest squared cosine rotated away in each sweep (float bits)
-  int fin_cos2[JAC_MAX_FINISH], fin_angle[JAC_MAX_FINISH];   // the same, and the largest angle, of each finishing step
+  int fin_cos2[JAC_MAX_FINISH], fin_turn[JAC_MAX_FINISH];    // the same, and the largest sum of a column's angles, of each finishing step
   double norms[128];                // squared norms of the columns in a finishing step
 };
 
@@ -604,17 +604,23 @@ __device__ __forceinline__ void cluster_barrier() {
 }
 
 // A finishing step on the columns of all CTAs (16 each; up to ROWS of them), once they are nearly orthogonal:
-// the whole Gram matrix, and then either nothing more (no cosine is left above the level of fp32), or, where every pair's
-// rotation angle g_ij / (g_jj - g_ii) is small, all rotations at once to first order, A <- A (I + T), or nothing because
+// the whole Gram matrix, and then either nothing more (no cosine is left above the level of fp32), or, where the
+// rotation angles T_ij = g_ij / (g_jj - g_ii) of all pairs are small, one rotation for all of them, A <- A exp(T), or nothing because
 // columns of nearly equal norm still turn by large angles.  Pairs that are orthogonal already are left alone, however
-// close their norms.  It takes some 12 000 cycles at 128 columns, where a sweep takes 100 000, and it converges as the
-// sweeps do at the end, quadratically.  Called by all threads of all CTAs; returns 0: no step, 1: one step, 2: converged,
-// -1: a barrier gave up.
-// cols: this CTA's columns in shared memory (CLUSTER), else they are in At, as the next sweep's first step pairs them.  The
-// norms pass through info.
+// close their norms.  It converges as the sweeps do at the end, quadratically: of the cosines it leaves products of two.
+// T is antisymmetric to the last bit (both CTAs of a pair add the same products in the same order), so exp(T) is a rotation
+// and A = B J keeps an orthogonal J, without which orthogonal columns need not be eigenvectors: I + T alone, off by T^2, turned
+// single eigenvectors of power laws by up to 1e-3 (64 and 128 columns), exp(T) by what fp32 leaves, as the sweeps do.
+// The series is summed until what is cut off is below JAC_TURN_REST: two to nine terms A T^m / m!, some 4000 cycles
+// each at 128 columns, after 8000 for the Gram matrix, where a sweep takes 100 000.
+// Called by all threads of all CTAs; returns 0: no step, 1: one step, 2: converged, -1: a barrier gave up.
+// CLUSTER: cols are this CTA's columns and term0, term1 two buffers for its columns of the terms, in shared memory (term0 holds
+// the Gram matrix before).  Else the columns are in At, as the next sweep's first step pairs them, the terms in terms (2 n x n), and
+// term0 holds the Gram matrix.  The norms pass through info.
 template <bool CLUSTER, int ROWS>
-__device__ __noinline__ int jacobi_finish(double (*cols)[ROWS + 2], double* At, int n, double (*T)[ROWS + 2], double (*Gp)[ROWS + 2],
-                                          double scale2, JacobiInfo* info, int attempt, unsigned& bar, unsigned poll_limit) {
+__device__ __noinline__ int jacobi_finish(double (*cols)[ROWS + 2], double* At, double* terms, int n, double (*T)[ROWS + 2],
+                                          double (*term0)[ROWS + 2], double (*term1)[ROWS + 2], double scale2, JacobiInfo* info,
+                                          int attempt, unsigned& bar, unsigned poll_limit) {
   __shared__ double norms[ROWS];
   __shared__ int worst[2];
   constexpr int WARPS = (JS_G_THREADS + ROWS) / 32;
@@ -631,6 +637,7 @@ __device__ __noinline__ int jacobi_finish(double (*cols)[ROWS + 2], double* At, 
     return grid_barrier(&info->bar, ++bar * gridDim.x, poll_limit);
   };
   // ---- Gp[i][j] = column i of this CTA times column j of all
+  double (*const Gp)[ROWS + 2] = term0;
   for (int job = warp; job < 2 * ctas; job += WARPS) {
     const int e = 8 * (job & 1) + g;
     const uint32_t other = CLUSTER ? cluster_smem(&cols[e][q4], job >> 1) : 0u;
@@ -664,65 +671,92 @@ __device__ __noinline__ int jacobi_finish(double (*cols)[ROWS + 2], double* At, 
   if (!meet()) return -1;
   for (int j = threadIdx.x; j < n; j += blockDim.x) norms[j] = __ldcg(&info->norms[j]);
   __syncthreads();
-  // ---- T: the angle by which column j of this CTA takes up column i
-  float cos2 = 0.f, angle = 0.f;
-  for (int idx = threadIdx.x; idx < JG_M * n; idx += blockDim.x) {
-    const int j = idx / n, i = idx % n, jj = JG_M * rank + j;
-    const double v = Gp[j][i], di = norms[i], dj = norms[jj];
-    const float c2 = i == jj ? 0.f : static_cast<float>(v * v / (di * dj));
-    double t = 0.0;
-    if (c2 > 1e-14f) {
-      t = v / (dj - di);
-      cos2 = fmaxf(cos2, fminf(c2, 1.f));
-      angle = fmaxf(angle, fminf(fabsf(static_cast<float>(t)), 1e30f));
+  // ---- T: the angle by which column j of this CTA takes up column i; turn: the sum of a column's angles
+  float cos2 = 0.f, turn = 0.f;
+  for (int j = warp; j < JG_M; j += WARPS) {
+    const int jj = JG_M * rank + j;
+    float sum = 0.f;
+    for (int i = lane; i < n; i += 32) {
+      const double v = Gp[j][i], di = norms[i], dj = norms[jj];
+      const float c2 = i == jj ? 0.f : static_cast<float>(v * v / (di * dj));
+      double t = 0.0;
+      if (c2 > 1e-14f) {
+        t = v / (dj - di);
+        cos2 = fmaxf(cos2, fminf(c2, 1.f));
+        sum += fabsf(static_cast<float>(t));
+      }
+      T[j][i] = t;
     }
-    T[j][i] = t;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    turn = fmaxf(turn, fminf(sum, 1e30f));
   }
-  const int w0 = __reduce_max_sync(0xffffffffu, __float_as_int(cos2)), w1 = __reduce_max_sync(0xffffffffu, __float_as_int(angle));
+  const int w0 = __reduce_max_sync(0xffffffffu, __float_as_int(cos2)), w1 = __reduce_max_sync(0xffffffffu, __float_as_int(turn));
   if (lane == 0) { atomicMax(&worst[0], w0); atomicMax(&worst[1], w1); }   // (non-negative floats order as ints)
   __syncthreads();
   if (threadIdx.x == 0) {
     atomicMax(&info->fin_cos2[attempt], worst[0]);
-    atomicMax(&info->fin_angle[attempt], worst[1]);
+    atomicMax(&info->fin_turn[attempt], worst[1]);
   }
   if (!meet()) return -1;
   cos2 = __int_as_float(*reinterpret_cast<volatile int*>(&info->fin_cos2[attempt]));
-  angle = __int_as_float(*reinterpret_cast<volatile int*>(&info->fin_angle[attempt]));
+  turn = __int_as_float(*reinterpret_cast<volatile int*>(&info->fin_turn[attempt]));
   if (cos2 < JAC_DONE_COS2) return 2;
-  if (!(angle <= JAC_STEP_ANGLE)) return 0;
-  // ---- columns of this CTA += all columns times T, eight rows at a time, into Gp
-  for (int band = warp; 8 * band < n; band += WARPS) {
-    double acc0[2] = {0.0, 0.0}, acc1[2] = {0.0, 0.0};
-    const int r = 8 * band + g;
-    for (int c = 0; c < ctas; ++c) {
-      const uint32_t other = CLUSTER ? cluster_smem(&cols[q4][r], c) : 0u;
+  if (!(turn <= JAC_STEP_TURN)) return 0;
+  // ---- columns of this CTA += all columns times T, times T^2 / 2, ..; a term is the product of the one before it, eight
+  // rows at a time.  turn is the 1-norm of T (and, T being antisymmetric, its infinity norm), so the terms after the m-th
+  // add up to turn^(m + 1) / (m + 1)! and a little
+  bool last = false;
+  float rest = turn;
+  for (int m = 1; !last; ++m) {
+    rest *= turn / static_cast<float>(m + 1);
+    last = rest <= JAC_TURN_REST;
+    double (*const from)[ROWS + 2] = m == 1 ? cols : ((m & 1) ? term1 : term0);
+    double (*const to)[ROWS + 2] = (m & 1) ? term0 : term1;
+    const long long nn = static_cast<long long>(n) * n;
+    const double* const from_mem = terms + ((m & 1) ? nn : 0);
+    double* const to_mem = terms + ((m & 1) ? 0 : nn) + static_cast<long long>(JG_M) * rank * n;
+    const double scale = 1.0 / m;
+    for (int band = warp; 8 * band < n; band += WARPS) {
+      double acc0[2] = {0.0, 0.0}, acc1[2] = {0.0, 0.0};
+      const int r = 8 * band + g;
+      for (int c = 0; c < ctas; ++c) {
+        const uint32_t other = CLUSTER ? cluster_smem(&from[q4][r], c) : 0u;
 #pragma unroll
-      for (int ks = 0; ks < JG_M / 4; ++ks) {
-        const double a = CLUSTER ? cluster_ld(other + ks * 4 * (ROWS + 2) * 8) : __ldcg(column(c, 4 * ks + q4) + r);
-        dmma_884(acc0, a, T[g][JG_M * c + 4 * ks + q4]);
-        dmma_884(acc1, a, T[8 + g][JG_M * c + 4 * ks + q4]);
+        for (int ks = 0; ks < JG_M / 4; ++ks) {
+          const int e = 4 * ks + q4;
+          const double a = CLUSTER ? cluster_ld(other + ks * 4 * (ROWS + 2) * 8)
+                                   : __ldcg(m == 1 ? column(c, e) + r : from_mem + static_cast<long long>(JG_M * c + e) * n + r);
+          dmma_884(acc0, a, T[g][JG_M * c + e]);
+          dmma_884(acc1, a, T[8 + g][JG_M * c + e]);
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        const int e = 8 * (h >> 1) + 2 * q4 + (h & 1);
+        const double v = scale * (h < 2 ? acc0[h] : acc1[h - 2]);
+        if (CLUSTER) to[e][r] = v;
+        else to_mem[e * n + r] = v;
       }
     }
-#pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      const int e = 8 * (h >> 1) + 2 * q4 + (h & 1);
-      const double old = CLUSTER ? cols[e][r] : __ldcg(column(rank, e) + r);
-      Gp[e][r] = old + (h < 2 ? acc0[h] : acc1[h - 2]);
+    if (!meet()) return -1;            // (this term is complete, and nobody reads the one before it any more)
+    for (int idx = threadIdx.x; idx < JG_M * n; idx += blockDim.x) {
+      const int e = idx / n, r = idx % n;
+      if (CLUSTER) {
+        cols[e][r] += to[e][r];
+      } else {
+        double* const o = column(rank, e) + r;
+        *o = __ldcg(o) + __ldcg(&to_mem[idx]);
+      }
     }
   }
-  if (!meet()) return -1;              // (nobody reads the old columns any more)
-  for (int idx = threadIdx.x; idx < JG_M * n; idx += blockDim.x) {
-    const int e = idx / n, r = idx % n;
-    if (CLUSTER) cols[e][r] = Gp[e][r];
-    else column(rank, e)[r] = Gp[e][r];
-  }
   if (!meet()) return -1;
-  return angle <= JAC_LAST_ANGLE ? 2 : 1;
+  return turn <= JAC_LAST_TURN ? 2 : 1;
 }
 
 template <bool CLUSTER, int ROWS>   // ROWS = 128 or 256 >= n
 __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
-    double* At, int n, int max_sweeps, JacobiInfo* info, int* dev_status, unsigned poll_limit) {
+    double* At, double* terms, int n, int max_sweeps, JacobiInfo* info, int* dev_status, unsigned poll_limit) {
   grid_dep_wait();
   __shared__ double part[8][3][64];
   __shared__ double G[2][JG_M][JG_P];
@@ -985,11 +1019,11 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
     if (alive) {
       mc2 = __int_as_float(*reinterpret_cast<volatile int*>(&info->max_cos2[sweep]));
       converged = mc2 < JAC_DONE_COS2;
-      if (ROWS == 128) {               // (128 columns: 449 -> 391 us in all; a step's two matrices of 256 columns do not fit beside the buffers)
+      if (ROWS == 128) {               // (128 columns: 449 -> 391 us in all; a step's three matrices of 256 columns do not fit beside the buffers)
         while (alive && !converged && mc2 < JAC_NEAR_COS2 && attempt < JAC_MAX_FINISH && refused < 3) {
           Cols const buf = reinterpret_cast<Cols>(jacobi_cols);
-          const int r = jacobi_finish<CLUSTER, ROWS>(buf + (visit & 1) * JG_M, At, n, buf + ((visit & 1) ^ 1) * JG_M, buf + 2 * JG_M,
-                                                     inv_scale * inv_scale, info, attempt++, bar, poll_limit);
+          const int r = jacobi_finish<CLUSTER, ROWS>(buf + (visit & 1) * JG_M, At, terms, n, buf + ((visit & 1) ^ 1) * JG_M, buf + 2 * JG_M,
+                                                     buf + 3 * JG_M, inv_scale * inv_scale, info, attempt++, bar, poll_limit);
           alive = r >= 0;
           converged = r == 2;
           if (r == 0) { ++refused; break; }
@@ -1541,16 +1575,17 @@ int launch_gaussian(uint64_t seed, uint64_t dc, int64_t d, int64_t r, float* S, 
 
 // Eigen-solver workspace: At n*n double | norms n double | info   (n = ell rounded up to 16)
 namespace {
-struct JacWs { double* At; double* norms; JacobiInfo* info; size_t bytes; int64_t n; };
+struct JacWs { double* At; double* norms; JacobiInfo* info; double* terms; size_t bytes; int64_t n; };
 JacWs carve_jac(void* ws, int64_t ell) {
   JacWs j;
   j.n = round_up(ell, 16);
   size_t off = 0;
   auto take = [&](size_t b) { size_t o = off; off += (b + 255) / 256 * 256; return o; };
   const size_t o1 = take(j.n * j.n * 8), o2 = take(j.n * 8), o3 = take(sizeof(JacobiInfo));
+  const size_t o4 = take(j.n <= 128 ? 2 * j.n * j.n * 8 : 0);
   char* b = static_cast<char*>(ws);
   j.At = reinterpret_cast<double*>(b + o1); j.norms = reinterpret_cast<double*>(b + o2);
-  j.info = reinterpret_cast<JacobiInfo*>(b + o3);
+  j.info = reinterpret_cast<JacobiInfo*>(b + o3); j.terms = reinterpret_cast<double*>(b + o4);
   j.bytes = off;
   return j;
 }
@@ -1626,12 +1661,12 @@ int jacobi_topk(const double* B, int64_t ldb, int64_t ell, int64_t k, float* Wse
     // one cluster on the hardware barrier (more than 8 CTAs is a cluster size the device has to
     // allow and be able to place: the occupancy query below decides), unless a test has shortened
     // the software barrier's poll limit, which only that barrier can honour.
-    void (*const on_cluster)(double*, int, int, JacobiInfo*, int*, unsigned) =
+    void (*const on_cluster)(double*, double*, int, int, JacobiInfo*, int*, unsigned) =
         n <= 128 ? jacobi_stream_kernel<true, 128> : jacobi_stream_kernel<true, 256>;
-    void (*const on_grid)(double*, int, int, JacobiInfo*, int*, unsigned) =
+    void (*const on_grid)(double*, double*, int, int, JacobiInfo*, int*, unsigned) =
         n <= 128 ? jacobi_stream_kernel<false, 128> : jacobi_stream_kernel<false, 256>;
     const unsigned threads = JS_G_THREADS + (n <= 128 ? 128 : 256);
-    const int cols_smem = (n <= 128 ? 3 : 2) * JG_M * ((n <= 128 ? 128 : 256) + 2) * 8;
+    const int cols_smem = (n <= 128 ? 4 : 2) * JG_M * ((n <= 128 ? 128 : 256) + 2) * 8;
     bool as_cluster = poll_limit == GRID_BARRIER_POLLS;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
@@ -1673,16 +1708,17 @@ int jacobi_topk(const double* B, int64_t ldb, int64_t ell, int64_t k, float* Wse
       }
     }
     if (as_cluster) {
-      PRAC_CUDA_TRY(cudaLaunchKernelEx(&cfg, on_cluster, at, ni, max_sweeps, info, dev_status, poll_limit));
+      PRAC_CUDA_TRY(cudaLaunchKernelEx(&cfg, on_cluster, at, j.terms, ni, max_sweeps, info, dev_status, poll_limit));
     } else {
-      void* sargs[] = {&at, &ni, &max_sweeps, &info, &dev_status, &poll_limit};
+      double* terms = j.terms;
+      void* sargs[] = {&at, &terms, &ni, &max_sweeps, &info, &dev_status, &poll_limit};
       static DeviceOnce grid_attr;
       if (n <= 128 && !grid_attr.done(dev)) {
         PRAC_CUDA_TRY(cudaFuncSetAttribute(on_grid, cudaFuncAttributeMaxDynamicSharedMemorySize, cols_smem));
         grid_attr.mark(dev);
       }
       PRAC_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(on_grid), dim3(grid), dim3(threads), sargs,
-                                                n <= 128 ? cols_smem : 0, stream));   // (a finishing step's two matrices)
+                                                n <= 128 ? cols_smem : 0, stream));   // (a finishing step's matrices)
     }
   } else if (gram) {
     void* gargs[] = {&at, &ni, &max_sweeps, &tol, &info, &dev_status, &poll_limit};
