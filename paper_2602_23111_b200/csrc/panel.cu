@@ -102,10 +102,14 @@ constexpr int JAC_MAX_SWEEPS = 30;
 // Sweeps that run out are an error only where a cosine of 1e-4 is left (JAC_FAIL_COS2).
 constexpr float JAC_DONE_COS2 = 1e-13f, JAC_FAIL_COS2 = 1e-8f;
 // A finishing step (jacobi_finish) is tried after a sweep that met cosines up to JAC_NEAR; it turns all columns at once where
-// no column's angles add up to more than JAC_STEP_TURN, by a rotation that is orthogonal to JAC_TURN_REST, and is the
-// last one where they add up to no more than JAC_LAST_TURN.
+// no column's angles add up to more than JAC_STEP_TURN, by a rotation that is orthogonal to JAC_TURN_REST.  The last step, like
+// the last sweep, is one that met no squared cosine above JAC_DONE_COS2.  (The angles alone say too little: two short
+// columns beside a long one keep the product of their cosines with it, however small the angles towards it are.)
+// Pairs with a squared cosine below JAC_ALONE_COS2 are left alone, as in the kernel for larger problems: 1e-9 is far below
+// what the fp32 result keeps, and below what a rounding of B in fp32 does to two columns so close that the pair would
+// still turn by a large angle.
 constexpr int JAC_MAX_FINISH = 8;
-constexpr float JAC_NEAR_COS2 = 1e-4f, JAC_STEP_TURN = 0.2f, JAC_TURN_REST = 1e-12f, JAC_LAST_TURN = 2e-5f;
+constexpr float JAC_NEAR_COS2 = 1e-4f, JAC_STEP_TURN = 0.2f, JAC_TURN_REST = 1e-10f, JAC_ALONE_COS2 = 1e-18f;
 struct JacobiInfo {
   GridBarrierState bar;             // zeroed before the launch
   int sweeps;
@@ -604,16 +608,16 @@ __device__ __forceinline__ void cluster_barrier() {
 }
 
 // A finishing step on the columns of all CTAs (16 each; up to ROWS of them), once they are nearly orthogonal:
-// the whole Gram matrix, and then either nothing more (no cosine is left above the level of fp32), or, where the
-// rotation angles T_ij = g_ij / (g_jj - g_ii) of all pairs are small, one rotation for all of them, A <- A exp(T), or nothing because
-// columns of nearly equal norm still turn by large angles.  Pairs that are orthogonal already are left alone, however
-// close their norms.  It converges as the sweeps do at the end, quadratically: of the cosines it leaves products of two.
+// the whole Gram matrix, and then, where the rotation angles T_ij = g_ij / (g_jj - g_ii) of all pairs are small, one rotation for
+// all of them, A <- A exp(T), else nothing, because columns of nearly equal norm still turn by large angles.  Pairs that
+// are orthogonal already are left alone, however close their norms.  It converges as the sweeps do at the end,
+// quadratically: of the cosines it leaves products of two.
 // T is antisymmetric to the last bit (both CTAs of a pair add the same products in the same order), so exp(T) is a rotation
 // and A = B J keeps an orthogonal J, without which orthogonal columns need not be eigenvectors: I + T alone, off by T^2, turned
 // single eigenvectors of power laws by up to 1e-3 (64 and 128 columns), exp(T) by what fp32 leaves, as the sweeps do.
-// The series is summed until what is cut off is below JAC_TURN_REST: two to nine terms A T^m / m!, some 4000 cycles
+// The series is summed until what is cut off is below JAC_TURN_REST: one to seven terms A T^m / m!, some 4000 cycles
 // each at 128 columns, after 8000 for the Gram matrix, where a sweep takes 100 000.
-// Called by all threads of all CTAs; returns 0: no step, 1: one step, 2: converged, -1: a barrier gave up.
+// Called by all threads of all CTAs; returns 0: no step, 1: one step, 2: the last step, -1: a barrier gave up.
 // CLUSTER: cols are this CTA's columns and term0, term1 two buffers for its columns of the terms, in shared memory (term0 holds
 // the Gram matrix before).  Else the columns are in At, as the next sweep's first step pairs them, the terms in terms (2 n x n), and
 // term0 holds the Gram matrix.  The norms pass through info.
@@ -680,7 +684,7 @@ __device__ __noinline__ int jacobi_finish(double (*cols)[ROWS + 2], double* At, 
       const double v = Gp[j][i], di = norms[i], dj = norms[jj];
       const float c2 = i == jj ? 0.f : static_cast<float>(v * v / (di * dj));
       double t = 0.0;
-      if (c2 > 1e-14f) {
+      if (c2 > JAC_ALONE_COS2) {
         t = v / (dj - di);
         cos2 = fmaxf(cos2, fminf(c2, 1.f));
         sum += fabsf(static_cast<float>(t));
@@ -701,7 +705,6 @@ __device__ __noinline__ int jacobi_finish(double (*cols)[ROWS + 2], double* At, 
   if (!meet()) return -1;
   cos2 = __int_as_float(*reinterpret_cast<volatile int*>(&info->fin_cos2[attempt]));
   turn = __int_as_float(*reinterpret_cast<volatile int*>(&info->fin_turn[attempt]));
-  if (cos2 < JAC_DONE_COS2) return 2;
   if (!(turn <= JAC_STEP_TURN)) return 0;
   // ---- columns of this CTA += all columns times T, times T^2 / 2, ..; a term is the product of the one before it, eight
   // rows at a time.  turn is the 1-norm of T (and, T being antisymmetric, its infinity norm), so the terms after the m-th
@@ -751,7 +754,7 @@ __device__ __noinline__ int jacobi_finish(double (*cols)[ROWS + 2], double* At, 
     }
   }
   if (!meet()) return -1;
-  return turn <= JAC_LAST_TURN ? 2 : 1;
+  return cos2 < JAC_DONE_COS2 ? 2 : 1;
 }
 
 template <bool CLUSTER, int ROWS>   // ROWS = 128 or 256 >= n
