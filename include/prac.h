@@ -98,6 +98,9 @@ void prac_debug_set_barrier_poll_limit(uint32_t polls);
  * Returns that count for the current device since the library was loaded (after waiting for the
  * device), -1 in the normal build, -2 if the count cannot be read. */
 int64_t prac_debug_bounds_violations(void);
+/* Test hook: q[i] = a[i] / b[i] for n doubles on the device, by the quotient that the Cholesky factorisation
+ * uses in place of a division (b and 1 / b normal numbers). */
+int prac_debug_quotients(const double* a, const double* b, double* q, int64_t n, void* stream);
 /* Static string for a status code. */
 const char* prac_status_string(int status);
 

@@ -46,3 +46,24 @@ def test_panel_whose_rank_ends_inside_a_block(k, rank):
     U, X64 = f64(b.get()[0]), f64(X)
     assert np.linalg.norm(U.T @ U - np.eye(k)) <= 1e-5
     assert np.linalg.norm(X64 - X64 @ U @ U.T) <= 1e-4 * np.linalg.norm(X64)
+
+
+def test_quotients_of_the_elimination_against_division():
+    # One step of the cubic iteration leaves 2^-60, its three roundings 2^-53 each with factors of one at most: two units of the
+    # last place, 2^-52 relative, of the correctly rounded quotient.  Pivots: squared norms of fp32 columns.
+    import ctypes
+    from paper_2602_23111_b200 import api
+    n = 1 << 20
+    g = torch.Generator(device="cuda")
+    g.manual_seed(9)
+    mantissa = 1 + torch.rand(n, generator=g, device="cuda", dtype=torch.float64)
+    mantissa[:64] = 1 + torch.arange(64, device="cuda", dtype=torch.float64) * 2.0 ** -52
+    mantissa[64:128] = 2 - torch.arange(1, 65, device="cuda", dtype=torch.float64) * 2.0 ** -52
+    exponent = torch.randint(-300, 280, (n,), generator=g, device="cuda")
+    b = torch.ldexp(mantissa, exponent)
+    a = torch.randn(n, generator=g, device="cuda", dtype=torch.float64) * torch.ldexp(torch.ones_like(b), exponent)
+    q = torch.empty_like(a)
+    p = lambda t: ctypes.c_void_p(t.data_ptr())
+    assert api.lib.prac_debug_quotients(p(a), p(b), p(q), n, ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)) == api.PRAC_OK
+    exact = a / b
+    assert float(((q - exact) / exact).abs().max()) <= 2 * 2.0 ** -52
