@@ -11,6 +11,7 @@
 
 #include "internal.h"
 #include "per_device.h"
+#include "ptx.cuh"
 
 namespace prac {
 namespace {
@@ -774,6 +775,7 @@ __global__ void __launch_bounds__(CHOL_MAIN + CHOL_HELP) chol_inv_kernel(const C
 // ------------------------------------------------------------------ the same on one cluster, up to 16 blocks of columns
 constexpr int CC_MAX = 16;                       // blocks of columns = CTAs of the cluster
 constexpr int CC_GROUPS = 2;                     // groups of 256 threads in a CTA
+constexpr uint64_t CC_WAIT_NS = 2000000000ull;   // what a wait may last
 // What the CTAs tell one another: barriers in the shared memory of the CTA that waits, each for one event.
 struct ChainWords {
   uint64_t row[CC_MAX][CC_MAX];   // [c][x]: block (c, x) of R is final in CTA x
@@ -795,8 +797,10 @@ struct ChainWords {
 // The chain of diagonal blocks is what this costs.  A factorisation whose CTAs met through flags in global memory
 // (chol_inv_kernel) took 13 400 cycles a block, most of them the way of a block through L2 and back.
 //
-// Every wait on another CTA is bounded; a CTA that gives up tells the others, and all of them meet at the
-// cluster's barrier before any leaves, so that nobody's shared memory goes away under a reader.
+// Every wait on another CTA is bounded, in polls and in time (a poll may itself block for a while); a CTA that gives up tells the
+// others.  Then every CTA that has not sent its rows of R_cc^-T sends zeros in their place, every CTA waits for all the rows
+// that it is to receive (that wait ends, since they have all been sent; it is bounded too), and all meet at the cluster's
+// barrier before any leaves: nobody's shared memory goes away under a reader or under a store on its way.
 //
 // A CTA walks most of this code once, with its instructions not in the SM's cache yet (see sub_chol).  So every CTA
 // first runs the chain's part of a step on an identity, before it waits for the kernel that makes G.
@@ -814,21 +818,29 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
   Blk const W = block(nb + 1), Dprev = block(nb + 2), Dfar = block(nb + 3);
   Blk const stage = block(nb + 4 + group);
   Blk const E = block(nb + 4);                                // (group 0's: it factors or it fetches)
-  bool fail = false;
+  bool fail = false, sent = false;               // sent: this CTA's rows are on their way to the next one
 
+  // After a poll in vain: whether to give up, because this wait has lasted too long (the others are told) or another gave up.
+  auto gives_up = [&](unsigned polls, uint64_t& since) {
+    bool late = polls >= a.poll_limit;
+    if ((polls & 63u) == 0u) {
+      if (*reinterpret_cast<volatile int*>(&words.abort)) return true;
+      const uint64_t now = ptx::globaltimer_ns();
+      if (since == 0) since = now;
+      late = late || now - since > CC_WAIT_NS;
+    }
+    if (late)
+      for (int x = 0; x < nb; ++x) cluster_st_flag(cluster_addr(&words.abort, x), 1);
+    return late;
+  };
   // Every lane waits for a barrier of its own (or none): cheap polls, and one that acquires (it takes 400 cycles) once
   // all of them are through.  Where a lane gives up the caller carries on with what it has, until the CTA next meets and leaves together.
   auto wait_for = [&](uint64_t* bar) {
     if (bar != nullptr && !fail) {
       unsigned polls = 0;
-      while (!cluster_try_wait(bar)) {
-        if (++polls >= a.poll_limit) {
-          fail = true;
-          for (int x = 0; x < nb; ++x) cluster_st_flag(cluster_addr(&words.abort, x), 1);
-          break;
-        }
-        if ((polls & 63u) == 0u && *reinterpret_cast<volatile int*>(&words.abort)) { fail = true; break; }
-      }
+      uint64_t since = 0;
+      while (!cluster_try_wait(bar))
+        if (gives_up(++polls, since)) { fail = true; break; }
     }
     __syncwarp();
     if (bar != nullptr && !fail) (void)cluster_try_wait_acquire(bar);
@@ -838,15 +850,17 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
   auto wait_rows = [&](uint64_t* bar) {
     if (lane == 0 && !fail) {
       unsigned polls = 0;
-      while (!cluster_try_wait_rows(bar)) {
-        if (++polls >= a.poll_limit || ((polls & 63u) == 0u && *reinterpret_cast<volatile int*>(&words.abort))) {
-          fail = true;
-          for (int x = 0; x < nb; ++x) cluster_st_flag(cluster_addr(&words.abort, x), 1);
-          break;
-        }
-      }
+      uint64_t since = 0;
+      while (!cluster_try_wait_rows(bar))
+        if (gives_up(++polls, since)) { fail = true; break; }
     }
     __syncwarp();
+  };
+  // Rows 8 s .. 8 s + 7 of R_qq^-T up to the diagonal tile, to the next CTA (128 threads): rows(r, cc) is the pair at column cc.
+  const uint32_t far = q + 1 < nb ? cluster_addr(Dprev, q + 1) : 0u, far_bar = q + 1 < nb ? cluster_addr(words.band, q + 1) : 0u;
+  auto send_rows = [&](int s, auto rows) {
+    const int i = tid & 127, r = 8 * s + (i & 7), cc = 2 * (i >> 3);
+    if (cc < 8 * (s + 1)) cluster_st_async(far + (r * CP + cc) * 8, rows(r, cc), far_bar + 8 * s);
   };
   // the pairs (row, 2 columns) of a block that a thread of a group moves
   auto pull = [&](uint32_t from, double2 (&v)[2]) {
@@ -967,10 +981,8 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
       if (group == 0) {
         Blk const Lin = dry ? block(nb) : inv(q);
         const bool next = !dry && q + 1 < nb;
-        const uint32_t far = next ? cluster_addr(Dprev, q + 1) : 0u, far_bar = next ? cluster_addr(words.band, q + 1) : 0u;
         blk_chol_inv(CholBlock{Dq, Lin, E, W, guard}, dry ? nullptr : a.dev_status, a.flag_bit, [&](int s) {
-          const int i = tid & 127, r = 8 * s + (i & 7), cc = 2 * (i >> 3);
-          if (next && cc < 8 * (s + 1)) cluster_st_async(far + (r * CP + cc) * 8, *reinterpret_cast<const double2*>(&Lin[r][cc]), far_bar + 8 * s);
+          if (next) send_rows(s, [&](int r, int cc) { return *reinterpret_cast<const double2*>(&Lin[r][cc]); });
         });
       } else if (!dry && c >= 0) {
         bar_sync(2, 256);                        // (Rbuf is complete)
@@ -981,6 +993,7 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
         bar_sync(2, 256);
         if (warp == 15 && lane < nb && lane != q) cluster_bar_arrive(cluster_addr(&words.row[c][q], lane));
       }
+      sent = !dry;
       // every thread leaves here if one has given up
       if (__syncthreads_or(fail)) { fail = true; break; }
       if (!dry && warp == 8 && lane < nb && lane != q) cluster_bar_arrive(cluster_addr(&words.diag[q], lane));
@@ -1038,10 +1051,20 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
       __syncthreads();
     }
   }
-  if (fail && lane == 0 && a.dev_status) atomicOr(a.dev_status, DEV_WAIT_EXPIRED);
+  fail = __syncthreads_or(fail) != 0;
+  if (fail) {
+    if (tid == 0 && a.dev_status) atomicOr(a.dev_status, DEV_WAIT_EXPIRED);
+    if (!sent && q + 1 < nb && tid < 128)
+      for (int s = 0; s < CB / 8; ++s) send_rows(s, [](int, int) { return make_double2(0.0, 0.0); });
+    if (tid == 0 && q > 0) {
+      const uint64_t since = ptx::globaltimer_ns();
+      for (int s = 0; s < CB / 8; ++s)
+        while (!cluster_try_wait_rows(&words.band[s]) && ptx::globaltimer_ns() - since <= 2 * CC_WAIT_NS) {}
+    }
+    __syncthreads();
+  }
   cluster_arrive();
   cluster_wait();
-  if (fail) for (int i = 0; i < 64; ++i) __nanosleep(1000);      // rows may still be on their way from the CTA before
 }
 
 size_t chol_cluster_smem(int nb) {

@@ -25,8 +25,8 @@ def f64(t):
 
 
 def test_grid_barrier_gives_up_reports_timeout_and_the_basis_stays_usable(api):
-    # panel of 96 columns: the Cholesky kernel runs on 3 CTAs and the eigen-solver on 4, so their
-    # grid barriers really wait; with a poll limit of 1 the first CTA to arrive gives up at once
+    # panel of 96 columns: the Cholesky kernel runs on a cluster of 3 CTAs and the eigen-solver on 4 (with such a
+    # limit on its grid barrier), so they really wait; with a poll limit of 1 the first CTA to arrive gives up at once
     N, d, k, r = 2048, 512, 64, 64
     X = inputs.make_planted(N, d, k, gap=4.0, seed=201, dtype="bf16")
     Xd = X.to("cuda", torch.bfloat16)
@@ -44,6 +44,26 @@ def test_grid_barrier_gives_up_reports_timeout_and_the_basis_stays_usable(api):
     assert orc.projector_distance(f64(U), orc.principal_basis(f64(X), k)) <= 1e-3
     Q0 = orc.random_basis(f64(U), orc.gaussian_draw(3, 1, d, r))
     assert np.linalg.norm(f64(Q) - Q0) / np.sqrt(r) <= 1e-4
+
+
+@pytest.mark.parametrize("r", [33, 96, 256, 320, 512])
+def test_a_factorisation_that_gives_up_leaves_nothing_behind(api, r):
+    # Without a principal part the draw has no bounded wait but those of the factorisation (a cluster of 2 to 16 CTAs
+    # that store rows into one another's shared memory).  Every CTA waits for the rows that were sent to it before it
+    # leaves, also after giving up: what runs next on the same SMs gets the bits that it gets without such a call before it.
+    b = api.Basis(2 * r + 19, 0, r, torch.float32)
+    b.draw_random(seed=4, draw_counter=2)
+    assert b.status() == api.PRAC_OK
+    good = b.projection()[0].clone()
+    for _ in range(10):
+        api.lib.prac_debug_set_barrier_poll_limit(1)
+        try:
+            b.draw_random(seed=4, draw_counter=2)
+        finally:
+            api.lib.prac_debug_set_barrier_poll_limit(0)
+        b.draw_random(seed=4, draw_counter=2)
+        assert b.status() == api.PRAC_ETIMEOUT          # (the first of the two)
+        assert torch.equal(b.projection()[0], good)
 
 
 def test_status_word_decoding(api):
