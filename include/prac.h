@@ -87,11 +87,13 @@ int prac_version(void);
 /* Number of CUDA kernels this library has launched so far in this process (host counter,
  * all entry points together).  Lets a caller assert that the CUDA path is what ran. */
 uint64_t prac_kernel_launches(void);
-/* Test hook: poll limit of the bounded grid barriers inside the cooperative kernels of the fit
- * (Cholesky factorisation, eigen-solver).  A limit of 1 makes the first CTA to reach a barrier
- * give up at once: every CTA then leaves through its normal exit and prac_device_status()
- * returns PRAC_ETIMEOUT; 0 restores the default (about 4 million polls).  Process-wide. */
+/* Test hook: poll limit of the bounded waits between the CTAs of a Cholesky factorisation and of the
+ * eigen-solver's grid barrier (any limit but the default selects its kernel with that barrier).  A limit of 1
+ * makes the first CTA that has to wait give up at once: every CTA then leaves through its normal exit and
+ * prac_device_status() returns PRAC_ETIMEOUT; 0 restores the default (about 4 million polls).  Process-wide. */
 void prac_debug_set_barrier_poll_limit(uint32_t polls);
+/* Test hook: the same for the eigen-solver's waits for columns where its CTAs are a cluster. */
+void prac_debug_set_column_poll_limit(uint32_t polls);
 /* Bounds-checking build (libprac_dbg.so, compiled with -DPRAC_DEBUG_BOUNDS; it stands in for a memory
  * checker where none can be run): the kernels that compute their own global-memory indices check
  * each one against the extent of its buffer, count the ones outside and skip those accesses.

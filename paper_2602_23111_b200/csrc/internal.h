@@ -21,6 +21,8 @@ enum : int {
 // Poll limit of the grid barriers of the cooperative kernels (default GRID_BARRIER_POLLS; a test
 // hook lowers it to make a barrier give up).
 unsigned barrier_poll_limit();
+// Poll limit of the eigen-solver's waits for columns inside a cluster (same default, a hook of its own).
+unsigned column_poll_limit();
 
 // Number of kernels this library has launched in the process (reported by
 // prac_kernel_launches so callers can check that the CUDA path is the one that ran).

@@ -7,6 +7,7 @@
 #include "grid_barrier.cuh"
 #include "internal.h"
 #include "per_device.h"
+#include "ptx.cuh"
 
 namespace prac {
 namespace {
@@ -118,6 +119,7 @@ struct JacobiInfo {
   int max_cos2[JAC_MAX_SWEEPS];     // largest squared cosine rotated away in each sweep (float bits)
   int fin_cos2[JAC_MAX_FINISH], fin_turn[JAC_MAX_FINISH];    // the same, and the largest sum of a column's angles, of each finishing step
   double norms[128];                // squared norms of the columns in a finishing step
+  int late[JAC_MAX_SWEEPS];         // a wait for a visit's columns gave up in this sweep
 };
 
 // Pair i of step `step` of the round-robin schedule on m (even) items, as p < q.
@@ -537,11 +539,15 @@ __global__ void __launch_bounds__(256) jacobi_gram_kernel(double* At, int n, int
 // later: the columns that this CTA needed meanwhile came from its two neighbours' visit after they had read it.  Only at the
 // end of a sweep do the CTAs meet at the hardware cluster barrier: every CTA runs the same
 // number of steps and sweeps (the stopping test reads values that are final before the barrier it
-// follows), so each barrier is reached by all of them.  Otherwise a cooperative launch with the
-// bounded software barrier, the columns in global memory.
+// follows), so each barrier is reached by all of them.  A wait for columns is bounded, in polls and in time (a poll may itself
+// block for a while).  A CTA that gives up sends its columns, such as they are, to the end of the sweep, so that nobody
+// waits for them in vain, but waits no more and arms its barriers no more (the one it gave up on is still in a phase that
+// must not be armed twice); at the end of the sweep all of them stop, and it waits for every byte that was sent to it before
+// it leaves.  Otherwise a cooperative launch with the bounded software barrier, the columns in global memory.
 constexpr int JS_G_THREADS = 256;      // form the Gram matrix; the first 64 walk the rounds
 constexpr int JS_R_THREADS = 64;
 constexpr int JS_MAX_ROWS = 256;
+constexpr uint64_t JS_WAIT_NS = 2000000000ull;   // what a wait for columns may last
 // (the warp has to be converged at these barriers)
 __device__ __forceinline__ void named_sync(int id, int threads) {
   __syncwarp();
@@ -761,6 +767,7 @@ template <bool CLUSTER, int ROWS>   // ROWS = 128 or 256 >= n
 __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
     double* At, double* terms, int n, int max_sweeps, JacobiInfo* info, int* dev_status, unsigned poll_limit) {
   grid_dep_wait();
+  constexpr unsigned VISIT_BYTES = JG_M * ROWS * 8;   // what a CTA receives per visit
   __shared__ double part[8][3][64];
   __shared__ double G[2][JG_M][JG_P];
   __shared__ float2 coef[JG_M][JG_B];            // every round of the visit, per pair: c, o
@@ -781,20 +788,21 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
   float mc2 = 1.f;
   int sweep = 0;
   unsigned visit = 0;
-  bool late = false;
+  bool late = false;                             // (lane 0 of each warp)
+  unsigned late_visit = 0;                       // the visit after which it gave up
+  __shared__ int gave_up;
   int attempt = 0, refused = 0;
   if (CLUSTER) {
-    if (threadIdx.x < 2)
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(&arrived[threadIdx.x]))) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (threadIdx.x < 2) ptx::mbar_init(&arrived[threadIdx.x], 1);
+    if (threadIdx.x == 0) gave_up = 0;
+    ptx::fence_mbar_init();
     int I, J;
     rr_pair(nb, 0, blockIdx.x, I, J);
     for (int e = warp; e < JG_M; e += (JS_G_THREADS + ROWS) / 32)
       for (int r = lane; r < ROWS; r += 32)
         reinterpret_cast<Cols>(jacobi_cols)[e][r] = r < n ? __ldcg(At + static_cast<long long>((e < b ? I * b + e : J * b + e - b)) * n + r) : 0.0;
     __syncthreads();
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");      // (every CTA of the cluster has started)
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_barrier();                 // (every CTA of the cluster has started)
   }
   for (; alive && sweep < max_sweeps && !converged; ++sweep) {
     for (int step = 0; alive && step < nb - 1; ++step) {
@@ -804,8 +812,7 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
       double* const colJ = At + static_cast<long long>(J) * b * n;
       const unsigned turn = visit & 1;
       Cols const here = reinterpret_cast<Cols>(jacobi_cols) + turn * JG_M, there = reinterpret_cast<Cols>(jacobi_cols) + (turn ^ 1) * JG_M;
-      if (CLUSTER && threadIdx.x == 0)
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(&arrived[turn ^ 1]))), "n"(JG_M * ROWS * 8) : "memory");
+      if (CLUSTER && threadIdx.x == 0 && !late) ptx::mbar_arrive_expect_tx(&arrived[turn ^ 1], VISIT_BYTES);
       const bool full = step == 0;
       const int rounds = full ? JG_M - 1 : JG_B;
       if (row_thread) {
@@ -997,28 +1004,30 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
         // work: a round 457 -> 540 cycles)
         __syncthreads();
         if (lane == 0 && !late) {
-          const uint32_t bar_addr = static_cast<uint32_t>(__cvta_generic_to_shared(&arrived[turn ^ 1]));
-          unsigned polls = 0, ok = 0;
-          while (true) {
-            asm volatile(
-                "{\n\t.reg .pred P;\n\t"
-                "mbarrier.try_wait.parity.shared::cta.b64 P, [%1], %2;\n\t"
-                "selp.b32 %0, 1, 0, P;\n\t}"
-                : "=r"(ok) : "r"(bar_addr), "r"((visit >> 1) & 1u) : "memory");
-            if (ok) break;
-            if (++polls >= poll_limit) { late = true; break; }    // (it carries on with what it has: everybody meets below)
+          unsigned polls = 0;
+          uint64_t since = 0;
+          while (!ptx::mbar_try_wait(&arrived[turn ^ 1], (visit >> 1) & 1u)) {
+            late = ++polls >= poll_limit;
+            if ((polls & 63u) == 0u) {
+              const uint64_t now = ptx::globaltimer_ns();
+              if (since == 0) since = now;
+              late = late || now - since > JS_WAIT_NS || *reinterpret_cast<volatile int*>(&gave_up);
+            }
+            if (!late) continue;
+            *reinterpret_cast<volatile int*>(&gave_up) = 1;
+            atomicOr(&info->late[sweep], 1);
+            late_visit = visit;
+            break;
           }
         }
         __syncwarp();
         ++visit;
-        if (step == nb - 2) {          // the sweep's largest cosine is complete
-          asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-          asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-        }
+        if (step == nb - 2) cluster_barrier();         // the sweep's largest cosine is complete
       } else {
         alive = grid_barrier(&info->bar, ++bar * nctas, poll_limit);
       }
     }
+    if (CLUSTER) alive = *reinterpret_cast<volatile int*>(&info->late[sweep]) == 0;     // (final before that barrier)
     if (alive) {
       mc2 = __int_as_float(*reinterpret_cast<volatile int*>(&info->max_cos2[sweep]));
       converged = mc2 < JAC_DONE_COS2;
@@ -1034,13 +1043,27 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
       }
     }
   }
+  if (CLUSTER && late && threadIdx.x == 0) {
+    // what has been sent here since the wait that gave up: the rest of that visit's columns, for which the barrier was armed,
+    // and those of the visits up to the end of the sweep (all sent by now), for which it was not; the other barrier's likewise
+    const uint64_t since = ptx::globaltimer_ns();
+    auto drained = [&](unsigned v) {
+      while (!ptx::mbar_try_wait(&arrived[(v & 1) ^ 1], (v >> 1) & 1u))
+        if (ptx::globaltimer_ns() - since > JS_WAIT_NS) return false;
+      return true;
+    };
+    bool ok = drained(late_visit);
+    for (unsigned v = late_visit + 1; ok && v <= late_visit + 2 && v < visit; ++v) {
+      ptx::mbar_arrive_expect_tx(&arrived[(v & 1) ^ 1], (visit - v + 1) / 2 * VISIT_BYTES);
+      ok = drained(v);
+    }
+  }
   if (CLUSTER) {                       // (the columns lie as the next sweep's first step has them)
     int I, J;
     rr_pair(nb, 0, blockIdx.x, I, J);
     for (int e = warp; e < JG_M; e += (JS_G_THREADS + ROWS) / 32)
       for (int r = lane; r < n; r += 32)
         At[static_cast<long long>((e < b ? I * b + e : J * b + e - b)) * n + r] = (reinterpret_cast<Cols>(jacobi_cols) + (visit & 1) * JG_M)[e][r];
-    if (late && dev_status) atomicOr(dev_status, DEV_WAIT_EXPIRED);
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     info->sweeps = sweep;
@@ -1711,7 +1734,7 @@ int jacobi_topk(const double* B, int64_t ldb, int64_t ell, int64_t k, float* Wse
       }
     }
     if (as_cluster) {
-      PRAC_CUDA_TRY(cudaLaunchKernelEx(&cfg, on_cluster, at, j.terms, ni, max_sweeps, info, dev_status, poll_limit));
+      PRAC_CUDA_TRY(cudaLaunchKernelEx(&cfg, on_cluster, at, j.terms, ni, max_sweeps, info, dev_status, column_poll_limit()));
     } else {
       double* terms = j.terms;
       void* sargs[] = {&at, &terms, &ni, &max_sweeps, &info, &dev_status, &poll_limit};

@@ -36,6 +36,8 @@ static std::atomic<uint64_t> g_launches{0};
 void count_launch(int n) { g_launches.fetch_add(static_cast<uint64_t>(n), std::memory_order_relaxed); }
 static std::atomic<unsigned> g_barrier_polls{1u << 22};
 unsigned barrier_poll_limit() { return g_barrier_polls.load(std::memory_order_relaxed); }
+static std::atomic<unsigned> g_column_polls{1u << 22};
+unsigned column_poll_limit() { return g_column_polls.load(std::memory_order_relaxed); }
 }  // namespace prac
 
 namespace {
@@ -263,6 +265,10 @@ int64_t prac_debug_bounds_violations(void) {
 
 void prac_debug_set_barrier_poll_limit(uint32_t polls) {
   prac::g_barrier_polls.store(polls == 0 ? (1u << 22) : polls, std::memory_order_relaxed);
+}
+
+void prac_debug_set_column_poll_limit(uint32_t polls) {
+  prac::g_column_polls.store(polls == 0 ? (1u << 22) : polls, std::memory_order_relaxed);
 }
 
 const char* prac_status_string(int status) {

@@ -66,6 +66,30 @@ def test_a_factorisation_that_gives_up_leaves_nothing_behind(api, r):
         assert torch.equal(b.projection()[0], good)
 
 
+@pytest.mark.parametrize("d,k", [(48, 24), (128, 64), (144, 72), (250, 125)])
+def test_an_eigen_solve_that_gives_up_leaves_nothing_behind(api, d, k):
+    # The eigen-solver's CTAs (3 to 16) store columns into one another's shared memory.  With a limit of one poll nearly
+    # every wait gives up in the first sweep; all CTAs stop at its end, each after everything sent to it has arrived.
+    g = torch.Generator(device="cuda")
+    g.manual_seed(8)
+    V = torch.linalg.qr(torch.randn(d, d, generator=g, device="cuda", dtype=torch.float64))[0]
+    C = ((V * torch.arange(1, d + 1, device="cuda", dtype=torch.float64) ** -1.3) @ V.t()).float().contiguous()
+    b = api.Basis(d, k, 0, torch.float32, oversample=d - k)
+    b.fit_principal_gram(C, seed=1)
+    assert b.status() == api.PRAC_OK
+    good = b.get()[0].clone()
+    for _ in range(10):
+        api.lib.prac_debug_set_column_poll_limit(1)
+        try:
+            b.fit_principal_gram(C, seed=1)
+        finally:
+            api.lib.prac_debug_set_column_poll_limit(0)
+        assert b.fit_report(1)["jacobi_sweeps"] == 1
+        b.fit_principal_gram(C, seed=1)
+        assert b.status() == api.PRAC_ETIMEOUT          # (the first of the two)
+        assert torch.equal(b.get()[0], good)
+
+
 def test_status_word_decoding(api):
     # the first four bytes of the basis storage are the device status word; written here from the
     # host side (a plain copy) to check how prac_device_status maps its bits and that it clears them.
