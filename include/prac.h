@@ -94,6 +94,9 @@ uint64_t prac_kernel_launches(void);
 void prac_debug_set_barrier_poll_limit(uint32_t polls);
 /* Test hook: the same for the eigen-solver's waits for columns where its CTAs are a cluster. */
 void prac_debug_set_column_poll_limit(uint32_t polls);
+/* Test hook: on != 0 makes every Cholesky factorisation take the cooperative kernel, which otherwise serves panels of more
+ * than 512 columns and devices that cannot place the cluster.  Process-wide. */
+void prac_debug_force_cooperative_cholesky(int32_t on);
 /* Bounds-checking build (libprac_dbg.so, compiled with -DPRAC_DEBUG_BOUNDS; it stands in for a memory
  * checker where none can be run): the kernels that compute their own global-memory indices check
  * each one against the extent of its buffer, count the ones outside and skip those accesses.

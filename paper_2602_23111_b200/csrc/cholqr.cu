@@ -1087,17 +1087,14 @@ void chol_cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2]
   cfg.numAttrs = 2;
 }
 
-// Whether the current device can place a cluster of nb CTAs of chol_cluster_kernel (asked once per device and size).
-bool chol_cluster_fits(int nb) {
-  if (nb < 1 || nb > CC_MAX) return false;
-  static DeviceValue known[CC_MAX + 1];          // 1: no, 2: yes
+// Whether a cluster of nb CTAs of chol_cluster_kernel can be placed where this stream's kernels run.  Asked for every
+// launch (0.3 us), as what a process may use can shrink; where the answer is no, chol_inv_kernel serves.
+bool chol_cluster_fits(int nb, cudaStream_t stream) {
+  if (nb < 1 || nb > CC_MAX || cooperative_cholesky_forced()) return false;
   static DeviceOnce attrs;
   int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess) { (void)cudaGetLastError(); return false; }
-  const int v = known[nb].get(dev);
-  if (v != 0) return v == 2;
-  bool ok = true;
-  if (!attrs.done(dev)) {
+  bool ok = cudaGetDevice(&dev) == cudaSuccess;
+  if (ok && !attrs.done(dev)) {
     ok = cudaFuncSetAttribute(chol_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               static_cast<int>(chol_cluster_smem(CC_MAX))) == cudaSuccess &&
          cudaFuncSetAttribute(chol_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
@@ -1106,12 +1103,11 @@ bool chol_cluster_fits(int nb) {
   if (ok) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
-    chol_cluster_config(cfg, attr, nb, nullptr);
+    chol_cluster_config(cfg, attr, nb, stream);
     int clusters = 0;
     ok = cudaOccupancyMaxActiveClusters(&clusters, chol_cluster_kernel, &cfg) == cudaSuccess && clusters >= 1;
   }
   if (!ok) (void)cudaGetLastError();
-  known[nb].set(dev, ok ? 2 : 1);
   return ok;
 }
 
@@ -1143,32 +1139,33 @@ void atb_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2], int til
 // Slices of the rows = CTAs of a tile's cluster: what lets the busiest SM go through the fewest chunks of 16 rows, two
 // chunks' time for every doubling (the sum over the slices).  Clusters do not fill every SM before one of them takes a
 // second CTA: 15 clusters of 8 ran side by side (2048 x 320 symmetric, 17 us), 16 did not (2048 x 256 by 256, 26 us).  16 is
-// more than the portable cluster size: only where the device can place it.
-int atb_slices(int tiles, int64_t d) {
-  static DeviceValue wide;                       // 1: no, 2: yes
+// more than the portable cluster size.  Whether the cluster can be placed is asked for every launch (see chol_cluster_fits).
+int atb_slices(int tiles, int64_t d, cudaStream_t stream) {
+  static DeviceOnce wide;
   int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess) { (void)cudaGetLastError(); return 8; }
-  int w = wide.get(dev);
-  if (w == 0) {
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attr[2];
-    atb_config(cfg, attr, 1, 16, nullptr);
-    int clusters = 0;
-    const bool ok = cudaFuncSetAttribute(atb_f64_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-                    cudaOccupancyMaxActiveClusters(&clusters, atb_f64_kernel, &cfg) == cudaSuccess && clusters >= 1;
-    if (!ok) (void)cudaGetLastError();
-    w = ok ? 2 : 1;
-    wide.set(dev, w);
+  bool ok = cudaGetDevice(&dev) == cudaSuccess;
+  if (ok && !wide.done(dev)) {
+    ok = cudaFuncSetAttribute(atb_f64_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    if (ok) wide.mark(dev);
   }
+  if (!ok) (void)cudaGetLastError();           // (then 16 cannot be placed)
   tc_init();
   const int sms = tc_num_sms() > 0 ? tc_num_sms() : 148;
   int best = 1;
   long long least = -1;
-  for (int s = 1, doublings = 0; s <= (w == 2 ? 16 : 8); s *= 2, ++doublings) {
+  for (int s = 1, doublings = 0; s <= 16; s *= 2, ++doublings) {
     const int room = s <= 4 ? sms : (s == 8 ? sms * 13 / 16 : sms * 3 / 4);
     const long long per_sm = (static_cast<long long>(tiles) * s + room - 1) / room;
     const long long cost = per_sm * ((d + AT_K * s - 1) / (AT_K * s)) + 2 * doublings;
     if (least < 0 || cost < least) { least = cost; best = s; }
+  }
+  for (; best > 1; best /= 2) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    atb_config(cfg, attr, tiles, best, stream);
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, atb_f64_kernel, &cfg) == cudaSuccess && clusters >= 1) break;
+    (void)cudaGetLastError();
   }
   return best;
 }
@@ -1202,7 +1199,7 @@ int atb_f64(const float* A, int64_t lda, const float* B, int64_t ldb, int64_t d,
   const int tiles = symmetric ? g.tiles_n * (g.tiles_n + 1) / 2 : tiles_m * g.tiles_n;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
-  atb_config(cfg, attr, tiles, atb_slices(tiles, d), stream);
+  atb_config(cfg, attr, tiles, atb_slices(tiles, d, stream), stream);
   PRAC_CUDA_TRY(cudaLaunchKernelEx(&cfg, atb_f64_kernel, g));
   count_launch();
   return PRAC_OK;
@@ -1276,7 +1273,7 @@ int cholqr_pass(const float* Vin, int64_t ldin, float* Vout, int64_t ldout, int6
   const bool tensor = run_if_mask == 0 && c.tensor && tc_init() == PRAC_OK && aligned16(Vout) && (ldout % 4) == 0;
   a.Rt3 = tensor ? c.Rt3 : nullptr;
   a.kp = static_cast<int>(c.kp);
-  if (chol_cluster_fits(a.nb)) {
+  if (chol_cluster_fits(a.nb, stream)) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     chol_cluster_config(cfg, attr, a.nb, stream);

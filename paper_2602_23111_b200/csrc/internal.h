@@ -23,6 +23,8 @@ enum : int {
 unsigned barrier_poll_limit();
 // Poll limit of the eigen-solver's waits for columns inside a cluster (same default, a hook of its own).
 unsigned column_poll_limit();
+// Whether a test asks for the cooperative Cholesky kernel where the cluster would serve.
+bool cooperative_cholesky_forced();
 
 // Number of kernels this library has launched in the process (reported by
 // prac_kernel_launches so callers can check that the CUDA path is the one that ran).

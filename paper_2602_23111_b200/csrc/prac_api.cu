@@ -37,6 +37,8 @@ void count_launch(int n) { g_launches.fetch_add(static_cast<uint64_t>(n), std::m
 static std::atomic<unsigned> g_barrier_polls{1u << 22};
 unsigned barrier_poll_limit() { return g_barrier_polls.load(std::memory_order_relaxed); }
 static std::atomic<unsigned> g_column_polls{1u << 22};
+static std::atomic<int> g_cooperative_cholesky{0};
+bool cooperative_cholesky_forced() { return g_cooperative_cholesky.load(std::memory_order_relaxed) != 0; }
 unsigned column_poll_limit() { return g_column_polls.load(std::memory_order_relaxed); }
 }  // namespace prac
 
@@ -269,6 +271,10 @@ void prac_debug_set_barrier_poll_limit(uint32_t polls) {
 
 void prac_debug_set_column_poll_limit(uint32_t polls) {
   prac::g_column_polls.store(polls == 0 ? (1u << 22) : polls, std::memory_order_relaxed);
+}
+
+void prac_debug_force_cooperative_cholesky(int32_t on) {
+  prac::g_cooperative_cholesky.store(on, std::memory_order_relaxed);
 }
 
 const char* prac_status_string(int status) {

@@ -34,6 +34,26 @@ def test_random_basis_is_the_unique_qr_factor(r):
     assert np.array_equal(f64(b.projection()[0]), Q)          # sums in a fixed order, whoever is first
 
 
+@pytest.mark.parametrize("r", [1, 8, 31, 32, 33, 64, 65, 97, 257, 320, 512])
+def test_cooperative_kernel_serves_where_no_cluster_can_be_placed(r):
+    # whether the cluster fits is asked for every launch: where it does not, the kernel for more than 512 columns takes over
+    from paper_2602_23111_b200 import api
+    d = max(256, 2 * r + 19)
+    b = api.Basis(d, 0, r, torch.float32)
+    api.lib.prac_debug_force_cooperative_cholesky(1)
+    try:
+        b.draw_random(seed=11, draw_counter=5)
+        Q = f64(b.projection()[0])
+        b.draw_random(seed=11, draw_counter=5)
+        assert b.status() == api.PRAC_OK
+    finally:
+        api.lib.prac_debug_force_cooperative_cholesky(0)
+    assert np.array_equal(f64(b.projection()[0]), Q)
+    Q0 = orc.random_basis(np.zeros((d, 0)), orc.gaussian_draw(11, 5, d, r))
+    assert np.max(np.linalg.norm(Q - Q0, axis=0)) <= 1e-4
+    assert np.linalg.norm(Q.T @ Q - np.eye(r)) <= max(1e-5, 2e-5 * r / 512)
+
+
 @pytest.mark.parametrize("k, rank", [(256, 100), (128, 33), (64, 64)])
 def test_panel_whose_rank_ends_inside_a_block(k, rank):
     # pivots are replaced from column `rank` on, in every block after it; the extra pass makes the rest orthonormal
