@@ -106,6 +106,10 @@ int64_t prac_debug_bounds_violations(void);
 /* Test hook: q[i] = a[i] / b[i] for n doubles on the device, by the quotient that the Cholesky factorisation
  * uses in place of a division (b and 1 / b normal numbers). */
 int prac_debug_quotients(const double* a, const double* b, double* q, int64_t n, void* stream);
+/* Test hook: one Cholesky-QR pass, Q = V R^-1 for contiguous fp32 panels of d rows and n columns (R^T R = V^T V).  ws is at least
+ * prac_debug_cholqr_ws_bytes(d, n) bytes, 256-byte aligned; a bad pivot sets bit 0 of the device word. */
+size_t prac_debug_cholqr_ws_bytes(int64_t d, int64_t n);
+int prac_debug_cholqr(const float* V, float* Q, int64_t d, int64_t n, void* ws, size_t ws_bytes, int32_t* word, void* stream);
 /* Static string for a status code. */
 const char* prac_status_string(int status);
 

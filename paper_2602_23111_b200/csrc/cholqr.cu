@@ -1413,3 +1413,9 @@ extern "C" int prac_debug_quotients(const double* a, const double* b, double* q,
   PRAC_CUDA_TRY(cudaGetLastError());
   return PRAC_OK;
 }
+
+extern "C" size_t prac_debug_cholqr_ws_bytes(int64_t d, int64_t n) { return d > 0 && n > 0 ? prac::cholqr_ws_bytes(n, d) : 0; }
+extern "C" int prac_debug_cholqr(const float* V, float* Q, int64_t d, int64_t n, void* ws, size_t ws_bytes, int32_t* word, void* stream) {
+  if (!V || !Q || !ws || !word || d <= 0 || n <= 0) return PRAC_EINVAL;
+  return prac::cholqr_pass(V, n, Q, n, d, n, ws, ws_bytes, word, prac::DEV_CHOL_PIVOT, static_cast<cudaStream_t>(stream));
+}

@@ -3,7 +3,7 @@ block of one column or one short), clusters above the portable eight CTAs, the k
 panel whose rank ends inside a block.  Through prac_draw_random without a principal part, which orthonormalises a
 Gaussian block: its thin QR factor with positive diagonal is unique.
 
-Bounds: each column of Q to 1e-4 (fp32 panel, R exact to double), and the orthonormality that rounding Q to fp32 leaves,
+Bounds: each column of Q to 1e-4 (fp32 panel; that R is exact to double is checked on ill-conditioned panels), and the orthonormality that rounding Q to fp32 leaves,
 ||Q^T Q - I||_F of about n 2^-24 with a constant of order one (8.5e-6 measured at 512 columns)."""
 import numpy as np
 import pytest
@@ -66,6 +66,39 @@ def test_panel_whose_rank_ends_inside_a_block(k, rank):
     U, X64 = f64(b.get()[0]), f64(X)
     assert np.linalg.norm(U.T @ U - np.eye(k)) <= 1e-5
     assert np.linalg.norm(X64 - X64 @ U @ U.T) <= 1e-4 * np.linalg.norm(X64)
+
+
+@pytest.mark.parametrize("cooperative", [0, 1])
+@pytest.mark.parametrize("n", [32, 33, 256, 257, 512, 513])
+@pytest.mark.parametrize("kappa", [1e2, 1e5, 1e6])
+def test_inverse_factor_of_an_ill_conditioned_panel_is_exact_to_double(n, kappa, cooperative):
+    # Singular values from 1 to 1 / kappa, columns mixed.  The panel's last n rows are eps I, so that those rows of Q are eps
+    # R^-1, element by element to fp32 (2^-22).  Rounding V^T V and its factor to double turns R^-1 by about kappa^2 2^-53
+    # (a tenth of it measured, at all sizes); a step in fp32, or with ten bits of a double lost, is far beyond that at 1e5 and 1e6.
+    # Pivots stay above 1e-13 of their column's norm, so none is replaced.
+    from paper_2602_23111_b200 import api
+    d = n + 300 + n // 2
+    rng = np.random.default_rng(n)
+    A = np.linalg.qr(rng.standard_normal((d - n, n)))[0] * np.logspace(0, -np.log10(kappa), n)
+    A = A @ np.linalg.qr(rng.standard_normal((n, n)))[0]
+    eps = 2.0 ** -10 / kappa
+    V = np.concatenate([A, eps * np.eye(n)]).astype(np.float32)
+    R = np.linalg.qr(V.astype(np.float64), mode="r")
+    R *= np.sign(np.diag(R))[:, None]
+    exact = np.linalg.solve(R, np.eye(n))
+    Vd, word = torch.from_numpy(V).cuda(), torch.zeros(1, dtype=torch.int32, device="cuda")
+    Q = torch.empty_like(Vd)
+    ws = torch.empty(api.lib.prac_debug_cholqr_ws_bytes(d, n), dtype=torch.uint8, device="cuda")
+    api.lib.prac_debug_force_cooperative_cholesky(cooperative)
+    try:
+        st = api.lib.prac_debug_cholqr(Vd.data_ptr(), Q.data_ptr(), d, n, ws.data_ptr(), ws.numel(), word.data_ptr(),
+                                       torch.cuda.current_stream().cuda_stream)
+    finally:
+        api.lib.prac_debug_force_cooperative_cholesky(0)
+    assert st == api.PRAC_OK and int(word.item()) == 0
+    got = f64(Q)[-n:] / eps
+    off = np.linalg.norm(got - exact) / np.linalg.norm(exact)
+    assert off <= 2.0 ** -22 + 2.0 ** -53 * kappa ** 2
 
 
 def test_quotients_of_the_elimination_against_division():
