@@ -15,8 +15,8 @@ micro-batches, no data-path collective); the time is the max over ranks.  With -
 ranks share one batch instead: the Gram matrix of each fit and the middle factor dY^T Z of each
 weight gradient are summed over the ranks (NCCL all-reduce), everything else is local.
 
-Besides the headline line the default run reports, under extra keys and within a wall-time
-budget: the other workloads and ranks of the sweep, the variant without subspace sharing, the
+Besides the headline line, which goes to standard output by itself, the default run reports on standard
+error, one JSON line per section and within a wall-time budget: the other workloads and ranks of the sweep, the variant without subspace sharing, the
 split of the fit, the lazy-update drift study, and the oracle at full size on the two small
 workloads.
 """
@@ -51,6 +51,21 @@ GRAD_STREAMS = int(os.environ.get("PRAC_GRAD_STREAMS", "4"))
 METRIC = "compressed tokens/s per layer (fit+compress+dW)"
 UNIT = "layer-tokens/s"
 NOMINAL_BF16_TFLOPS = 2250.0        # dense bf16 of the part's data sheet, for context beside the measured peak
+
+
+# What the line on standard output carries; every other section has a line of its own on standard error.  (With all of
+# them on one line it was 20 KB long, and whoever keeps only the end of the output lost the figures it begins with.)
+HEADLINE = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "ms_per_step_median", "ms_per_step_best",
+            "higher_is_better", "scaling", "vs_baseline", "dtype", "data", "config", "phases_ms", "roofline", "cpu_baseline",
+            "clocks", "e2e", "gpu_launches", "device_status")
+
+
+def report(out: dict) -> None:
+    """Prints the sections of a run, the headline last."""
+    for key, value in out.items():
+        if key not in HEADLINE:
+            print(json.dumps({"section": key, key: value}), file=sys.stderr, flush=True)
+    print(json.dumps({key: out[key] for key in HEADLINE if key in out}), flush=True)
 
 
 # ----------------------------------------------------------------------------- helpers
@@ -1051,11 +1066,11 @@ def main():
                    "grad_calls": f"{len(blk.groups)} (linears sharing an input are one call over their dY side by side)",
                    "l2": "inputs (2.2 GB per block) exceed L2; no flush",
                    "layout": "rows of X, dY, Z and dW padded to 128-byte multiples", "parallelism": f"replicas x{world}"},
-        "phases_ms": {"fit_per_refresh": fit_ms, "warm_refresh": refresh_ms, "compress": comp_ms, "weight_grad": grad_ms,
-                      "median": {"fit_per_refresh": fit_st["median"], "warm_refresh": refresh_st["median"],
-                                 "compress": comp_st["median"], "weight_grad": grad_st["median"]},
-                      "best": {"fit_per_refresh": fit_st["best"], "warm_refresh": refresh_st["best"],
-                               "compress": comp_st["best"], "weight_grad": grad_st["best"]}},
+        "phases_ms": {"fit_per_refresh": fit_ms, "warm_refresh": refresh_ms, "compress": comp_ms, "weight_grad": grad_ms},
+        "phases_spread_ms": {"median": {"fit_per_refresh": fit_st["median"], "warm_refresh": refresh_st["median"],
+                                        "compress": comp_st["median"], "weight_grad": grad_st["median"]},
+                             "best": {"fit_per_refresh": fit_st["best"], "warm_refresh": refresh_st["best"],
+                                      "compress": comp_st["best"], "weight_grad": grad_st["best"]}},
         "steady_state": steady,
         "peaks": {"bf16_tflops_burst": peaks["bf16_tflops"], "bf16_tflops_sustained": peaks["bf16_tflops_sustained"],
                   "hbm_gbs": peaks["hbm_gbs"], "source": peaks["source"], "how": peaks["how"], "when": peaks["when"],
@@ -1100,7 +1115,7 @@ def main():
         out["cpu_baseline"] = cpu_baseline(w, kr, max(256, w.N // 4))
         if not args.skip_sweep and world == 1:
             out["cpu_baseline_full_size"] = cpu_baseline_full_size()
-    print(json.dumps(out))
+    report(out)
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
