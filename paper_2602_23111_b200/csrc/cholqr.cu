@@ -46,38 +46,10 @@ __device__ __forceinline__ bool pass_is_off(const int* run_if, int mask) {
   return run_if != nullptr && (*reinterpret_cast<const volatile int*>(run_if) & mask) == 0;
 }
 
-// Shared memory of another CTA of the cluster.
-__device__ __forceinline__ uint32_t cluster_addr(const void* own, unsigned rank) {
-  uint32_t r;
-  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(own))), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ double2 cluster_ld(uint32_t addr) {
-  double2 v;
-  asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(addr) : "memory");
-  return v;
-}
-__device__ __forceinline__ double cluster_ld1(uint32_t addr) {
-  double v;
-  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr) : "memory");
-  return v;
-}
-// (the store's 16 bytes are counted on the barrier when they have arrived)
-__device__ __forceinline__ void cluster_st_async(uint32_t addr, double2 v, uint32_t bar) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%0], {%1, %2}, [%3];" ::"r"(addr), "d"(v.x), "d"(v.y), "r"(bar)
-               : "memory");
-}
-__device__ __forceinline__ void cluster_st_flag(uint32_t addr, int v) {
-  asm volatile("st.release.cluster.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
-// A barrier for one event: an arrival, or, where bytes > 0, that many bytes stored by cluster_st_async.
+// A barrier for one event: an arrival, or, where bytes > 0, that many bytes stored by ptx::cluster_st_async.
 __device__ __forceinline__ void cluster_bar_init(uint64_t* own, unsigned bytes) {
-  const uint32_t b = static_cast<uint32_t>(__cvta_generic_to_shared(own));
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b) : "memory");
-  if (bytes) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void cluster_bar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+  ptx::mbar_init(own, 1);
+  if (bytes) ptx::mbar_arrive_expect_tx(own, bytes);
 }
 __device__ __forceinline__ bool cluster_try_wait(uint64_t* own) {
   uint32_t ok;
@@ -97,23 +69,6 @@ __device__ __forceinline__ bool cluster_try_wait_acquire(uint64_t* own) {
       : "=r"(ok) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(own))) : "memory");
   return ok != 0;
 }
-__device__ __forceinline__ bool cluster_try_wait_rows(uint64_t* own) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred P;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 P, [%1], 0;\n\t"
-      "selp.b32 %0, 1, 0, P;\n\t}"
-      : "=r"(ok) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(own))) : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ void cluster_arrive() {
-  __syncwarp();
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait() {
-  __syncwarp();
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 
 __device__ __forceinline__ void atb_tile(const AtbArgs& g, int tile, int& ti, int& tj) {
   if (!g.symmetric) { ti = tile / g.tiles_n; tj = tile % g.tiles_n; return; }
@@ -124,13 +79,6 @@ __device__ __forceinline__ void atb_tile(const AtbArgs& g, int tile, int& ti, in
     rest -= cnt;
     ++row;
   }
-}
-
-// One double-precision tensor-core product: D (8 x 8) += A (8 x 4, row-major fragment) * B (4 x 8,
-// column-major fragment).  Lane L holds A[L / 4][L % 4], B[L % 4][L / 4] and D[L / 4][2 (L % 4) + {0, 1}].
-__device__ __forceinline__ void dmma_884(double (&d)[2], double a, double b) {
-  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
-               : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
 }
 
 // A 64 x 64 output tile by one cluster: each CTA takes a slice of the rows, 16 at a time, three chunks ahead of the
@@ -202,8 +150,8 @@ __global__ void __launch_bounds__(256) atb_f64_kernel(const AtbArgs g) {
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         const double bv = b[c * 8];
-        dmma_884(acc[0][c], a0, bv);
-        dmma_884(acc[1][c], a1, bv);
+        ptx::dmma_884(acc[0][c], a0, bv);
+        ptx::dmma_884(acc[1][c], a1, bv);
       }
     }
     stage = (stage + 1) % AT_STAGES;
@@ -215,8 +163,8 @@ __global__ void __launch_bounds__(256) atb_f64_kernel(const AtbArgs g) {
 #pragma unroll
     for (int c = 0; c < 4; ++c)
       *reinterpret_cast<double2*>(&tile[(wa + h * 8 + gq) * AT_P + wb + c * 8 + 2 * q4]) = make_double2(acc[h][c][0], acc[h][c][1]);
-  cluster_arrive();
-  cluster_wait();
+  ptx::cluster_arrive();
+  ptx::cluster_wait();
   // rows [64 rank / slices, 64 (rank + 1) / slices) of the tile
   const int rows = AT_T / slices;
 #pragma unroll 1
@@ -225,7 +173,7 @@ __global__ void __launch_bounds__(256) atb_f64_kernel(const AtbArgs g) {
     const int i = m0 + r, j = n0 + c;
     double v = 0.0;
 #pragma unroll 4
-    for (int s = 0; s < slices; ++s) v += cluster_ld1(cluster_addr(&tile[r * AT_P + c], s));
+    for (int s = 0; s < slices; ++s) v += ptx::cluster_ld_f64(ptx::cluster_addr(&tile[r * AT_P + c], s));
     v *= g.alpha;
     if (i >= g.m || j >= g.n || (g.symmetric && i > j)) continue;
     const int copies = g.symmetric && i != j ? 2 : 1;
@@ -237,8 +185,8 @@ __global__ void __launch_bounds__(256) atb_f64_kernel(const AtbArgs g) {
       else static_cast<float*>(g.out)[o] = static_cast<float>(v);
     }
   }
-  cluster_arrive();                  // (nobody's tile goes away under a reader)
-  cluster_wait();
+  ptx::cluster_arrive();                  // (nobody's tile goes away under a reader)
+  ptx::cluster_wait();
 }
 
 // ------------------------------------------------------------------ Cholesky + inverse, one launch
@@ -303,8 +251,8 @@ __device__ __forceinline__ void blk_mm(double (*C)[CP], const double (*A)[CP], c
     const double a = (mode >= 2) ? A[row0 + g][ks * 4 + q] : A[ks * 4 + q][row0 + g];
     const double b0 = B[ks * 4 + q][col0 + g];
     const double b1 = B[ks * 4 + q][col0 + 8 + g];
-    dmma_884(acc0, a, b0);
-    dmma_884(acc1, a, b1);
+    ptx::dmma_884(acc0, a, b0);
+    ptx::dmma_884(acc1, a, b1);
   }
   double* c0 = &C[row0 + g][col0 + 2 * q];
   double* c1 = &C[row0 + g][col0 + 8 + 2 * q];
@@ -456,8 +404,8 @@ __device__ __forceinline__ void sub_update(double (*C)[CP], int p, int q, const 
   double2* const o = reinterpret_cast<double2*>(&C[8 * p + g][8 * q + 2 * q4]);
   const double2 old = *o;
   double a0[2] = {0.0, 0.0}, a1[2] = {0.0, 0.0};
-  dmma_884(a0, R[q4][8 * p + g], B[q4][8 * q + g]);
-  dmma_884(a1, R[4 + q4][8 * p + g], B[4 + q4][8 * q + g]);
+  ptx::dmma_884(a0, R[q4][8 * p + g], B[q4][8 * q + g]);
+  ptx::dmma_884(a1, R[4 + q4][8 * p + g], B[4 + q4][8 * q + g]);
   *o = make_double2((fresh ? 0.0 : old.x) - (a0[0] + a1[0]), (fresh ? 0.0 : old.y) - (a0[1] + a1[1]));
 }
 
@@ -830,7 +778,7 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
       late = late || now - since > CC_WAIT_NS;
     }
     if (late)
-      for (int x = 0; x < nb; ++x) cluster_st_flag(cluster_addr(&words.abort, x), 1);
+      for (int x = 0; x < nb; ++x) ptx::cluster_st_release(ptx::cluster_addr(&words.abort, x), 1);
     return late;
   };
   // Every lane waits for a barrier of its own (or none): cheap polls, and one that acquires (it takes 400 cycles) once
@@ -851,22 +799,22 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
     if (lane == 0 && !fail) {
       unsigned polls = 0;
       uint64_t since = 0;
-      while (!cluster_try_wait_rows(bar))
+      while (!ptx::mbar_try_wait(bar, 0))
         if (gives_up(++polls, since)) { fail = true; break; }
     }
     __syncwarp();
   };
   // Rows 8 s .. 8 s + 7 of R_qq^-T up to the diagonal tile, to the next CTA (128 threads): rows(r, cc) is the pair at column cc.
-  const uint32_t far = q + 1 < nb ? cluster_addr(Dprev, q + 1) : 0u, far_bar = q + 1 < nb ? cluster_addr(words.band, q + 1) : 0u;
+  const uint32_t far = q + 1 < nb ? ptx::cluster_addr(Dprev, q + 1) : 0u, far_bar = q + 1 < nb ? ptx::cluster_addr(words.band, q + 1) : 0u;
   auto send_rows = [&](int s, auto rows) {
     const int i = tid & 127, r = 8 * s + (i & 7), cc = 2 * (i >> 3);
-    if (cc < 8 * (s + 1)) cluster_st_async(far + (r * CP + cc) * 8, rows(r, cc), far_bar + 8 * s);
+    if (cc < 8 * (s + 1)) ptx::cluster_st_async(far + (r * CP + cc) * 8, rows(r, cc), far_bar + 8 * s);
   };
   // the pairs (row, 2 columns) of a block that a thread of a group moves
   auto pull = [&](uint32_t from, double2 (&v)[2]) {
 #pragma unroll
     for (int e = 0; e < 2; ++e)
-      v[e] = cluster_ld(from + (((gt + 256 * e) >> 4) * CP + 2 * (gt & 15)) * 8);
+      v[e] = ptx::cluster_ld_f64x2(from + (((gt + 256 * e) >> 4) * CP + 2 * (gt & 15)) * 8);
   };
   auto put = [&](Blk to, const double2 (&v)[2]) {
 #pragma unroll
@@ -891,10 +839,10 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
           cluster_bar_init(&words.band[s], q > 0 ? 8 * 8 * (s + 1) * 8 : 0);      // eight rows up to the diagonal tile, in bytes
         }
         if (tid == 511) words.abort = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        ptx::fence_mbar_init();
       }
       __syncthreads();
-      cluster_arrive();
+      ptx::cluster_arrive();
       // this CTA's column of G, padded with the identity
       for (int i0 = tid / CB; i0 < (q + 1) * CB; i0 += 8 * (256 * CC_GROUPS / CB)) {       // (eight loads in flight)
         double v[8];
@@ -913,7 +861,7 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
       for (int idx = tid; idx < (nb - q) * CB * CP; idx += 256 * CC_GROUPS)      // the running sums
         inv(q)[0][idx] = 0.0;
       if (group == 1 && !dry) chol_emit_zeros(a, q, nb);
-      cluster_wait();
+      ptx::cluster_wait();
       __syncthreads();
       if (tid < CB) guard[tid] = dry ? 1e-13 : pivot_guard(col(q)[tid][tid]);
       if (dry) {
@@ -939,8 +887,8 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
           double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
 #pragma unroll 2
           for (int ks = 0; ks < 2 * s + 2; ks += 2) {
-            dmma_884(acc[0], Dprev[r0 + g][ks * 4 + q4], mine[ks * 4 + q4][c0 + g]);
-            dmma_884(acc[1], Dprev[r0 + g][ks * 4 + 4 + q4], mine[ks * 4 + 4 + q4][c0 + g]);
+            ptx::dmma_884(acc[0], Dprev[r0 + g][ks * 4 + q4], mine[ks * 4 + q4][c0 + g]);
+            ptx::dmma_884(acc[1], Dprev[r0 + g][ks * 4 + 4 + q4], mine[ks * 4 + 4 + q4][c0 + g]);
           }
           *reinterpret_cast<double2*>(&Rbuf[r0 + g][c0 + 2 * q4]) = make_double2(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
           bar_arrive(9 + s, 128 + 256);
@@ -961,11 +909,11 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
         for (int s = 0; s < CB / 8; ++s) {
           bar_sync(9 + s, 128 + 256);
           const double (*R)[CP] = Rbuf + 8 * s;
-          dmma_884(acc[0][0], R[q4][8 * p0 + g], R[q4][8 * x0 + g]);
-          dmma_884(acc[0][1], R[4 + q4][8 * p0 + g], R[4 + q4][8 * x0 + g]);
+          ptx::dmma_884(acc[0][0], R[q4][8 * p0 + g], R[q4][8 * x0 + g]);
+          ptx::dmma_884(acc[0][1], R[4 + q4][8 * p0 + g], R[4 + q4][8 * x0 + g]);
           if (u1 >= 0) {
-            dmma_884(acc[1][0], R[q4][8 * p1 + g], R[q4][8 * x1 + g]);
-            dmma_884(acc[1][1], R[4 + q4][8 * p1 + g], R[4 + q4][8 * x1 + g]);
+            ptx::dmma_884(acc[1][0], R[q4][8 * p1 + g], R[q4][8 * x1 + g]);
+            ptx::dmma_884(acc[1][1], R[4 + q4][8 * p1 + g], R[4 + q4][8 * x1 + g]);
           }
         }
         double2* o = reinterpret_cast<double2*>(&Dq[8 * p0 + g][8 * x0 + 2 * q4]);
@@ -991,12 +939,12 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
         for (int e = 0; e < 2; ++e) v[e] = *reinterpret_cast<const double2*>(&Rbuf[(gt + 256 * e) >> 4][2 * (gt & 15)]);
         put(col(c), v);
         bar_sync(2, 256);
-        if (warp == 15 && lane < nb && lane != q) cluster_bar_arrive(cluster_addr(&words.row[c][q], lane));
+        if (warp == 15 && lane < nb && lane != q) ptx::mbar_arrive_cluster(ptx::cluster_addr(&words.row[c][q], lane));
       }
       sent = !dry;
       // every thread leaves here if one has given up
       if (__syncthreads_or(fail)) { fail = true; break; }
-      if (!dry && warp == 8 && lane < nb && lane != q) cluster_bar_arrive(cluster_addr(&words.diag[q], lane));
+      if (!dry && warp == 8 && lane < nb && lane != q) ptx::mbar_arrive_cluster(ptx::cluster_addr(&words.diag[q], lane));
     }
     if (dry || (c >= 0 && c != q - 1)) {
       const bool left = c < q;
@@ -1006,7 +954,7 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
         if (!dry) wait_for(lane == 0 ? &words.diag[c] : nullptr);
         {
           const int r = tid >> 4, cc = 2 * (tid & 15);
-          const double2 v = cluster_ld(cluster_addr(&(dry ? Dprev : block(c + 1))[r][cc], dry ? q : c));
+          const double2 v = ptx::cluster_ld_f64x2(ptx::cluster_addr(&(dry ? Dprev : block(c + 1))[r][cc], dry ? q : c));
           *reinterpret_cast<double2*>(&Dfar[r][cc]) = v;
         }
         __syncthreads();
@@ -1019,13 +967,13 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
             const int k = (ks + e) * 4 + q4;
-            dmma_884(acc[e], left ? Dfar[r0 + g][k] : own[r0 + g][k], left ? own[k][c0 + g] : Dfar[c0 + g][k]);
+            ptx::dmma_884(acc[e], left ? Dfar[r0 + g][k] : own[r0 + g][k], left ? own[k][c0 + g] : Dfar[c0 + g][k]);
           }
         }
         __syncthreads();
         *reinterpret_cast<double2*>(&own[r0 + g][c0 + 2 * q4]) = make_double2(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
         if (__syncthreads_or(fail)) { fail = true; break; }
-        if (!dry && left && warp == 15 && lane < nb && lane != q) cluster_bar_arrive(cluster_addr(&words.row[c][q], lane));
+        if (!dry && left && warp == 15 && lane < nb && lane != q) ptx::mbar_arrive_cluster(ptx::cluster_addr(&words.row[c][q], lane));
       }
       // ---- the blocks it brings up to date, dealt to the groups: (p, q), c < p <= q, of G, (q, q) first, which needs nobody
       // else's block; or (q, x), x > c, of the inverse
@@ -1037,13 +985,13 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
       if (first < end) {
         const int mine = first + CC_GROUPS * lane;
         if (!dry) wait_for(mine < end ? &words.row[c][mine] : nullptr);
-        pull(cluster_addr(from, dry ? q : first), v);
+        pull(ptx::cluster_addr(from, dry ? q : first), v);
       }
       for (int x = first; x < end; x += CC_GROUPS) {
         bar_sync(1 + group, 256);            // the block before this one is done with
         put(stage, v);
         bar_sync(1 + group, 256);
-        if (x + CC_GROUPS < end) pull(cluster_addr(from, x + CC_GROUPS), v);
+        if (x + CC_GROUPS < end) pull(ptx::cluster_addr(from, x + CC_GROUPS), v);
         Blk const C = dry ? Dfar : (left ? col(x) : inv(x));
         if (left) blk_mm(C, stage, own, 1);
         else blk_mm(C, own, stage, c == q ? 1 : 3);
@@ -1059,12 +1007,12 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
     if (tid == 0 && q > 0) {
       const uint64_t since = ptx::globaltimer_ns();
       for (int s = 0; s < CB / 8; ++s)
-        while (!cluster_try_wait_rows(&words.band[s]) && ptx::globaltimer_ns() - since <= 2 * CC_WAIT_NS) {}
+        while (!ptx::mbar_try_wait(&words.band[s], 0) && ptx::globaltimer_ns() - since <= 2 * CC_WAIT_NS) {}
     }
     __syncthreads();
   }
-  cluster_arrive();
-  cluster_wait();
+  ptx::cluster_arrive();
+  ptx::cluster_wait();
 }
 
 size_t chol_cluster_smem(int nb) {

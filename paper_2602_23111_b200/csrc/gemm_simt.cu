@@ -16,6 +16,7 @@
 
 #include "internal.h"
 #include "per_device.h"
+#include "ptx.cuh"
 
 namespace prac {
 namespace {
@@ -73,25 +74,6 @@ __device__ __forceinline__ float4 as_floats(const float4& v, int bf16) {
   if (!bf16) return v;
   const uint32_t a = __float_as_uint(v.x), b = __float_as_uint(v.y);
   return make_float4(bf16_bits(a & 0xffffu), __uint_as_float(a & 0xffff0000u), bf16_bits(b & 0xffffu), __uint_as_float(b & 0xffff0000u));
-}
-
-__device__ __forceinline__ uint32_t cluster_addr(const void* p, int rank) {
-  uint32_t a;
-  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(p))), "r"(rank));
-  return a;
-}
-__device__ __forceinline__ float4 cluster_load4(uint32_t a) {
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
-  return v;
-}
-__device__ __forceinline__ float cluster_load1(uint32_t a) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
-  return v;
-}
-__device__ __forceinline__ void cluster_meet() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // One CTA: a TM x TN tile of C over its share of K.  SL groups of 256 / SL threads; group g of CTA
@@ -243,7 +225,7 @@ __global__ void __launch_bounds__(THREADS, 2) gemm_simt_kernel(const DevGemm g) 
       *reinterpret_cast<float4*>(o) = v;
     }
   }
-  if (g.parts > 1) cluster_meet();
+  if (g.parts > 1) ptx::cluster_sync_all();
   const int rows = TM / g.parts;             // this CTA closes the rows [part * rows, + rows) of the tile
   if (g.vec_c && !g.symmetric) {             // fp32 rows on the 16-byte grid: four columns per thread
     for (int q = threadIdx.x; q < rows * ROW4; q += THREADS) {
@@ -251,9 +233,9 @@ __global__ void __launch_bounds__(THREADS, 2) gemm_simt_kernel(const DevGemm g) 
       const float* o = sm + row * S::RED_P + col;
       float4 v;
       if (g.parts > 1) {
-        v = cluster_load4(cluster_addr(o, 0));
+        v = ptx::cluster_ld_f32x4(ptx::cluster_addr(o, 0));
         for (int h = 1; h < g.parts; ++h) {
-          const float4 w = cluster_load4(cluster_addr(o, h));
+          const float4 w = ptx::cluster_ld_f32x4(ptx::cluster_addr(o, h));
           v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
         }
       } else {
@@ -292,8 +274,8 @@ __global__ void __launch_bounds__(THREADS, 2) gemm_simt_kernel(const DevGemm g) 
       const float* o = sm + row * S::RED_P + col;
       float v;
       if (g.parts > 1) {
-        v = cluster_load1(cluster_addr(o, 0));
-        for (int h = 1; h < g.parts; ++h) v += cluster_load1(cluster_addr(o, h));
+        v = ptx::cluster_ld_f32(ptx::cluster_addr(o, 0));
+        for (int h = 1; h < g.parts; ++h) v += ptx::cluster_ld_f32(ptx::cluster_addr(o, h));
       } else {
         v = *o;
 #pragma unroll
@@ -320,7 +302,7 @@ __global__ void __launch_bounds__(THREADS, 2) gemm_simt_kernel(const DevGemm g) 
       }
     }
   }
-  if (g.parts > 1) cluster_meet();           // a CTA's shared memory is read until its peers are done
+  if (g.parts > 1) ptx::cluster_sync_all();           // a CTA's shared memory is read until its peers are done
 }
 
 template <int TM, int TN, int SL, bool TA, bool TB>

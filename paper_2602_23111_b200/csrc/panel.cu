@@ -316,13 +316,6 @@ __global__ void jacobi_kernel(double* At, int n, int b, int max_sweeps, double t
 }
 
 // ------------------------------------------------------------------ block Jacobi through the Gram matrix
-// One double-precision tensor-core product: D (8 x 8) += A (8 x 4, row-major fragment) * B (4 x 8,
-// column-major fragment).  Lane L holds A[L / 4][L % 4], B[L % 4][L / 4] and D[L / 4][2 (L % 4) + {0, 1}].
-__device__ __forceinline__ void dmma_884(double (&d)[2], double a, double b) {
-  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
-               : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
-}
-
 constexpr int JG_B = 8;          // columns per block
 constexpr int JG_M = 2 * JG_B;   // columns a CTA holds
 constexpr int JG_P = JG_M + 1;   // pitch of the small matrices
@@ -387,9 +380,9 @@ __global__ void __launch_bounds__(256) jacobi_gram_kernel(double* At, int n, int
           for (int ks = warp * kpw; ks < ks_end; ++ks) {
             const int r = ks * 4 + q4;
             const double a0 = cols[g * ns + r], a1 = cols[(8 + g) * ns + r];
-            dmma_884(t00, a0, a0);
-            dmma_884(t01, a0, a1);
-            dmma_884(t11, a1, a1);
+            ptx::dmma_884(t00, a0, a0);
+            ptx::dmma_884(t01, a0, a1);
+            ptx::dmma_884(t11, a1, a1);
           }
           double* pw = part + warp * 192 + g * 8 + 2 * q4;
           pw[0] = t00[0]; pw[1] = t00[1];
@@ -483,8 +476,8 @@ __global__ void __launch_bounds__(256) jacobi_gram_kernel(double* At, int n, int
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
               const double a = cols[(kk * 4 + q4) * ns + r];
-              dmma_884(o0, a, b0[kk]);
-              dmma_884(o1, a, b1[kk]);
+              ptx::dmma_884(o0, a, b0[kk]);
+              ptx::dmma_884(o1, a, b1[kk]);
             }
             cols[(2 * q4) * ns + r] = o0[0];
             cols[(2 * q4 + 1) * ns + r] = o0[1];
@@ -597,22 +590,6 @@ __device__ __forceinline__ void rr_where(int m, int step, int X, int& cta, int& 
   slot = X < partner ? 0 : 1;
 }
 
-__device__ __forceinline__ uint32_t cluster_smem(const void* own, int cta) {
-  uint32_t r;
-  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(own))), "r"(cta));
-  return r;
-}
-__device__ __forceinline__ double cluster_ld(uint32_t addr) {
-  double v;
-  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr) : "memory");
-  return v;
-}
-__device__ __forceinline__ void cluster_barrier() {
-  __syncwarp();
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
 // A finishing step on the columns of all CTAs (16 each; up to ROWS of them), once they are nearly orthogonal:
 // the whole Gram matrix, and then, where the rotation angles T_ij = g_ij / (g_jj - g_ii) of all pairs are small, one rotation for
 // all of them, A <- A exp(T), else nothing, because columns of nearly equal norm still turn by large angles.  Pairs that
@@ -643,14 +620,14 @@ __device__ __noinline__ int jacobi_finish(double (*cols)[ROWS + 2], double* At, 
     return At + static_cast<long long>(e < JG_B ? I * JG_B + e : J * JG_B + e - JG_B) * n;
   };
   auto meet = [&]() {
-    if (CLUSTER) { cluster_barrier(); return true; }
+    if (CLUSTER) { ptx::cluster_sync_all(); return true; }
     return grid_barrier(&info->bar, ++bar * gridDim.x, poll_limit);
   };
   // ---- Gp[i][j] = column i of this CTA times column j of all
   double (*const Gp)[ROWS + 2] = term0;
   for (int job = warp; job < 2 * ctas; job += WARPS) {
     const int e = 8 * (job & 1) + g;
-    const uint32_t other = CLUSTER ? cluster_smem(&cols[e][q4], job >> 1) : 0u;
+    const uint32_t other = CLUSTER ? ptx::cluster_addr(&cols[e][q4], job >> 1) : 0u;
     const double* const in_mem = CLUSTER ? nullptr : column(job >> 1, e) + q4;
     const double* const own0 = CLUSTER ? &cols[g][q4] : column(rank, g) + q4;
     const double* const own1 = CLUSTER ? &cols[8 + g][q4] : column(rank, 8 + g) + q4;
@@ -659,15 +636,15 @@ __device__ __noinline__ int jacobi_finish(double (*cols)[ROWS + 2], double* At, 
     for (int ks = 0; ks < ROWS / 4; ++ks) {
       double a0, a1, b;
       if (CLUSTER) {
-        b = cluster_ld(other + ks * 32);
+        b = ptx::cluster_ld_f64(other + ks * 32);
         a0 = own0[4 * ks]; a1 = own1[4 * ks];
       } else {                         // (n is a multiple of 16)
         const bool in = 4 * ks < n;
         b = in ? __ldcg(in_mem + 4 * ks) : 0.0;
         a0 = in ? __ldcg(own0 + 4 * ks) : 0.0; a1 = in ? __ldcg(own1 + 4 * ks) : 0.0;
       }
-      dmma_884(acc0, a0, b);
-      dmma_884(acc1, a1, b);
+      ptx::dmma_884(acc0, a0, b);
+      ptx::dmma_884(acc1, a1, b);
     }
 #pragma unroll
     for (int e2 = 0; e2 < 2; ++e2) {
@@ -730,14 +707,14 @@ __device__ __noinline__ int jacobi_finish(double (*cols)[ROWS + 2], double* At, 
       double acc0[2] = {0.0, 0.0}, acc1[2] = {0.0, 0.0};
       const int r = 8 * band + g;
       for (int c = 0; c < ctas; ++c) {
-        const uint32_t other = CLUSTER ? cluster_smem(&from[q4][r], c) : 0u;
+        const uint32_t other = CLUSTER ? ptx::cluster_addr(&from[q4][r], c) : 0u;
 #pragma unroll
         for (int ks = 0; ks < JG_M / 4; ++ks) {
           const int e = 4 * ks + q4;
-          const double a = CLUSTER ? cluster_ld(other + ks * 4 * (ROWS + 2) * 8)
+          const double a = CLUSTER ? ptx::cluster_ld_f64(other + ks * 4 * (ROWS + 2) * 8)
                                    : __ldcg(m == 1 ? column(c, e) + r : from_mem + static_cast<long long>(JG_M * c + e) * n + r);
-          dmma_884(acc0, a, T[g][JG_M * c + e]);
-          dmma_884(acc1, a, T[8 + g][JG_M * c + e]);
+          ptx::dmma_884(acc0, a, T[g][JG_M * c + e]);
+          ptx::dmma_884(acc1, a, T[8 + g][JG_M * c + e]);
         }
       }
 #pragma unroll
@@ -802,7 +779,7 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
       for (int r = lane; r < ROWS; r += 32)
         reinterpret_cast<Cols>(jacobi_cols)[e][r] = r < n ? __ldcg(At + static_cast<long long>((e < b ? I * b + e : J * b + e - b)) * n + r) : 0.0;
     __syncthreads();
-    cluster_barrier();                 // (every CTA of the cluster has started)
+    ptx::cluster_sync_all();                 // (every CTA of the cluster has started)
   }
   for (; alive && sweep < max_sweeps && !converged; ++sweep) {
     for (int step = 0; alive && step < nb - 1; ++step) {
@@ -875,12 +852,9 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
           for (int h = 0; h < 2; ++h) {
             int cta, slot;
             rr_where(nb, next, h ? J : I, cta, slot);
-            uint32_t to, bar;
-            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(&there[JG_B * slot][r]))), "r"(cta));
-            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(bar) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(&arrived[turn ^ 1]))), "r"(cta));
+            const uint32_t to = ptx::cluster_addr(&there[JG_B * slot][r], cta), bar = ptx::cluster_addr(&arrived[turn ^ 1], cta);
 #pragma unroll
-            for (int e = 0; e < JG_B; ++e)
-              asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f64 [%0], %1, [%2];" ::"r"(to + e * (ROWS + 2) * 8), "d"(x[JG_B * h + e]), "r"(bar) : "memory");
+            for (int e = 0; e < JG_B; ++e) ptx::cluster_st_async(to + e * (ROWS + 2) * 8, x[JG_B * h + e], bar);
           }
         } else if (r < n) {
 #pragma unroll
@@ -916,9 +890,9 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
             const double a1[4] = {v[h][2].x, v[h][2].y, v[h][3].x, v[h][3].y};
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks) {
-              dmma_884(t00, a0[ks], a0[ks]);
-              dmma_884(t01, a0[ks], a1[ks]);
-              dmma_884(t11, a1[ks], a1[ks]);
+              ptx::dmma_884(t00, a0[ks], a0[ks]);
+              ptx::dmma_884(t01, a0[ks], a1[ks]);
+              ptx::dmma_884(t11, a1[ks], a1[ks]);
             }
           }
           const int o = g * 8 + 2 * q4;
@@ -1022,7 +996,7 @@ __global__ void __launch_bounds__(JS_G_THREADS + ROWS, 1) jacobi_stream_kernel(
         }
         __syncwarp();
         ++visit;
-        if (step == nb - 2) cluster_barrier();         // the sweep's largest cosine is complete
+        if (step == nb - 2) ptx::cluster_sync_all();         // the sweep's largest cosine is complete
       } else {
         alive = grid_barrier(&info->bar, ++bar * nctas, poll_limit);
       }

@@ -1,5 +1,6 @@
 // Thin wrappers over the sm_100a PTX used by the tensor-core GEMMs: mbarriers with bounded
-// waits, 2-D TMA tile loads, tcgen05 MMA / TMEM management, and the descriptors they take.
+// waits, 2-D TMA tile loads, tcgen05 MMA / TMEM management and the descriptors they take; and over that of the
+// clusters of the small-matrix kernels: barrier, one another's shared memory, fp64 products.
 #pragma once
 #include <cstdint>
 #include <cuda.h>
@@ -172,15 +173,57 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
-__device__ __forceinline__ void cluster_sync_all() {
+// The cluster's barrier (a warp has to be converged at it).
+__device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_sync_all() {
+  cluster_arrive();
+  cluster_wait();
 }
 // shared::cluster address of the same shared-memory location in CTA `rank` of the cluster
 __device__ __forceinline__ uint32_t mapa_shared(uint32_t cta_addr, uint32_t rank) {
   uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(cta_addr), "r"(rank));
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(cta_addr), "r"(rank));
   return r;
+}
+__device__ __forceinline__ uint32_t cluster_addr(const void* own, uint32_t rank) { return mapa_shared(smem_u32(own), rank); }
+// Loads and stores at such addresses.
+__device__ __forceinline__ float cluster_ld_f32(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ float4 cluster_ld_f32x4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ double cluster_ld_f64(uint32_t addr) {
+  double v;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ double2 cluster_ld_f64x2(uint32_t addr) {
+  double2 v;
+  asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(addr) : "memory");
+  return v;
+}
+// (the bytes are counted on the barrier, in the same CTA as addr, when they have arrived)
+__device__ __forceinline__ void cluster_st_async(uint32_t addr, double v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f64 [%0], %1, [%2];" ::"r"(addr), "d"(v), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void cluster_st_async(uint32_t addr, double2 v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%0], {%1, %2}, [%3];" ::"r"(addr), "d"(v.x), "d"(v.y), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void cluster_st_release(uint32_t addr, int v) {
+  asm volatile("st.release.cluster.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 // arrive on an mbarrier given by its shared::cluster address (own CTA or the peer)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
@@ -234,6 +277,15 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t* bar, uint16_t cta_mas
       : "memory");
 }
 
+// ---------------------------------------------------------------- fp64 tensor cores
+// D (8 x 8) += A (8 x 4, row-major fragment) * B (4 x 8, column-major fragment).  Lane L holds A[L / 4][L % 4],
+// B[L % 4][L / 4] and D[L / 4][2 (L % 4) + {0, 1}].
+__device__ __forceinline__ void dmma_884(double (&d)[2], double a, double b) {
+  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
+               : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
+}
+
+// ---------------------------------------------------------------- tensor memory to registers
 // 32 lanes x 32 consecutive 32-bit columns -> 32 registers per thread (lane = TMEM lane).
 __device__ __forceinline__ void tmem_ld_32x32(uint32_t taddr, uint32_t (&v)[32]) {
   asm volatile(
