@@ -34,7 +34,6 @@ struct AtbArgs {
   double alpha;
   void* out; long long ldo;
   int out_double;                  // out is double, else float
-  int next_early;                  // the next kernel may be set up from the start of this one
   const int* run_if;               // optional: the kernel does nothing unless *run_if & run_if_mask
   int run_if_mask;
   int* zero_words; int zero_count; // words that the next kernel on the stream expects zeroed
@@ -92,7 +91,6 @@ constexpr int AT_STAGES = 4;
 constexpr int AT_P = AT_T + 8;      // pitch of a row in shared memory: what four rows of a fragment load read lies in 32 banks
 __global__ void __launch_bounds__(256) atb_f64_kernel(const AtbArgs g) {
   grid_dep_wait();
-  if (g.next_early) grid_dep_launch();
   __shared__ __align__(16) double tile[AT_T * AT_P];        // the chunks in flight (fp32), then the slice's tile
   static_assert(AT_STAGES * 2 * AT_K * AT_P * sizeof(float) <= sizeof(tile), "the tile takes the place of the chunks");
   if (pass_is_off(g.run_if, g.run_if_mask)) return;
@@ -750,8 +748,10 @@ struct ChainWords {
 // that it is to receive (that wait ends, since they have all been sent; it is bounded too), and all meet at the cluster's
 // barrier before any leaves: nobody's shared memory goes away under a reader or under a store on its way.
 //
-// A CTA walks most of this code once, with its instructions not in the SM's cache yet (see sub_chol).  So every CTA
-// first runs the chain's part of a step on an identity, before it waits for the kernel that makes G.
+// A CTA walks most of this code once, with its instructions not in the SM's cache yet (270 cycles per 128 bytes).  A dry run
+// of the chain's part of a step on an identity, while the product before this kernel was still running, was no gain: the
+// product fills the GPU at 160 columns and more, and below that the dry run's own time shows (draws of 320 columns 104 us with
+// it, 96 without; fits of 2048 x 256 1559 and 1526, of the small fp32 layer 390 and 383; four fits side by side the same).
 __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const CholArgs a) {
   extern __shared__ __align__(16) double chol_smem[];
   __shared__ double guard[CB];
@@ -821,68 +821,52 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
     for (int e = 0; e < 2; ++e) *reinterpret_cast<double2*>(&to[(gt + 256 * e) >> 4][2 * (gt & 15)]) = v[e];
   };
 
-  // c = -2: the dry run (an optional pass, which is nearly always off, goes without); c = -1: set-up, and CTA 0
-  // factors its block; then the steps
-  for (int c = a.run_if_mask ? -1 : -2; c < nb; ++c) {
-    const bool dry = c == -2;
-    if (c < 0) {
-      const int rows = dry ? 0 : n;              // (the dry run reads and writes no global memory)
-      if (!dry) {
-        grid_dep_wait();
-        if (a.run_if_mask && pass_is_off(a.dev_status, a.run_if_mask)) return;
-      }
-      if (!dry) {
-        if (tid < CC_MAX * CC_MAX) cluster_bar_init(&words.row[0][0] + tid, 0);
-        else if (tid < CC_MAX * CC_MAX + CC_MAX) cluster_bar_init(&words.diag[tid - CC_MAX * CC_MAX], 0);
-        else if (tid < CC_MAX * CC_MAX + CC_MAX + CB / 8) {
-          const int s = tid - CC_MAX * CC_MAX - CC_MAX;
-          cluster_bar_init(&words.band[s], q > 0 ? 8 * 8 * (s + 1) * 8 : 0);      // eight rows up to the diagonal tile, in bytes
-        }
-        if (tid == 511) words.abort = 0;
-        ptx::fence_mbar_init();
-      }
-      __syncthreads();
-      ptx::cluster_arrive();
-      // this CTA's column of G, padded with the identity
-      for (int i0 = tid / CB; i0 < (q + 1) * CB; i0 += 8 * (256 * CC_GROUPS / CB)) {       // (eight loads in flight)
-        double v[8];
+  grid_dep_wait();
+  if (a.run_if_mask && pass_is_off(a.dev_status, a.run_if_mask)) return;
+  if (tid < CC_MAX * CC_MAX) cluster_bar_init(&words.row[0][0] + tid, 0);
+  else if (tid < CC_MAX * CC_MAX + CC_MAX) cluster_bar_init(&words.diag[tid - CC_MAX * CC_MAX], 0);
+  else if (tid < CC_MAX * CC_MAX + CC_MAX + CB / 8) {
+    const int s = tid - CC_MAX * CC_MAX - CC_MAX;
+    cluster_bar_init(&words.band[s], q > 0 ? 8 * 8 * (s + 1) * 8 : 0);          // eight rows up to the diagonal tile, in bytes
+  }
+  if (tid == 511) words.abort = 0;
+  ptx::fence_mbar_init();
+  __syncthreads();
+  ptx::cluster_arrive();
+  // this CTA's column of G, padded with the identity
+  for (int i0 = tid / CB; i0 < (q + 1) * CB; i0 += 8 * (256 * CC_GROUPS / CB)) {           // (eight loads in flight)
+    double v[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const int i = i0 + e * (256 * CC_GROUPS / CB), j = q * CB + tid % CB;
-          v[e] = i == j ? 1.0 : 0.0;
-          if (i < rows && j < rows) v[e] = __ldcg(&a.G[static_cast<long long>(i) * n + j]);
-        }
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const int i = i0 + e * (256 * CC_GROUPS / CB);
-          if (i < (q + 1) * CB) col(i / CB)[i % CB][tid % CB] = v[e];
-        }
-      }
-      for (int idx = tid; idx < (nb - q) * CB * CP; idx += 256 * CC_GROUPS)      // the running sums
-        inv(q)[0][idx] = 0.0;
-      if (group == 1 && !dry) chol_emit_zeros(a, q, nb);
-      ptx::cluster_wait();
-      __syncthreads();
-      if (tid < CB) guard[tid] = dry ? 1e-13 : pivot_guard(col(q)[tid][tid]);
-      if (dry) {
-        for (int idx = tid; idx < CB * CB; idx += 256 * CC_GROUPS) {
-          const int i = idx / CB, j = idx % CB;
-          Dprev[i][j] = block(nb + 4)[i][j] = i == j ? 1.0 : 0.0;
-          block(nb + 5)[i][j] = i == j ? 2.0 : 0.0;
-        }
-      }
-      __syncthreads();
+    for (int e = 0; e < 8; ++e) {
+      const int i = i0 + e * (256 * CC_GROUPS / CB), j = q * CB + tid % CB;
+      v[e] = i == j ? 1.0 : 0.0;
+      if (i < n && j < n) v[e] = __ldcg(&a.G[static_cast<long long>(i) * n + j]);
     }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int i = i0 + e * (256 * CC_GROUPS / CB);
+      if (i < (q + 1) * CB) col(i / CB)[i % CB][tid % CB] = v[e];
+    }
+  }
+  for (int idx = tid; idx < (nb - q) * CB * CP; idx += 256 * CC_GROUPS)          // the running sums
+    inv(q)[0][idx] = 0.0;
+  if (group == 1) chol_emit_zeros(a, q, nb);
+  ptx::cluster_wait();
+  __syncthreads();
+  if (tid < CB) guard[tid] = pivot_guard(col(q)[tid][tid]);
+  __syncthreads();
 
-    if (dry || c == q - 1) {
+  // c = -1: CTA 0 factors its block; then the steps
+  for (int c = -1; c < nb; ++c) {
+    if (c == q - 1) {
       // ---- the chain: block (c, q) of R and the diagonal block, by rows of R_cc^-T as they come; then the factorisation
-      Blk const Dq = dry ? block(nb + 5) : col(q), Rbuf = Dfar;
+      Blk const Dq = col(q), Rbuf = Dfar;
       if (c == -1) {
         // (CTA 0: nothing to take off)
       } else if (group == 1) {
         for (int s = (warp >> 2) & 1; s < CB / 8; s += 2) {
-          if (!dry) wait_rows(&words.band[s]);
-          Blk const mine = dry ? block(nb + 4) : col(c);
+          wait_rows(&words.band[s]);
+          Blk const mine = col(c);
           const int r0 = 8 * s, c0 = 8 * (warp & 3);
           double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
 #pragma unroll 2
@@ -927,12 +911,12 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
         main_sync();
       }
       if (group == 0) {
-        Blk const Lin = dry ? block(nb) : inv(q);
-        const bool next = !dry && q + 1 < nb;
-        blk_chol_inv(CholBlock{Dq, Lin, E, W, guard}, dry ? nullptr : a.dev_status, a.flag_bit, [&](int s) {
+        Blk const Lin = inv(q);
+        const bool next = q + 1 < nb;
+        blk_chol_inv(CholBlock{Dq, Lin, E, W, guard}, a.dev_status, a.flag_bit, [&](int s) {
           if (next) send_rows(s, [&](int r, int cc) { return *reinterpret_cast<const double2*>(&Lin[r][cc]); });
         });
-      } else if (!dry && c >= 0) {
+      } else if (c >= 0) {
         bar_sync(2, 256);                        // (Rbuf is complete)
         double2 v[2];
 #pragma unroll
@@ -941,20 +925,20 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
         bar_sync(2, 256);
         if (warp == 15 && lane < nb && lane != q) ptx::mbar_arrive_cluster(ptx::cluster_addr(&words.row[c][q], lane));
       }
-      sent = !dry;
+      sent = true;
       // every thread leaves here if one has given up
       if (__syncthreads_or(fail)) { fail = true; break; }
-      if (!dry && warp == 8 && lane < nb && lane != q) ptx::mbar_arrive_cluster(ptx::cluster_addr(&words.diag[q], lane));
+      if (warp == 8 && lane < nb && lane != q) ptx::mbar_arrive_cluster(ptx::cluster_addr(&words.diag[q], lane));
     }
-    if (dry || (c >= 0 && c != q - 1)) {
+    if (c >= 0 && c != q - 1) {
       const bool left = c < q;
-      Blk const own = dry ? block(nb + 5) : (left ? col(c) : inv(c));
+      Blk const own = left ? col(c) : inv(c);
       // ---- R_cc^-T, then this CTA's own block of step c
       if (c != q) {
-        if (!dry) wait_for(lane == 0 ? &words.diag[c] : nullptr);
+        wait_for(lane == 0 ? &words.diag[c] : nullptr);
         {
           const int r = tid >> 4, cc = 2 * (tid & 15);
-          const double2 v = ptx::cluster_ld_f64x2(ptx::cluster_addr(&(dry ? Dprev : block(c + 1))[r][cc], dry ? q : c));
+          const double2 v = ptx::cluster_ld_f64x2(ptx::cluster_addr(&block(c + 1)[r][cc], c));
           *reinterpret_cast<double2*>(&Dfar[r][cc]) = v;
         }
         __syncthreads();
@@ -973,26 +957,26 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
         __syncthreads();
         *reinterpret_cast<double2*>(&own[r0 + g][c0 + 2 * q4]) = make_double2(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
         if (__syncthreads_or(fail)) { fail = true; break; }
-        if (!dry && left && warp == 15 && lane < nb && lane != q) ptx::mbar_arrive_cluster(ptx::cluster_addr(&words.row[c][q], lane));
+        if (left && warp == 15 && lane < nb && lane != q) ptx::mbar_arrive_cluster(ptx::cluster_addr(&words.row[c][q], lane));
       }
       // ---- the blocks it brings up to date, dealt to the groups: (p, q), c < p <= q, of G, (q, q) first, which needs nobody
       // else's block; or (q, x), x > c, of the inverse
-      if (left && !dry && group == 0) blk_mm(col(q), own, own, 1);
+      if (left && group == 0) blk_mm(col(q), own, own, 1);
       if (!left && group == 1) chol_emit(a, own, q, c, c == q);
-      const int first = dry ? 0 : c + 1 + (left ? 1 - group : group), end = dry ? 1 : (left ? q : nb);
-      Blk const from = dry ? Dprev : block(c);
+      const int first = c + 1 + (left ? 1 - group : group), end = left ? q : nb;
+      Blk const from = block(c);
       double2 v[2];
       if (first < end) {
         const int mine = first + CC_GROUPS * lane;
-        if (!dry) wait_for(mine < end ? &words.row[c][mine] : nullptr);
-        pull(ptx::cluster_addr(from, dry ? q : first), v);
+        wait_for(mine < end ? &words.row[c][mine] : nullptr);
+        pull(ptx::cluster_addr(from, first), v);
       }
       for (int x = first; x < end; x += CC_GROUPS) {
         bar_sync(1 + group, 256);            // the block before this one is done with
         put(stage, v);
         bar_sync(1 + group, 256);
         if (x + CC_GROUPS < end) pull(ptx::cluster_addr(from, x + CC_GROUPS), v);
-        Blk const C = dry ? Dfar : (left ? col(x) : inv(x));
+        Blk const C = left ? col(x) : inv(x);
         if (left) blk_mm(C, stage, own, 1);
         else blk_mm(C, own, stage, c == q ? 1 : 3);
       }
@@ -1130,7 +1114,7 @@ PRAC_BOUNDS_READER(bounds_violations_cholqr)
 // ------------------------------------------------------------------ host side
 int atb_f64(const float* A, int64_t lda, const float* B, int64_t ldb, int64_t d, int64_t m, int64_t n,
             int symmetric, double alpha, void* out, int64_t ldo, int out_double, cudaStream_t stream, const int* run_if,
-            int run_if_mask, void* zero_words, int zero_bytes, bool next_early) {
+            int run_if_mask, void* zero_words, int zero_bytes) {
   if (m <= 0 || n <= 0) return PRAC_OK;
   if (d <= 0 || (symmetric && (A != B || m != n))) return PRAC_EINVAL;
   AtbArgs g{};
@@ -1141,7 +1125,6 @@ int atb_f64(const float* A, int64_t lda, const float* B, int64_t ldb, int64_t d,
   g.symmetric = symmetric;
   g.alpha = alpha;
   g.out = out; g.ldo = ldo; g.out_double = out_double;
-  g.next_early = next_early ? 1 : 0;
   g.run_if = run_if; g.run_if_mask = run_if_mask;
   g.zero_words = static_cast<int*>(zero_words); g.zero_count = zero_bytes / 4;
   const int tiles = symmetric ? g.tiles_n * (g.tiles_n + 1) / 2 : tiles_m * g.tiles_n;
@@ -1208,9 +1191,8 @@ int cholqr_pass(const float* Vin, int64_t ldin, float* Vout, int64_t ldout, int6
   if (ws == nullptr || ws_bytes < c.bytes) return PRAC_EWORKSPACE;
   const int* run_if = run_if_mask ? dev_status : nullptr;
   // (the product's kernel also zeroes the state of the factorisation that follows it)
-  const int64_t nb = (n + CB - 1) / CB;
   int st = atb_f64(Vin, ldin, Vin, ldin, d, n, n, 1, 1.0, c.G, n, 1, stream, run_if, run_if_mask,
-                   c.sync, static_cast<int>(sizeof(CholSync)), nb <= CC_MAX);
+                   c.sync, static_cast<int>(sizeof(CholSync)));
   if (st != PRAC_OK) return st;
   CholArgs a{};
   a.G = c.G; a.R = c.R; a.Dinv = c.Dinv; a.X = c.X; a.diag0 = c.diag0; a.Rinv = c.Rinv; a.ldr = n;

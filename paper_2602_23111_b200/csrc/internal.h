@@ -274,12 +274,10 @@ int launch_gaussian(uint64_t seed, uint64_t draw_counter, int64_t d, int64_t r, 
 // A (d x m, lda) and B (d x n, ldb), accumulated in double over row slices that are summed in a
 // fixed order.  symmetric != 0 (A == B, m == n) computes the upper tiles and mirrors them.
 // run_if != nullptr: the kernel returns at once unless *run_if & run_if_mask (a device word).
-// zero_words: up to 1 KB (a multiple of 4 bytes) that the kernel sets to zero.  next_early: the next kernel on the
-// stream, a small grid, may be set up from the start of this one.
+// zero_words: up to 1 KB (a multiple of 4 bytes) that the kernel sets to zero.
 int atb_f64(const float* A, int64_t lda, const float* B, int64_t ldb, int64_t d, int64_t m, int64_t n,
             int symmetric, double alpha, void* out, int64_t ldo, int out_double, cudaStream_t stream,
-            const int* run_if = nullptr, int run_if_mask = 0, void* zero_words = nullptr, int zero_bytes = 0,
-            bool next_early = false);
+            const int* run_if = nullptr, int run_if_mask = 0, void* zero_words = nullptr, int zero_bytes = 0);
 
 // One Cholesky-QR pass: Vout (d x n, ldout) = Vin (d x n, ldin) R^-1 with R^T R = Vin^T Vin, the
 // Gram matrix accumulated and factored in double.  R has a positive diagonal.  Vout != Vin.
