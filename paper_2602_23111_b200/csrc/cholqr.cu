@@ -219,7 +219,8 @@ struct CholArgs {
   long long ldr;
   int n, nb;
   int* dev_status;
-  int flag_bit;
+  int flag_bit;            // set for a bad pivot
+  int weak_bit;            // set for a weak column (0: not looked at)
   CholSync* sync;          // zeroed before the launch
   unsigned poll_limit;
   int run_if_mask;         // != 0: the kernel does nothing unless *dev_status has one of these bits
@@ -491,6 +492,14 @@ __device__ __forceinline__ void chol_emit(const CholArgs& a, const double (*S)[C
     }
   }
 }
+// A column is weak where the columns before it leave less than 1e-3 of its squared norm.  The fp32 product V R^-1 is then off
+// orthonormal by 2^-24 times a condition number of 30 and more, and what is left of that decides how well the panel spans what it should: a
+// few weak columns in the null space of a rank-deficient input (noise, as many vectors as it has dimensions) turned the dominant
+// space by 1e-3 in 6 % of such fits and left U off orthonormal by up to 0.7.  inv: the column's entry of R^-1 on the diagonal.
+__device__ __forceinline__ void chol_report_weak(const CholArgs& a, double inv, double diagonal_on_entry) {
+  if (a.weak_bit && inv * inv * diagonal_on_entry > 1e3) atomicOr(a.dev_status, a.weak_bit);
+}
+
 // What lies below the diagonal blocks of R^-1 (and the padding of the transposed pieces) is zero.
 __device__ __forceinline__ void chol_emit_zeros(const CholArgs& a, int worker, int workers) {
   for (int row = worker; row < a.n; row += workers) {
@@ -714,7 +723,11 @@ __global__ void __launch_bounds__(CHOL_MAIN + CHOL_HELP) chol_inv_kernel(const C
       __threadfence();
       atomicAdd(&sy->work, 1u);
     }
-    if (worker == static_cast<int>(workers) - 1) { chol_emit(a, S1, j, j); sync(); }
+    if (worker == static_cast<int>(workers) - 1) {
+      chol_emit(a, S1, j, j);
+      if (t < CB && j * CB + t < n) chol_report_weak(a, S1[t][t], __ldcg(&a.diag0[j * CB + t]));
+      sync();
+    }
   }
 }
 
@@ -962,7 +975,10 @@ __global__ void __launch_bounds__(256 * CC_GROUPS, 1) chol_cluster_kernel(const 
       // ---- the blocks it brings up to date, dealt to the groups: (p, q), c < p <= q, of G, (q, q) first, which needs nobody
       // else's block; or (q, x), x > c, of the inverse
       if (left && group == 0) blk_mm(col(q), own, own, 1);
-      if (!left && group == 1) chol_emit(a, own, q, c, c == q);
+      if (!left && group == 1) {
+        chol_emit(a, own, q, c, c == q);
+        if (c == q && gt < CB) chol_report_weak(a, own[gt][gt], 1e13 * guard[gt]);       // (a zero column is a bad pivot anyway)
+      }
       const int first = c + 1 + (left ? 1 - group : group), end = left ? q : nb;
       Blk const from = block(c);
       double2 v[2];
@@ -1198,6 +1214,7 @@ int cholqr_pass(const float* Vin, int64_t ldin, float* Vout, int64_t ldout, int6
   a.G = c.G; a.R = c.R; a.Dinv = c.Dinv; a.X = c.X; a.diag0 = c.diag0; a.Rinv = c.Rinv; a.ldr = n;
   a.n = static_cast<int>(n); a.nb = static_cast<int>((n + CB - 1) / CB);
   a.dev_status = dev_status; a.flag_bit = flag_bit;
+  a.weak_bit = dev_status && flag_bit == DEV_CHOL_RETRY ? flag_bit : 0;
   a.sync = c.sync; a.poll_limit = barrier_poll_limit(); a.run_if_mask = run_if_mask;
   // an optional pass (run_if_mask != 0) is rare and small: it takes the general product
   const bool tensor = run_if_mask == 0 && c.tensor && tc_init() == PRAC_OK && aligned16(Vout) && (ldout % 4) == 0;
@@ -1328,8 +1345,8 @@ int cholqr_final(const float* Vin, int64_t ldin, float* Vout, int64_t ldout, flo
   if (st != PRAC_OK) return st;
   // A bad pivot means the panel was (numerically) rank deficient: the guarded column of Vout is
   // amplified rounding noise, a direction of its own but neither normalised nor orthogonal to
-  // the rest.  One more pass orthonormalises it; only if that pass breaks down too is the
-  // failure reported.
+  // the rest.  A weak column (chol_report_weak) is not as orthogonal to the rest as fp32 allows.  One more pass
+  // orthonormalises them; only if that pass breaks down is the failure reported.
   st = cholqr_pass(Vout, ldout, tmp, n, d, n, ws, ws_bytes, dev_status, DEV_CHOL_PIVOT, stream, DEV_CHOL_RETRY);
   if (st != PRAC_OK) return st;
   return launch_copy2d_if(tmp, n, Vout, ldout, d, n, dev_status, DEV_CHOL_RETRY, DEV_CHOL_RETRY, stream);
