@@ -1084,12 +1084,15 @@ void atb_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2], int til
   cfg.numAttrs = 2;
 }
 
-// Slices of the rows = CTAs of a tile's cluster: what lets the busiest SM go through the fewest chunks of 16 rows, two
-// chunks' time for every doubling (the sum over the slices).  Clusters do not fill every SM before one of them takes a
-// second CTA: 15 clusters of 8 ran side by side (2048 x 320 symmetric, 17 us), 16 did not (2048 x 256 by 256, 26 us).  16 is
-// more than the portable cluster size.  Whether the cluster can be placed is asked for every launch (see chol_cluster_fits).
+// Slices of the rows = CTAs of a tile's cluster: what lets the busiest SM go through the fewest chunks of 16 rows.  A chunk takes
+// 0.7 us whether one or several CTAs share the SM (the fp64 rate), a launch 5 to 7 us beside that, at every number of
+// slices.  Clusters have to lie within a group of SMs: with a CTA per SM the device holds 74, 33, 15 and 7 clusters of 2, 4, 8 and 16, so on
+// 148, 132, 120 and 112 SMs.  Up to three CTAs per SM the SMs with one more set the time, above that it evens out.  Where the count is the
+// same 8 is taken, the fastest or within 5 % of it.  Symmetric, us with 4 / 8 / 16 slices: 2048 x 128 28.4 / 16.8 / 11.3, x 256
+// 29.0 / 17.1 / 16.9, x 320 29.0 / 17.3 / 21.7, x 384 29.3 / 27.3 / 22.3, x 512 48.4 / 37.4 / 33.2, x 640 49.4 / 47.7 / 48.9; 5461 x 512
+// 118 / 89.0 / 76.7, x 640 120 / 116 / 117.  Whether the cluster can be placed is asked for every launch (see chol_cluster_fits).
 int atb_slices(int tiles, int64_t d, cudaStream_t stream) {
-  static DeviceOnce wide;
+  static DeviceOnce wide;                      // (16 is more than the portable cluster size)
   int dev = -1;
   bool ok = cudaGetDevice(&dev) == cudaSuccess;
   if (ok && !wide.done(dev)) {
@@ -1099,13 +1102,13 @@ int atb_slices(int tiles, int64_t d, cudaStream_t stream) {
   if (!ok) (void)cudaGetLastError();           // (then 16 cannot be placed)
   tc_init();
   const int sms = tc_num_sms() > 0 ? tc_num_sms() : 148;
-  int best = 1;
-  long long least = -1;
-  for (int s = 1, doublings = 0; s <= 16; s *= 2, ++doublings) {
-    const int room = s <= 4 ? sms : (s == 8 ? sms * 13 / 16 : sms * 3 / 4);
-    const long long per_sm = (static_cast<long long>(tiles) * s + room - 1) / room;
-    const long long cost = per_sm * ((d + AT_K * s - 1) / (AT_K * s)) + 2 * doublings;
-    if (least < 0 || cost < least) { least = cost; best = s; }
+  int best = 0;
+  long long least = 0;
+  for (const int s : {8, 16, 4, 2, 1}) {
+    const int room = s <= 2 ? sms : sms * (s == 4 ? 132 : (s == 8 ? 120 : 112)) / 148;
+    const long long ctas = static_cast<long long>(tiles) * s, rows = (d + AT_K * s - 1) / (AT_K * s);
+    const long long chunks = ctas <= 3ll * room ? (ctas + room - 1) / room * rows : (ctas * rows + room - 1) / room;
+    if (best == 0 || chunks < least) { least = chunks; best = s; }
   }
   for (; best > 1; best /= 2) {
     cudaLaunchConfig_t cfg;
